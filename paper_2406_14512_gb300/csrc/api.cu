@@ -31,18 +31,20 @@ int fail(int code, const std::string &m) {
 
 // Particles per work item of the tiled push.  A grid whose tiles already
 // give the GPU enough items (tiles x species >= 4096) keeps 8192, so that
-// every item amortises the staging of its tile; a small instance takes the
-// largest power of two from 512 to 8192 at or below capacity / 4096, so that
-// it still offers a few thousand items (blocks) to the GPU.  Members of an
-// ensemble keep 8192 (the members fill the GPU together, and short items
-// only re-stage their tiles).  The work list is sized for the shortest.
-constexpr int kChunkMin = 512, kChunkMax = 8192;
+// every item amortises the staging of its tile (about 2,000 warp
+// instructions, those of 64 particles); a small instance takes the largest
+// power of two from 256 to 8192 at or below n_species x capacity / 4096, so
+// that it still offers a few thousand items to the GPU, and down to one
+// particle per thread.  Members of an ensemble keep 8192 (the members fill
+// the GPU together, and short items only re-stage their tiles).  The work
+// list is sized for the shortest.
+constexpr int kChunkMin = 256, kChunkMax = 8192;
 int chunk_of(const hff_config &c) {
   const int tr = c.tile_r > 0 ? c.tile_r : 16, tt = c.tile_t > 0 ? c.tile_t : 32;
   const int64_t tiles = (int64_t)((c.nr + tr - 1) / tr) * ((c.nt + tt - 1) / tt);
   if (tiles * c.n_species >= 4096) return kChunkMax;
   int k = kChunkMin;
-  while (k < kChunkMax && (int64_t)(2 * k) * 4096 <= c.capacity) k *= 2;
+  while (k < kChunkMax && (int64_t)(2 * k) * 4096 <= c.n_species * c.capacity) k *= 2;
   return k;
 }
 
@@ -191,6 +193,7 @@ struct Offsets {
   size_t sidx[kMaxSpecies];  // sorted order of the last sort, per species
   size_t items;
   size_t qnode, rows, psi64;
+  size_t jacc;           // flux accumulators of the push
   size_t fsnap;          // halo snapshot of the fused field update
   int seg_rows;          // rows per segment of the fused field update
   size_t ev[8];          // pair-creation events: key cell xo yo ur ut up w
@@ -214,7 +217,7 @@ struct Small {  // device counters, one 256-byte block
   unsigned long long clamps;
   unsigned status;
   int n_items;
-  int next;
+  int next, done;             // work queue of the tiled push (both 0 between pushes)
 };
 
 int tile_r_of(const hff_config &c) { return c.tile_r > 0 ? c.tile_r : 16; }
@@ -272,6 +275,7 @@ void layout(const hff_config &c, Offsets &o) {
   o.ev_cap = c.gamma_th > 0 ? cap / 4 + 1024 : 0;
   for (int k = 0; k < 8; ++k) o.ev[k] = o.ev_cap ? L.take((size_t)o.ev_cap * (k < 2 ? 4 : R)) : 0;
   o.spec = L.take(4096 * 8);
+  o.jacc = cap ? L.take(push_acc_bytes(c.nr, c.nt, R)) : 0;
   o.qnode = L.take(nn * 8);
   o.rows = L.take((nr + 1) * 8 * 8);
   o.psi64 = L.take(nn * 8);
@@ -443,6 +447,7 @@ void fill_params(hff_handle *h) {
     p.pushed = h->small->pushed;
     p.status = &h->small->status;
     p.clamps = &h->small->clamps;
+    p.jacc = reinterpret_cast<R *>(b + o.jacc);
     p.tile_r = tile_r_of(c); p.tile_t = tile_t_of(c); p.ntt = o.ntt;
     p.pairs = c.gamma_th > 0 ? 1 : 0;
     p.gamma_th2 = (R)(c.gamma_th * c.gamma_th);
@@ -648,29 +653,35 @@ int enqueue_step(hff_handle *h, int par, int stages, cudaStream_t s, int parts =
     if (fused) launch_ffcell<R>(p, s);
     else launch_node_a<R>(p, s);
   }
-  if ((parts & 1) && (stages & HFF_ST_PUSH) && h->c.sort_every > 0)
-    CK(cudaMemsetAsync(&h->small->next, 0, sizeof(int), s));
   if ((parts & 1) && (stages & HFF_ST_PUSH) && h->c.gamma_th > 0)  // events of this step only
     CK(cudaMemsetAsync(&h->small->pe_count, 0, sizeof(unsigned), s));
-  if ((parts & 2) && (stages & HFF_ST_PUSH) && h->c.sort_every > 0)
+  if ((parts & 2) && (stages & HFF_ST_PUSH) && h->c.sort_every > 0 && h->c.capacity > 0)
     launch_push_tiled<R>(p, h->wl, h->halo, s, h->push_grid, gather);
   if (!(parts & 4)) {
     CK(cudaGetLastError());
     return HFF_OK;
   }
-  if (stages & HFF_ST_PUSH) launch_push_tail<R>(p, s, h->tail_grid);
+  // the push's flux accumulators become J_PIC together with other grid work
+  // where the same call has some, else on their own
+  bool collect = (stages & HFF_ST_PUSH) && h->c.capacity > 0;
+  if (collect && h->c.sort_every == 0) launch_push_tail<R>(p, s, h->tail_grid);
+  const bool carried = fused || ((stages & HFF_ST_FARADAY1) && faraday_carries_collect<R>(p));
+  if (collect && !carried) {
+    launch_collect<R>(p, s);
+    collect = false;
+  }
   if (fused) {
     // the whole field update in one pass; J_PIC cleared for the next deposit
-    launch_field_fused<R>(p, h->seg_rows, h->base + h->o.fsnap, s);
+    launch_field_fused<R>(p, h->seg_rows, h->base + h->o.fsnap, collect, s);
     const int64_t nr = h->c.nr, nt = h->c.nt;
     CK(cudaMemsetAsync(p.f.jr, 0, (size_t)(nr * (nt + 1)) * sizeof(R), s));
     CK(cudaMemsetAsync(p.f.jt, 0, (size_t)((nr + 1) * nt) * sizeof(R), s));
     CK(cudaMemsetAsync(p.f.jp, 0, (size_t)((nr + 1) * (nt + 1)) * sizeof(R), s));
   } else {
-    if (stages & HFF_ST_FARADAY1) launch_faraday<R>(p, R(0.5), false, s);
+    if (stages & HFF_ST_FARADAY1) launch_faraday<R>(p, R(0.5), false, collect, s);
     if (stages & HFF_ST_AMPERE) launch_ampere<R>(p, s);
     if (stages & HFF_ST_CORRECT) launch_correct<R>(p, s);
-    if (stages & HFF_ST_FARADAY2) launch_faraday<R>(p, R(0.5), true, s);
+    if (stages & HFF_ST_FARADAY2) launch_faraday<R>(p, R(0.5), true, false, s);
   }
   if (stages & HFF_ST_INJECT) launch_inject<R>(p, s);
   else if (!(stages & HFF_ST_NOCOUNT)) launch_step_done<R>(p, s);
@@ -1126,6 +1137,7 @@ static int init_one(const hff_config *cfg, void *dev_mem, size_t bytes, void *st
   h->wl.items = reinterpret_cast<int4 *>(h->base + h->o.items);
   h->wl.n_items = &h->small->n_items;
   h->wl.next = &h->small->next;
+  h->wl.done = &h->small->done;
   h->wl.max_items = h->o.max_items;
   h->wl.chunk = chunk_of(*cfg);
   h->ss.keys_a = reinterpret_cast<uint32_t *>(h->base + h->o.keys_a);
@@ -1161,7 +1173,7 @@ static int init_one(const hff_config *cfg, void *dev_mem, size_t bytes, void *st
     rc = init_state<float>(h);
     if (rc == HFF_OK && cfg->sort_every > 0) {
       const size_t smem = push_tiled_smem<float>(h->pf[0], h->halo);
-      if (smem > 200 * 1024) return bail(fail(HFF_ERR_ARG, "tile + halo too large for shared memory"));
+      if (!push_tile_fits<float>(h->pf[0], h->halo)) return bail(fail(HFF_ERR_ARG, "tile + halo too large for shared memory"));
       if (set_push_smem<float>(smem) != cudaSuccess) return bail(fail(HFF_ERR_CUDA, "cannot set shared memory size"));
       h->push_grid = nsm * std::max(1, std::min(8, push_tiled_blocks_per_sm<float>(smem)));
     }
@@ -1170,7 +1182,7 @@ static int init_one(const hff_config *cfg, void *dev_mem, size_t bytes, void *st
     rc = init_state<double>(h);
     if (rc == HFF_OK && cfg->sort_every > 0) {
       const size_t smem = push_tiled_smem<double>(h->pd[0], h->halo);
-      if (smem > 200 * 1024) return bail(fail(HFF_ERR_ARG, "tile + halo too large for shared memory"));
+      if (!push_tile_fits<double>(h->pd[0], h->halo)) return bail(fail(HFF_ERR_ARG, "tile + halo too large for shared memory"));
       if (set_push_smem<double>(smem) != cudaSuccess) return bail(fail(HFF_ERR_CUDA, "cannot set shared memory size"));
       h->push_grid = nsm * std::max(1, std::min(8, push_tiled_blocks_per_sm<double>(smem)));
     }

@@ -16,6 +16,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "collect.cuh"
 #include "hff_common.cuh"
 
 namespace hff {
@@ -200,11 +201,17 @@ __global__ void __launch_bounds__(kRowThreads) k_node_a(Params<R> p) {
 
 // ---------------------------------------------------------------- Faraday
 // Eq. 18 over the exact primary faces, dB -= h dt curl E; optionally the
-// absorber B -= sigma (B - B_0), i.e. dB -= sigma dB, afterwards.
+// absorber B -= sigma (B - B_0), i.e. dB -= sigma dB, afterwards.  Blocks
+// past the rows collect the push's current, if the launch has any.
+static_assert(kRowThreads == kCollectThreads, "k_faraday's collecting blocks");
 template <typename R>
-__global__ void __launch_bounds__(kRowThreads) k_faraday(Params<R> p, R hdt, bool absorb) {
-  const int i = blockIdx.y, j = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(kRowThreads) k_faraday(const __grid_constant__ Params<R> p, R hdt, bool absorb) {
   const int nr = p.nr, nt = p.nt, n1 = nt + 1;
+  if (blockIdx.y > nr) {
+    collect_block(p, blockIdx.x, blockIdx.y - (nr + 1));
+    return;
+  }
+  const int i = blockIdx.y, j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j > nt) return;
   const Fields<R> &f = p.f;
   const Tables<R> &t = p.t;
@@ -445,7 +452,7 @@ __global__ void __launch_bounds__(kRowThreads) k_correct(Params<R> p) {
 // launch; so a block reads E^n and dB^n live only inside its own area (which
 // no other block writes, and which it overwrites only rows below the one it
 // is reading), and everywhere else from a snapshot of those regions taken
-// just before (k_fuse_snap_cols, k_fuse_snap_rows).  J_PIC is only read, and
+// just before (k_fuse_prepare).  J_PIC is only read, and
 // the caller clears it after the launch.
 constexpr int kFuseThreads = 128;     // columns of a strip, halo included
 constexpr int kFuseHalo = 4;          // columns recomputed on each side
@@ -506,29 +513,44 @@ __device__ __forceinline__ const R *fuse_array(const Params<R> &p, int a, int &l
   }
 }
 
-// the snapshot: halo columns (block 2 kFuseHalo x 32: column, row) ...
+// The snapshot in one launch: the first `nc` blocks copy halo columns (one
+// array of one boundary over kSnapThreads / (2 kFuseHalo) rows each), the next
+// `nw` blocks copy warm-up / trailing rows (kSnapThreads columns of one row of
+// one array of one boundary each), and the rest collect the push's current.
+constexpr int kSnapThreads = kCollectThreads;
+constexpr int kSnapRows = kSnapThreads / (2 * kFuseHalo);
 template <typename R>
-__global__ void k_fuse_snap_cols(Params<R> p, R *snap_c) {
-  const int cc = threadIdx.x, row = blockIdx.x * blockDim.y + threadIdx.y, ba = blockIdx.y;
-  if (row > p.nr) return;
-  const int a = ba % kFuseArrays, b = ba / kFuseArrays + 1;
-  const int col = b * kFuseOwn - kFuseHalo + cc;
+__global__ void __launch_bounds__(kSnapThreads) k_fuse_prepare(const __grid_constant__ Params<R> p, R *snap_c,
+                                                               R *snap_r, int seg_rows, int nc, int nw) {
+  int blk = blockIdx.x;
   int ld, rows, cols;
-  const R *src = fuse_array(p, a, ld, rows, cols);
-  const R v = (row < rows && col >= 0 && col < cols) ? src[(int64_t)row * ld + col] : R(0);
-  snap_c[((int64_t)ba * (p.nr + 1) + row) * (2 * kFuseHalo) + cc] = v;
-}
-// ... and warm-up / trailing rows (grid: columns, row of the window, boundary x array)
-template <typename R>
-__global__ void k_fuse_snap_rows(Params<R> p, R *snap_r, int seg_rows) {
-  const int col = blockIdx.x * blockDim.x + threadIdx.x, rr = blockIdx.y, ba = blockIdx.z;
-  if (col > p.nt) return;
-  const int a = ba % kFuseArrays, b = ba / kFuseArrays + 1;
-  const int row = b * seg_rows - kFuseWarm + rr;
-  int ld, rows, cols;
-  const R *src = fuse_array(p, a, ld, rows, cols);
-  const R v = (row >= 0 && row < rows && col < cols) ? src[(int64_t)row * ld + col] : R(0);
-  snap_r[((int64_t)ba * (kFuseWarm + kFuseTrail) + rr) * (p.nt + 1) + col] = v;
+  if (blk < nc) {
+    const int per = (p.nr + kSnapRows) / kSnapRows, ba = blk / per;
+    const int cc = threadIdx.x % (2 * kFuseHalo), row = (blk - ba * per) * kSnapRows + threadIdx.x / (2 * kFuseHalo);
+    if (row > p.nr) return;
+    const int a = ba % kFuseArrays, b = ba / kFuseArrays + 1;
+    const int col = b * kFuseOwn - kFuseHalo + cc;
+    const R *src = fuse_array(p, a, ld, rows, cols);
+    const R v = (row < rows && col >= 0 && col < cols) ? src[(int64_t)row * ld + col] : R(0);
+    snap_c[((int64_t)ba * (p.nr + 1) + row) * (2 * kFuseHalo) + cc] = v;
+    return;
+  }
+  blk -= nc;
+  if (blk < nw) {
+    const int per = p.nt / kSnapThreads + 1, w = blk / per;
+    const int col = (blk - w * per) * kSnapThreads + threadIdx.x;
+    if (col > p.nt) return;
+    const int rr = w % (kFuseWarm + kFuseTrail), ba = w / (kFuseWarm + kFuseTrail);
+    const int a = ba % kFuseArrays, b = ba / kFuseArrays + 1;
+    const int row = b * seg_rows - kFuseWarm + rr;
+    const R *src = fuse_array(p, a, ld, rows, cols);
+    const R v = (row >= 0 && row < rows && col < cols) ? src[(int64_t)row * ld + col] : R(0);
+    snap_r[(int64_t)w * (p.nt + 1) + col] = v;
+    return;
+  }
+  blk -= nw;
+  const int cx = collect_blocks_x(p);
+  collect_block(p, blk % cx, blk / cx);
 }
 
 // a ring of rows in shared memory, one element per column of the strip
@@ -620,7 +642,7 @@ __global__ void __launch_bounds__(kFuseThreads) k_field_fused(Params<R> p, R hdt
       x.bt = cbt ? f.bt[kn] : R(0);
       x.bp = cbp ? f.bp[kh] : R(0);
     } else {
-      // array a of the snapshot at s + a as (see k_fuse_snap_rows / _cols)
+      // array a of the snapshot at s + a as (see k_fuse_prepare)
       const R *s;
       int64_t as;
       if (own) {
@@ -967,16 +989,14 @@ size_t fuse_snap_bytes(int nr, int nt, int seg_rows, size_t real) {
   const FuseGeom fg = fuse_geom(nr, nt, seg_rows);
   return (size_t)(fuse_snap_cols(nr, fg.strips) + fuse_snap_rows(nt, fg.segs)) * real;
 }
-template <typename R> void launch_field_fused(const Params<R> &p, int seg_rows, void *snap, cudaStream_t s) {
+template <typename R> void launch_field_fused(const Params<R> &p, int seg_rows, void *snap, bool collect, cudaStream_t s) {
   const FuseGeom fg = fuse_geom(p.nr, p.nt, seg_rows);
   R *sc = reinterpret_cast<R *>(snap);
   R *sr = sc + fuse_snap_cols(p.nr, fg.strips);
-  if (fg.strips > 1)
-    k_fuse_snap_cols<R><<<dim3((p.nr + 1 + 31) / 32, (fg.strips - 1) * kFuseArrays), dim3(2 * kFuseHalo, 32), 0, s>>>(
-        p, sc);
-  if (fg.segs > 1)
-    k_fuse_snap_rows<R><<<dim3((p.nt + 1 + 255) / 256, kFuseWarm + kFuseTrail, (fg.segs - 1) * kFuseArrays), 256, 0,
-                          s>>>(p, sr, seg_rows);
+  const int nc = (fg.strips - 1) * kFuseArrays * ((p.nr + kSnapRows) / kSnapRows);
+  const int nw = (fg.segs - 1) * kFuseArrays * (kFuseWarm + kFuseTrail) * (p.nt / kSnapThreads + 1);
+  const int nj = collect ? collect_blocks_x(p) * collect_blocks_y(p) : 0;
+  if (nc + nw + nj > 0) k_fuse_prepare<R><<<nc + nw + nj, kSnapThreads, 0, s>>>(p, sc, sr, seg_rows, nc, nw);
   k_field_fused<R><<<dim3(fg.strips, fg.segs), kFuseThreads, fuse_smem_bytes<R>(), s>>>(p, R(0.5) * p.dt, fg, sc, sr);
 }
 
@@ -1031,8 +1051,16 @@ template <typename R> void launch_node_a(const Params<R> &p, cudaStream_t s) {
 template <typename R> void launch_ffcell(const Params<R> &p, cudaStream_t s) {
   k_ffcell<R><<<dim3((p.nt + kRowThreads - 1) / kRowThreads, (p.nr + kFfRows - 1) / kFfRows), kRowThreads, 0, s>>>(p);
 }
-template <typename R> void launch_faraday(const Params<R> &p, R half, bool absorb, cudaStream_t s) {
-  k_faraday<R><<<row_grid(p.nr + 1, p.nt), kRowThreads, 0, s>>>(p, half * p.dt, absorb);
+template <typename R> bool faraday_carries_collect(const Params<R> &p) {
+  return p.nr + 1 + collect_blocks_y(p) <= 65535;  // gridDim.y
+}
+template <typename R> void launch_faraday(const Params<R> &p, R half, bool absorb, bool collect, cudaStream_t s) {
+  dim3 g = row_grid(p.nr + 1, p.nt);
+  if (collect) {
+    g.x = std::max<unsigned>(g.x, collect_blocks_x(p));
+    g.y += collect_blocks_y(p);
+  }
+  k_faraday<R><<<g, kRowThreads, 0, s>>>(p, half * p.dt, absorb);
 }
 template <typename R> void launch_ampere(const Params<R> &p, cudaStream_t s) {
   k_ampere<R><<<row_grid(p.nr + 1, p.nt), kRowThreads, 0, s>>>(p);
@@ -1064,11 +1092,12 @@ template <typename R> void launch_combine(R *dst, const R *a, const R *b, int64_
   template size_t psi_smem<R>(int);                                            \
   template void launch_node_a<R>(const Params<R> &, cudaStream_t);             \
   template void launch_ffcell<R>(const Params<R> &, cudaStream_t);             \
-  template void launch_faraday<R>(const Params<R> &, R, bool, cudaStream_t);   \
+  template bool faraday_carries_collect<R>(const Params<R> &);                 \
+  template void launch_faraday<R>(const Params<R> &, R, bool, bool, cudaStream_t); \
   template void launch_ampere<R>(const Params<R> &, cudaStream_t);             \
   template void launch_correct<R>(const Params<R> &, cudaStream_t);            \
   template void launch_blend_out<R>(const Params<R> &, R *, R *, R *, uint8_t *, cudaStream_t); \
-  template void launch_field_fused<R>(const Params<R> &, int, void *, cudaStream_t);            \
+  template void launch_field_fused<R>(const Params<R> &, int, void *, bool, cudaStream_t);      \
   template size_t field_fused_smem<R>();                                                         \
   template cudaError_t set_field_fused_smem<R>(size_t);                                          \
   template int field_fused_blocks_per_sm<R>();

@@ -147,7 +147,7 @@ struct Fields {
   R *br, *bt, *bp;                  // B^n - B_0 (B^{n+1/2} - B_0 between the half steps)
   R *br0, *bt0, *bp0;               // initial field B_0 (also the absorber reference)
   R *sr, *st, *sp;                  // curl B_0 at the E locations (computed in FP64)
-  R *jr, *jt, *jp;                  // J_PIC accumulators (E locations)
+  R *jr, *jt, *jp;                  // J_PIC (E locations)
   typename PsiOf<R>::T *psi;        // Psi at nodes (FP64, or a float pair)
   R *jpr, *jpt, *jpp;               // J_perp at nodes
   R *der, *det, *dep;               // Delta E at nodes
@@ -201,6 +201,7 @@ struct Params {
   unsigned *status;
   unsigned long long *clamps;  // running count of E^2 > B^2 renormalisations (Eq. 26)
   int tile_r, tile_t, ntt;  // sort tiles
+  R *jacc;                  // the push's flux accumulators (zero between pushes; see deposit)
   // threshold pair creation (Sect. 5.1): events recorded by the push, the
   // pairs appended after the injection
   int pairs;
@@ -269,7 +270,9 @@ template <typename R> size_t psi_smem(int nt);  // dynamic shared memory of the 
 template <typename R> void launch_node_a(const Params<R> &p, cudaStream_t s);
 // the per-cell force-free flags alone (the fused field update computes J_perp)
 template <typename R> void launch_ffcell(const Params<R> &p, cudaStream_t s);
-template <typename R> void launch_faraday(const Params<R> &p, R half, bool absorb, cudaStream_t s);
+// collect: also turn the push's flux accumulators into J_PIC (collect.cuh)
+template <typename R> void launch_faraday(const Params<R> &p, R half, bool absorb, bool collect, cudaStream_t s);
+template <typename R> bool faraday_carries_collect(const Params<R> &p);  // its grid has room for that
 template <typename R> void launch_ampere(const Params<R> &p, cudaStream_t s);
 template <typename R> void launch_correct(const Params<R> &p, cudaStream_t s);
 // f at the E_r edges, E_th edges and nodes, and the force-free cell flags,
@@ -278,7 +281,7 @@ template <typename R> void launch_blend_out(const Params<R> &p, R *fr, R *ft, R 
 // the whole field update between the push and the injection (Faraday half,
 // Ampere, renormalisation, return, Faraday half with absorber) in one pass
 // over row segments of seg_rows rows
-template <typename R> void launch_field_fused(const Params<R> &p, int seg_rows, void *snap, cudaStream_t s);
+template <typename R> void launch_field_fused(const Params<R> &p, int seg_rows, void *snap, bool collect, cudaStream_t s);
 int fuse_own_cols(size_t real);                                     // theta columns a strip owns
 int fuse_seg_rows(int nr, int nt, int wave_blocks, size_t real);    // rows per segment of the launch
 template <typename R> int field_fused_blocks_per_sm();              // its occupancy (0 = unknown)
@@ -291,7 +294,8 @@ template <typename R> void launch_combine(R *dst, const R *a, const R *b, int64_
 struct WorkList {
   int4 *items;          // (species, tile, start, count)
   int *n_items;         // device count
-  int *next;            // dynamic scheduling counter
+  int *next;            // dynamic scheduling counter (0 between pushes)
+  int *done;            // blocks of the running push that have finished
   int max_items;
   int chunk;            // particles per item
 };
@@ -300,6 +304,10 @@ template <typename R> void launch_push_tail(const Params<R> &p, cudaStream_t s, 
 template <typename R> void launch_push_tiled(const Params<R> &p, const WorkList &wl, int halo,
                                              cudaStream_t s, int grid, bool gather);
 template <typename R> size_t push_tiled_smem(const Params<R> &p, int halo);
+template <typename R> bool push_tile_fits(const Params<R> &p, int halo);  // accepted by hff_init
+// the push's flux accumulators added to J_PIC and cleared
+template <typename R> void launch_collect(const Params<R> &p, cudaStream_t s);
+size_t push_acc_bytes(int nr, int nt, size_t real);  // their size
 template <typename R> void launch_inject(const Params<R> &p, cudaStream_t s);
 template <typename R> void launch_step_done(const Params<R> &p, cudaStream_t s);
 template <typename R> cudaError_t set_push_smem(size_t bytes);

@@ -8,14 +8,16 @@
 //  * k_push_tiled -- persistent blocks take (species, tile, chunk) work items
 //    from a list built by the sort.  The block stages E, B and the force-free
 //    flags of the tile plus a halo (the farthest a particle can drift between
-//    sorts) into shared memory, accumulates J in shared memory with shared
-//    atomics, and flushes the tile's J with one global atomic per nonzero
-//    entry.  Particles of a tile are contiguous, so the particle stream is
-//    read and written once, fully coalesced.
-//  * k_push_tail -- particles appended since the last sort (injection) and
-//    the no-sort configuration: gathers through L1/L2 and global atomics.
+//    sorts) into shared memory.  Particles of a tile are contiguous, so the
+//    particle stream is read and written once, fully coalesced.
+//    Particles appended since the last sort (injection, created pairs) follow
+//    in the same launch, gathering through L1/L2.
+//  * k_push_tail -- all particles of the no-sort configuration, the same way.
+// Both deposit into the flux accumulators in global memory (see deposit);
+// those become J_PIC at the end of the push stage (collect.cuh).
 #include <type_traits>
 
+#include "collect.cuh"
 #include "hff_common.cuh"
 
 namespace hff {
@@ -34,23 +36,6 @@ struct GlobalMesh {
   __device__ __forceinline__ R bt(int i, int j) const { const int64_t k = ix(i, j, p.nt + 1); return p.f.bt0[k] + p.f.bt[k]; }
   __device__ __forceinline__ R bp(int i, int j) const { const int64_t k = ix(i, j, p.nt); return p.f.bp0[k] + p.f.bp[k]; }
   __device__ __forceinline__ bool ff(int i, int j) const { return p.f.ffcell[ix(i, j, p.nt)] != 0; }
-  // raw charge flux through a dual face (J_r, J_th) or charge x velocity at
-  // a node (J_ph), converted to a current density with the face area or
-  // node volume and dt here
-  // (indices outside the arrays carry zero flux for every valid move; they
-  // are still checked here, on the global path)
-  __device__ __forceinline__ void add_jr(int i, int j, R v) const {
-    if (i >= 0 && i < p.nr && j >= 0 && j <= p.nt)
-      atomicAdd(&p.f.jr[ix(i, j, p.nt + 1)], v * p.t.dep_r[i] * p.t.inv_dch[j]);
-  }
-  __device__ __forceinline__ void add_jt(int i, int j, R v) const {
-    if (i >= 0 && i <= p.nr && j >= 0 && j < p.nt)
-      atomicAdd(&p.f.jt[ix(i, j, p.nt)], v * p.t.dep_t[i] * p.t.inv_sh[j]);
-  }
-  __device__ __forceinline__ void add_jp(int i, int j, R v) const {
-    if (i >= 0 && i <= p.nr && j >= 0 && j <= p.nt)
-      atomicAdd(&p.f.jp[ix(i, j, p.nt + 1)], v * p.t.dep_p[i] * p.t.inv_dch[j]);
-  }
   __device__ __forceinline__ R rn(int i) const { return p.t.rn[i]; }
   __device__ __forceinline__ R sn(int j) const { return p.t.sn[j]; }
   __device__ __forceinline__ R cn(int j) const { return p.t.cn[j]; }
@@ -60,7 +45,7 @@ struct GlobalMesh {
 // component (indices are global; the caller guarantees they fall inside).
 template <typename R>
 struct SharedMesh {
-  R *s_er, *s_et, *s_ep, *s_br, *s_bt, *s_bp, *s_jr, *s_jt, *s_jp;
+  R *s_er, *s_et, *s_ep, *s_br, *s_bt, *s_bp;
   R *s_rn, *s_sn, *s_cn;   // row / column tables of the region
   uint8_t *s_ff;
   int i0, j0, lt;
@@ -72,9 +57,6 @@ struct SharedMesh {
   __device__ __forceinline__ R bt(int i, int j) const { return s_bt[o(i, j)]; }
   __device__ __forceinline__ R bp(int i, int j) const { return s_bp[o(i, j)]; }
   __device__ __forceinline__ bool ff(int i, int j) const { return s_ff[o(i, j)] != 0; }
-  __device__ __forceinline__ void add_jr(int i, int j, R v) const { atomicAdd(&s_jr[o(i, j)], v); }
-  __device__ __forceinline__ void add_jt(int i, int j, R v) const { atomicAdd(&s_jt[o(i, j)], v); }
-  __device__ __forceinline__ void add_jp(int i, int j, R v) const { atomicAdd(&s_jp[o(i, j)], v); }
   __device__ __forceinline__ R rn(int i) const { return s_rn[i - i0]; }
   __device__ __forceinline__ R sn(int j) const { return s_sn[j - j0]; }
   __device__ __forceinline__ R cn(int j) const { return s_cn[j - j0]; }
@@ -305,11 +287,10 @@ __device__ __forceinline__ bool move_small(R r, R sn, R cs, R dt, const R u[3], 
 // a+1 in row b is -q (dS_x[0] + .. + dS_x[a]) (S0_y[b] + S1_y[b]) / 2, and
 // likewise in theta; J_ph uses the mid-point weights.  For linear weights the
 // nonzero radial fluxes always lie in a 2-face x 3-row window (and the polar
-// ones in a 3 x 2 window) placed by the direction of any cell crossing, so
-// every particle runs the same 16 predicated updates, with no data-dependent
-// loops.  The accessor receives raw charge fluxes (charge x velocity for
-// J_ph); the face areas, node volumes and dt are applied where the flux
-// reaches global memory.
+// ones in a 3 x 2 window) placed by the direction of any cell crossing; the
+// second face and the third node carry charge only if the particle crosses.
+// The accumulators hold raw charge fluxes (charge x velocity for J_ph);
+// the collection (collect.cuh) applies the face areas, node volumes and dt.
 template <typename R>
 struct Axis {  // weights along one direction
   R f0, f1;       // prefix-summed dS on the two faces of the window
@@ -342,152 +323,57 @@ __device__ __forceinline__ Axis<R> axis_weights(R x0, R X1) {
   return w;
 }
 
-// With `runs` (a work item whose particles sit cell by cell, decided once
-// per item), lanes of a warp that deposit into the same windows (equal J_r
-// / J_th window base and equal J_ph base) and sit next to each other form a
-// run; with at least kRunMin such neighbours in the warp, a segmented scan
-// sums each run's 16 site values and only the run's last lane issues the
-// shared atomics.  FP32 (and FP64) shared atomic adds are retry loops of
-// about six instructions on this GPU, which serialise on equal addresses: particles of one
-// cell next to each other in memory (co-located injected pairs, or any
-// cell-coherent order) otherwise cost one retry per lane and site (a
-// cell-ordered 4096^2 workload measured 2.7x the push time of a scattered
-// order).
-constexpr int kRunMin = 4;
-constexpr int kRunItemMin = 16;  // equal neighbour cells among 256 sampled pairs of a work item
-template <typename R>
-__device__ __forceinline__ void deposit_sh_runs(const SharedMesh<R> &m, R qw, int i0, int j0, R x0, R y0, R X1,
-                                                R Y1, R vphi) {
-  const Axis<R> ax = axis_weights(x0, X1), ay = axis_weights(y0, Y1);
-  const R nq = -qw;
-  const int lt = m.lt;
-  const int ob = m.o(i0 - 1 + ax.a0, j0 - 1 + ay.a0);
-  R v[16];
-  {
-    const R g0 = nq * ax.f0, g1 = nq * ax.f1;
-    v[0] = g0 * ay.m0; v[1] = g0 * ay.m1; v[2] = g0 * ay.m2;
-    v[3] = g1 * ay.m0; v[4] = g1 * ay.m1; v[5] = g1 * ay.m2;
-  }
-  {
-    const R g0 = nq * ay.f0, g1 = nq * ay.f1;
-    v[6] = g0 * ax.m0; v[7] = g0 * ax.m1; v[8] = g0 * ax.m2;
-    v[9] = g1 * ax.m0; v[10] = g1 * ax.m1; v[11] = g1 * ax.m2;
-  }
-  int op;
-  {
-    const R xm = R(0.5) * (x0 + X1), ym = R(0.5) * (y0 + Y1);
-    const int km = (xm < R(0)) ? -1 : (xm < R(1) ? 0 : 1);
-    const int lm = (ym < R(0)) ? -1 : (ym < R(1) ? 0 : 1);
-    const R wx = xm - R(km), wy = ym - R(lm);
-    const R qv = qw * vphi;
-    const R a0 = qv * (R(1) - wx), a1 = qv * wx;
-    v[12] = a0 * (R(1) - wy); v[13] = a0 * wy; v[14] = a1 * (R(1) - wy); v[15] = a1 * wy;
-    op = m.o(i0 + km, j0 + lm);
-  }
-  const unsigned act = __activemask();
-  const int lane = threadIdx.x & 31;
-  const int pob = __shfl_up_sync(act, ob, 1), pop = __shfl_up_sync(act, op, 1);
-  const bool cont = lane > 0 && ((act >> (lane - 1)) & 1u) && pob == ob && pop == op;
-  const unsigned conts = __ballot_sync(act, cont);
-  if (__popc(conts) >= kRunMin) {  // the same decision in every lane of act
-    // a run starts at every lane that does not continue its predecessor
-    // (inactive lanes included), so a run holds active lanes only
-    const unsigned upto = (lane == 31) ? 0xffffffffu : ((2u << lane) - 1u);
-    const int start = 31 - __clz(~conts & upto);
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-#pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        const R y = __shfl_up_sync(act, v[k], d);
-        if (lane - d >= start) v[k] += y;
-      }
-    }
-    if (lane < 31 && ((conts >> (lane + 1)) & 1u)) return;  // not the run's last lane
-  }
-#pragma unroll
-  for (int k = 0; k < 6; ++k)
-    if (v[k] != R(0)) atomicAdd(&m.s_jr[ob + (k / 3) * lt + k % 3], v[k]);
-#pragma unroll
-  for (int k = 0; k < 6; ++k)
-    if (v[6 + k] != R(0)) atomicAdd(&m.s_jt[ob + (k % 3) * lt + k / 3], v[6 + k]);
-#pragma unroll
-  for (int k = 0; k < 4; ++k)
-    if (v[12 + k] != R(0)) atomicAdd(&m.s_jp[op + (k / 2) * lt + k % 2], v[12 + k]);
+// FP32: one 32-byte record per cell,
+//   [J_r(i+1/2; j, j+1) | J_th(j+1/2; i, i+1) | J_ph(i,j; i,j+1; i+1,j; i+1,j+1)],
+// so that a particle that stays in its cell (most do: a step moves it by at
+// most half of the innermost cell) deposits with two 16-byte vector
+// reductions performed by the L2, and a crossing adds one more per cell
+// entered.  Nothing waits for them.  FP32 adds in shared memory are compiled
+// to retry loops (load, add, compare-and-swap, test) and cost a third of the
+// push's issue slots.  Measured alone, in ns per 1000 particles: two vector
+// reductions 10.7 (random cells of a tile) to 11.9 (consecutive particles in
+// one cell), eight shared adds 11.8 and 140; eight scalar reductions 51.
+__device__ __forceinline__ void red_add4(float *p, float a, float b, float c, float d) {
+  asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d)
+               : "memory");
 }
-
+// FP64: three arrays of (nr+2) x (nt+2) values (the window of a particle next
+// to the outer walls reaches one past the mesh), one scalar reduction each;
+// the L2 adds, not the SM, whose FP64 pipe bounds the FP64 push.
 template <typename R>
-__device__ __forceinline__ void deposit_sh(const SharedMesh<R> &m, R qw, int i0, int j0, R x0, R y0, R X1, R Y1,
-                                           R vphi, bool runs) {
-  if (runs) {
-    deposit_sh_runs<R>(m, qw, i0, j0, x0, y0, X1, Y1, vphi);
-    return;
-  }
-  const Axis<R> ax = axis_weights(x0, X1), ay = axis_weights(y0, Y1);
-  const R nq = -qw;
-  const int lt = m.lt;
-  const int ob = m.o(i0 - 1 + ax.a0, j0 - 1 + ay.a0);
-  {
-    const R g0 = nq * ax.f0, g1 = nq * ax.f1;
-    const R v[6] = {g0 * ay.m0, g0 * ay.m1, g0 * ay.m2, g1 * ay.m0, g1 * ay.m1, g1 * ay.m2};
-#pragma unroll
-    for (int k = 0; k < 6; ++k)
-      if (v[k] != R(0)) atomicAdd(&m.s_jr[ob + (k / 3) * lt + k % 3], v[k]);
-  }
-  {
-    const R g0 = nq * ay.f0, g1 = nq * ay.f1;
-    const R v[6] = {g0 * ax.m0, g0 * ax.m1, g0 * ax.m2, g1 * ax.m0, g1 * ax.m1, g1 * ax.m2};
-#pragma unroll
-    for (int k = 0; k < 6; ++k)
-      if (v[k] != R(0)) atomicAdd(&m.s_jt[ob + (k % 3) * lt + k / 3], v[k]);
-  }
-  {
-    const R xm = R(0.5) * (x0 + X1), ym = R(0.5) * (y0 + Y1);
-    const int km = (xm < R(0)) ? -1 : (xm < R(1) ? 0 : 1);
-    const int lm = (ym < R(0)) ? -1 : (ym < R(1) ? 0 : 1);
-    const R wx = xm - R(km), wy = ym - R(lm);
-    const R qv = qw * vphi;
-    const R a0 = qv * (R(1) - wx), a1 = qv * wx;
-    const R v[4] = {a0 * (R(1) - wy), a0 * wy, a1 * (R(1) - wy), a1 * wy};
-    const int op = m.o(i0 + km, j0 + lm);
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (v[k] != R(0)) atomicAdd(&m.s_jp[op + (k / 2) * lt + k % 2], v[k]);
-  }
-}
-
-template <typename R, typename M>
-__device__ __forceinline__ void deposit(const M &m, R qw, int i0, int j0, R x0, R y0, R X1, R Y1, R vphi) {
+__device__ __forceinline__ void deposit(const Params<R> &p, R qw, int i0, int j0, R x0, R y0, R X1, R Y1, R vphi) {
   const Axis<R> ax = axis_weights(x0, X1), ay = axis_weights(y0, Y1);
   const R nq = -qw;
   const int ib = i0 - 1 + ax.a0, jb = j0 - 1 + ay.a0;
-  // radial faces ib, ib+1 (E_r rows) x nodes jb .. jb+2
-  {
-    const R g0 = nq * ax.f0, g1 = nq * ax.f1;
-    const R v[6] = {g0 * ay.m0, g0 * ay.m1, g0 * ay.m2, g1 * ay.m0, g1 * ay.m1, g1 * ay.m2};
-#pragma unroll
-    for (int k = 0; k < 6; ++k)
-      if (v[k] != R(0)) m.add_jr(ib + k / 3, jb + k % 3, v[k]);
-  }
-  // polar faces jb, jb+1 (E_th columns) x nodes ib .. ib+2
-  {
-    const R g0 = nq * ay.f0, g1 = nq * ay.f1;
-    const R v[6] = {g0 * ax.m0, g0 * ax.m1, g0 * ax.m2, g1 * ax.m0, g1 * ax.m1, g1 * ax.m2};
-#pragma unroll
-    for (int k = 0; k < 6; ++k)
-      if (v[k] != R(0)) m.add_jt(ib + k % 3, jb + k / 3, v[k]);
-  }
+  const R gx0 = nq * ax.f0, gx1 = nq * ax.f1, gy0 = nq * ay.f0, gy1 = nq * ay.f1;
   // J_ph at the mid-point
-  {
-    const R xm = R(0.5) * (x0 + X1), ym = R(0.5) * (y0 + Y1);
-    const int km = (xm < R(0)) ? -1 : (xm < R(1) ? 0 : 1);
-    const int lm = (ym < R(0)) ? -1 : (ym < R(1) ? 0 : 1);
-    const R wx = xm - R(km), wy = ym - R(lm);
-    const R qv = qw * vphi;
-    const R a0 = qv * (R(1) - wx), a1 = qv * wx;
-    const R v[4] = {a0 * (R(1) - wy), a0 * wy, a1 * (R(1) - wy), a1 * wy};
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (v[k] != R(0)) m.add_jp(i0 + km + k / 2, j0 + lm + k % 2, v[k]);
+  const R xm = R(0.5) * (x0 + X1), ym = R(0.5) * (y0 + Y1);
+  const int km = (xm < R(0)) ? -1 : (xm < R(1) ? 0 : 1);
+  const int lm = (ym < R(0)) ? -1 : (ym < R(1) ? 0 : 1);
+  const R wx = xm - R(km), wy = ym - R(lm);
+  const R qv = qw * vphi;
+  const R a0 = qv * (R(1) - wx), a1 = qv * wx;
+  if constexpr (sizeof(R) == 4) {
+    const int n1 = p.nt + 1;
+    float *rec = p.jacc + 8 * ix(ib, jb, n1);
+    red_add4(rec, gx0 * ay.m0, gx0 * ay.m1, gy0 * ax.m0, gy0 * ax.m1);
+    red_add4(p.jacc + 8 * ix(i0 + km, j0 + lm, n1) + 4, a0 * (R(1) - wy), a0 * wy, a1 * (R(1) - wy), a1 * wy);
+    const bool cx = X1 < R(0) || X1 >= R(1), cy = Y1 < R(0) || Y1 >= R(1);
+    if (cx) red_add4(rec + 8 * n1, gx1 * ay.m0, gx1 * ay.m1, R(0), gy0 * ax.m2);
+    if (cy) red_add4(rec + 8, R(0), gx0 * ay.m2, gy1 * ax.m0, gy1 * ax.m1);
+    if (cx && cy) red_add4(rec + 8 * n1 + 8, R(0), gx1 * ay.m2, R(0), gy1 * ax.m2);
+  } else {
+    const int ld = p.nt + 2;
+    const int64_t nn = (int64_t)(p.nr + 2) * ld;
+    R *jr = p.jacc + ix(ib, jb, ld), *jt = jr + nn, *jp = p.jacc + 2 * nn + ix(i0 + km, j0 + lm, ld);
+    auto add = [](R *q, R v) {
+      if (v != R(0)) atomicAdd(q, v);
+    };
+    add(jr, gx0 * ay.m0); add(jr + 1, gx0 * ay.m1); add(jr + 2, gx0 * ay.m2);
+    add(jr + ld, gx1 * ay.m0); add(jr + ld + 1, gx1 * ay.m1); add(jr + ld + 2, gx1 * ay.m2);
+    add(jt, gy0 * ax.m0); add(jt + ld, gy0 * ax.m1); add(jt + 2 * ld, gy0 * ax.m2);
+    add(jt + 1, gy1 * ax.m0); add(jt + ld + 1, gy1 * ax.m1); add(jt + 2 * ld + 1, gy1 * ax.m2);
+    add(jp, a0 * (R(1) - wy)); add(jp + 1, a0 * wy); add(jp + ld, a1 * (R(1) - wy)); add(jp + ld + 1, a1 * wy);
   }
 }
 
@@ -544,7 +430,7 @@ __device__ __forceinline__ void record_pair(const Params<R> &p, const SpeciesCon
 // push also performs a sort's payload gather, kGather, which writes w too).
 template <typename R, bool kGather, typename M>
 __device__ __forceinline__ void push_one(const M &m, const Params<R> &p, const SpeciesConst<R> &K, int q,
-                                         int qi, int i, int j, Tally<R> &tl, bool runs = false) {
+                                         int qi, int i, int j, Tally<R> &tl) {
   constexpr bool kShared = std::is_same<M, SharedMesh<R>>::value;
   const Species<R> &S = K.S;
   const Species<R> &In = K.In;
@@ -601,9 +487,8 @@ __device__ __forceinline__ void push_one(const M &m, const Params<R> &p, const S
   const int i1 = i + di;
   int j1 = j + dj;
   if (j1 >= nt) { j1 = nt - 1; yn = one_minus_ulp<R>(); }
-  if (!dead && m.ff(i1, j1)) dead = true;
-  if constexpr (kShared) deposit_sh<R>(m, K.q * w, i, j, xo, yo, X1, Y1, un[2] * ginv, runs);
-  else deposit<R>(m, K.q * w, i, j, xo, yo, X1, Y1, un[2] * ginv);
+  if (!dead && (i1 >= nr || m.ff(i1, j1))) dead = true;  // off the mesh (no absorber), or force-free
+  deposit<R>(p, K.q * w, i, j, xo, yo, X1, Y1, un[2] * ginv);
   if (dead) {
     S.cell[q] = -1;
     tl.killed += w;
@@ -650,15 +535,18 @@ __device__ __forceinline__ void flush_tally(const Tally<R> &tl, double *acc, uns
 }
 
 // ----------------------------------------------------------- tail kernel
+// slots count_sorted .. count of every species, block-strided over the grid
+// from its last block (which the tiled kernel gives a work item last)
 template <typename R>
-__global__ void __launch_bounds__(256) k_push_tail(Params<R> p) {
+__device__ __forceinline__ Tally<R> push_tail(const Params<R> &p) {
   GlobalMesh<R> m(p);
   Tally<R> tl{R(0), R(0), 0u, 0u};
   for (int s = 0; s < p.n_species; ++s) {
-    const SpeciesConst<R> K(p, s);
     const int64_t n0 = p.count_sorted[s], n1 = p.count[s];
-    for (int64_t q = n0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n1;
-         q += (int64_t)gridDim.x * blockDim.x) {
+    int64_t q = n0 + (gridDim.x - 1 - blockIdx.x) * (int64_t)blockDim.x + threadIdx.x;
+    if (q >= n1) continue;
+    const SpeciesConst<R> K(p, s);
+    for (; q < n1; q += (int64_t)gridDim.x * blockDim.x) {
       const int c = p.sp[s].cell[q];
       if (c < 0) continue;
       int i, j;
@@ -666,12 +554,16 @@ __global__ void __launch_bounds__(256) k_push_tail(Params<R> p) {
       push_one<R, false>(m, p, K, (int)q, (int)q, i, j, tl);
     }
   }
-  flush_tally(tl, p.acc, p.status, &p.pushed[1]);
+  return tl;
+}
+template <typename R>
+__global__ void __launch_bounds__(256) k_push_tail(const __grid_constant__ Params<R> p) {
+  flush_tally(push_tail(p), p.acc, p.status, &p.pushed[1]);
 }
 
 // ---------------------------------------------------------- tiled kernel
 // Region of a tile: cells [ti*TR - H, (ti+1)*TR + H) (and likewise in theta)
-// widened by the stencil: one node below, two above.
+// widened by the gather's stencil: one node on either side.
 // Register budget: five blocks of 256 per SM in FP32 (48 registers, a few
 // spilled values in L1; the region of a 16 x 24 tile fits five times in
 // shared memory), three in FP64, whose doubled region leaves room for no more.
@@ -680,13 +572,12 @@ template <typename R, bool kGather>
 __global__ void __launch_bounds__(256, push_tiled_min_blocks<R>())
     k_push_tiled(const __grid_constant__ Params<R> p, WorkList wl, int halo) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int lr = p.tile_r + 2 * halo + 4, lt = p.tile_t + 2 * halo + 4, area = lr * lt;
+  const int lr = p.tile_r + 2 * halo + 2, lt = p.tile_t + 2 * halo + 2, area = lr * lt;
   R *base = reinterpret_cast<R *>(smem);
   SharedMesh<R> m;
   m.s_er = base; m.s_et = base + area; m.s_ep = base + 2 * area;
   m.s_br = base + 3 * area; m.s_bt = base + 4 * area; m.s_bp = base + 5 * area;
-  m.s_jr = base + 6 * area; m.s_jt = base + 7 * area; m.s_jp = base + 8 * area;
-  m.s_rn = base + 9 * area; m.s_sn = m.s_rn + lr; m.s_cn = m.s_sn + lt;
+  m.s_rn = base + 6 * area; m.s_sn = m.s_rn + lr; m.s_cn = m.s_sn + lt;
   m.s_ff = reinterpret_cast<uint8_t *>(m.s_cn + lt);
   m.lt = lt;
   __shared__ int s_item;
@@ -702,7 +593,7 @@ __global__ void __launch_bounds__(256, push_tiled_min_blocks<R>())
     const int ti = tile / p.ntt, tj = tile - ti * p.ntt;
     m.i0 = ti * p.tile_r - halo - 1;
     m.j0 = tj * p.tile_t - halo - 1;
-    // stage E, B, flags (edge values replicated outside each array); clear J
+    // stage E, B, flags (edge values replicated outside each array)
     for (int k = threadIdx.x; k < area; k += blockDim.x) {
       const int a = k / lt, c = k - a * lt;
       const int gi = m.i0 + a, gj = m.j0 + c;
@@ -716,7 +607,6 @@ __global__ void __launch_bounds__(256, push_tiled_min_blocks<R>())
       m.s_bt[k] = p.f.bt0[kt] + p.f.bt[kt];
       m.s_bp[k] = p.f.bp0[kp] + p.f.bp[kp];
       m.s_ff[k] = (gi >= 0 && gj >= 0 && gi < nr && gj < nt) ? p.f.ffcell[ix(gi, gj, nt)] : 1;
-      m.s_jr[k] = R(0); m.s_jt[k] = R(0); m.s_jp[k] = R(0);
     }
     for (int k = threadIdx.x; k < lr; k += blockDim.x) {
       const int gi = m.i0 + k;
@@ -729,36 +619,10 @@ __global__ void __launch_bounds__(256, push_tiled_min_blocks<R>())
     }
     const SpeciesConst<R> K(p, s, kGather);
     const int q0 = item.z, q1 = item.z + item.w;
-    // particles of one cell next to each other (co-located injected pairs
-    // keep their order through the stable sort)?  Decided once per item from
-    // blockDim.x neighbour pairs spread over it, so a scattered item pays
-    // nothing in the deposit.
-    int same = 0;
-    {
-      const int stride = max(1, (q1 - q0 - 1) / (int)blockDim.x);
-      const int qa = q0 + 1 + (int)threadIdx.x * stride;
-      if (qa < q1) {
-        const int ca = K.In.cell[kGather ? (int)K.sidx[qa] : qa];
-        const int cb = K.In.cell[kGather ? (int)K.sidx[qa - 1] : qa - 1];
-        same = (ca == cb && ca >= 0) ? 1 : 0;
-      }
-    }
-    const bool runs = __syncthreads_count(same) >= kRunItemMin;
-    // the particles this thread visits: block-strided in a scattered item;
-    // in a cell-coherent one every warp walks its own contiguous slice, so
-    // that its lanes stay consecutive (the runs) while the warps work on
-    // different cells (their atomics then rarely meet)
-    int qs = q0 + (int)threadIdx.x, qe = q1, qstep = (int)blockDim.x;
-    if (runs) {
-      const int nw = (int)blockDim.x >> 5, w = (int)threadIdx.x >> 5;
-      const int slice = ((q1 - q0 + nw - 1) / nw + 31) & ~31;
-      qs = q0 + w * slice + ((int)threadIdx.x & 31);
-      qe = min(q1, q0 + (w + 1) * slice);
-      qstep = 32;
-    }
-    // a particle is handled in shared memory when its whole stencil (start
-    // cell -1 .. +2 in both directions) lies inside the region
-    for (int q = qs; q < qe; q += qstep) {
+    __syncthreads();
+    // a particle is handled in shared memory when its gather stencil and the
+    // cells it can reach (start cell -1 .. +1) lie inside the region
+    for (int q = q0 + (int)threadIdx.x; q < q1; q += (int)blockDim.x) {
       const int qi = kGather ? (int)K.sidx[q] : q;
       const int c = K.In.cell[qi];
       if (c < 0) {
@@ -767,8 +631,8 @@ __global__ void __launch_bounds__(256, push_tiled_min_blocks<R>())
       }
       int i, j;
       decode_cell(p, c, i, j);
-      if (i - 1 >= m.i0 && i + 2 < m.i0 + lr && j - 1 >= m.j0 && j + 2 < m.j0 + lt)
-        push_one<R, kGather>(m, p, K, q, qi, i, j, tl, runs);
+      if (i - 1 >= m.i0 && i + 1 < m.i0 + lr && j - 1 >= m.j0 && j + 1 < m.j0 + lt)
+        push_one<R, kGather>(m, p, K, q, qi, i, j, tl);
       else {
         const Tally<R> t = push_one_global<R, kGather>(p, s, q, qi, i, j);
         tl.killed += t.killed; tl.radiated += t.radiated;
@@ -776,26 +640,39 @@ __global__ void __launch_bounds__(256, push_tiled_min_blocks<R>())
       }
     }
     __syncthreads();
-    for (int k = threadIdx.x; k < area; k += blockDim.x) {
-      const int a = k / lt, c = k - a * lt;
-      const int gi = m.i0 + a, gj = m.j0 + c;
-      if (gi < 0 || gj < 0) continue;
-      // raw fluxes -> current densities (face areas, node volumes, dt)
-      if (m.s_jr[k] != R(0) && gi < nr && gj <= nt)
-        atomicAdd(&p.f.jr[ix(gi, gj, n1)], m.s_jr[k] * p.t.dep_r[gi] * p.t.inv_dch[gj]);
-      if (m.s_jt[k] != R(0) && gi <= nr && gj < nt)
-        atomicAdd(&p.f.jt[ix(gi, gj, nt)], m.s_jt[k] * p.t.dep_t[gi] * p.t.inv_sh[gj]);
-      if (m.s_jp[k] != R(0) && gi <= nr && gj <= nt)
-        atomicAdd(&p.f.jp[ix(gi, gj, n1)], m.s_jp[k] * p.t.dep_p[gi] * p.t.inv_dch[gj]);
-    }
-    __syncthreads();
   }
   flush_tally(tl, p.acc, p.status, &p.pushed[0]);
+  flush_tally(push_tail(p), p.acc, p.status, &p.pushed[1]);
+  // the last block to finish rewinds the work queue for the next push
+  __syncthreads();
+  if (threadIdx.x == 0 && atomicAdd(wl.done, 1) == (int)gridDim.x - 1) {
+    *wl.next = 0;
+    *wl.done = 0;
+  }
 }
 
 template <typename R> size_t push_tiled_smem(const Params<R> &p, int halo) {
-  const size_t lr = p.tile_r + 2 * halo + 4, lt = p.tile_t + 2 * halo + 4, area = lr * lt;
-  return area * (9 * sizeof(R) + 1) + (lr + 2 * lt) * sizeof(R);
+  const size_t lr = p.tile_r + 2 * halo + 2, lt = p.tile_t + 2 * halo + 2, area = lr * lt;
+  return area * (6 * sizeof(R) + 1) + (lr + 2 * lt) * sizeof(R);
+}
+
+// The tiles and cadences that hff_init accepts: those whose region, two
+// cells wider than the gather needs and with nine values and a flag per
+// location, fits 200 KB.  The kernel's own need is always below that.
+template <typename R> bool push_tile_fits(const Params<R> &p, int halo) {
+  const size_t lr = p.tile_r + 2 * halo + 4, lt = p.tile_t + 2 * halo + 4;
+  return lr * lt * (9 * sizeof(R) + 1) + (lr + 2 * lt) * sizeof(R) <= 200 * 1024;
+}
+
+template <typename R>
+__global__ void __launch_bounds__(kCollectThreads) k_collect(const __grid_constant__ Params<R> p) {
+  collect_block(p, blockIdx.x, blockIdx.y);
+}
+template <typename R> void launch_collect(const Params<R> &p, cudaStream_t s) {
+  k_collect<R><<<dim3(collect_blocks_x(p), collect_blocks_y(p)), kCollectThreads, 0, s>>>(p);
+}
+size_t push_acc_bytes(int nr, int nt, size_t real) {
+  return real == 4 ? (size_t)(nr + 1) * (nt + 1) * 32 : (size_t)3 * (nr + 2) * (nt + 2) * 8;
 }
 
 template <typename R> void launch_push_tail(const Params<R> &p, cudaStream_t s, int grid) {
@@ -867,6 +744,7 @@ __global__ void __launch_bounds__(1024) k_inject_scan(Params<R> p) {
       p.count[s] = end;
     }
     atomicAdd(&p.acc[0], (double)total * (double)p.w_inj * p.n_inj);
+    *p.step += 1;  // the step is counted here (k_step_done does without injection)
   }
 }
 
@@ -876,7 +754,7 @@ __global__ void __launch_bounds__(128) k_inject_write(Params<R> p) {
   const int nt = p.nt;
   if (j < nt) {
     const int k0 = p.inj_prefix[j], n = p.inj_prefix[j + 1] - k0;
-    const long long step = *p.step;
+    const long long step = *p.step - 1;  // the scan has counted this step
     for (int k = 0; k < n; ++k) {
       uint32_t c[4] = {(uint32_t)step, (uint32_t)((unsigned long long)step >> 32), (uint32_t)j, (uint32_t)k};
       philox4x32_10(c, p.seed_lo, p.seed_hi);
@@ -963,7 +841,7 @@ template <typename R> void launch_inject(const Params<R> &p, cudaStream_t s) {
     k_inject_write<R><<<(p.nt + 127) / 128, 128, 0, s>>>(p);
   }
   if (p.pairs) k_pairs_append<R><<<1, 1024, 0, s>>>(p);
-  k_step_done<R><<<1, 32, 0, s>>>(p);
+  if (!p.inject) k_step_done<R><<<1, 32, 0, s>>>(p);
 }
 template <typename R> void launch_step_done(const Params<R> &p, cudaStream_t s) {
   k_step_done<R><<<1, 32, 0, s>>>(p);
@@ -985,6 +863,8 @@ template <typename R> int push_tiled_blocks_per_sm(size_t bytes) {
 
 #define HFF_INST(R)                                                                         \
   template size_t push_tiled_smem<R>(const Params<R> &, int);                               \
+  template bool push_tile_fits<R>(const Params<R> &, int);                                  \
+  template void launch_collect<R>(const Params<R> &, cudaStream_t);                         \
   template void launch_push_tail<R>(const Params<R> &, cudaStream_t, int);                  \
   template void launch_push_tiled<R>(const Params<R> &, const WorkList &, int, cudaStream_t, int, bool); \
   template void launch_inject<R>(const Params<R> &, cudaStream_t);                          \
