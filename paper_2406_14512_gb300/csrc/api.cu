@@ -38,7 +38,7 @@ int fail(int code, const std::string &m) {
 // particle per thread.  Members of an ensemble keep 8192 (the members fill
 // the GPU together, and short items only re-stage their tiles).  The work
 // list is sized for the shortest.
-constexpr int kChunkMin = 256, kChunkMax = 8192;
+constexpr int kChunkMin = kPushThreads, kChunkMax = kMaxItem;
 int chunk_of(const hff_config &c) {
   const int tr = c.tile_r > 0 ? c.tile_r : 16, tt = c.tile_t > 0 ? c.tile_t : 32;
   const int64_t tiles = (int64_t)((c.nr + tr - 1) / tr) * ((c.nt + tt - 1) / tt);
@@ -371,6 +371,7 @@ void fill_params(hff_handle *h) {
     p.nr = c.nr; p.nt = c.nt;
     p.dt = (R)h->dt; p.dlog = (R)h->g.dlog; p.dth = (R)h->g.dth; p.omega = (R)(1.0 / c.r_lc);
     p.r_min = (R)c.r_min; p.xi_abs = (R)h->xi_abs; p.shell_r2 = (R)(c.shell_r * c.shell_r);
+    p.i_abs = (int)std::fmin(std::floor(h->xi_abs), 2e9) - 3;  // a move ends below i + 2
     p.inv_dlog = (R)(1.0 / h->g.dlog); p.inv_dth = (R)(1.0 / h->g.dth);
     p.small_grid = (h->g.dlog < 0.03 && h->g.dth < 0.03) ? 1 : 0;
     p.div_nt = make_fastdiv((uint32_t)c.nt);  // cell index -> row
@@ -423,6 +424,8 @@ void fill_params(hff_handle *h) {
       p.sidx[s] = c.sort_every > 0 ? reinterpret_cast<const uint32_t *>(b + o.sidx[s]) : nullptr;
     }
     p.cap = c.capacity;
+    // the real arrays of a species follow each other (see layout)
+    p.pstride = (int64_t)(o.part[0][0][2] - o.part[0][0][1]) / (int64_t)sizeof(R);
     p.count = h->small->count;
     p.count_sorted = h->small->count_sorted;
     p.rr_scale = &h->small->rr;

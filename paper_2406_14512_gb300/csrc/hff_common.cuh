@@ -165,6 +165,7 @@ struct Params {
   int nr, nt;
   R dt, dlog, dth, omega, r_min, xi_abs, shell_r2;
   R inv_dlog, inv_dth;
+  int i_abs;                // rows below it end inside xi_abs for any move of a step
   int small_grid;           // dlog and dtheta both below the series threshold
   FastDiv div_nt;           // cell / nt by multiplication (see decode_cell)
   int n_breaks;
@@ -182,6 +183,7 @@ struct Params {
   Species<R> src[kMaxSpecies];
   const uint32_t *sidx[kMaxSpecies];
   int64_t cap;
+  int64_t pstride;          // elements from one real array of a species to the next (xo .. w)
   long long *count;         // [kMaxSpecies] slots in use (device)
   long long *count_sorted;  // [kMaxSpecies] length of the tile-sorted prefix
   const double *rr_scale;   // device scalar (ramp)
@@ -291,6 +293,10 @@ template <typename R> cudaError_t set_field_fused_smem(size_t bytes);
 // dst[k] = a[k] + sign * b[k], k < n (B <-> B - B_0 at the ABI)
 template <typename R> void launch_combine(R *dst, const R *a, const R *b, int64_t n, int sign, cudaStream_t s);
 
+// threads of a block of the tiled push, and the most particles of a work item
+constexpr int kPushThreads = 256;
+constexpr int kMaxItem = 8192;
+
 struct WorkList {
   int4 *items;          // (species, tile, start, count)
   int *n_items;         // device count
@@ -321,6 +327,7 @@ struct SortScratch {
   int *tile_start;             // [ntiles + 1] first sorted slot of each tile
   int *tile_end;               // [ntiles + 1] one past its last slot
   int64_t cap;
+  int64_t pstride;          // elements from one real array of a species to the next (xo .. w)
   int ntiles;
 };
 

@@ -43,25 +43,186 @@ struct GlobalMesh {
 
 // Shared-memory view of a tile region [i0, i0 + LR) x [j0, j0 + LT) of every
 // component (indices are global; the caller guarantees they fall inside).
+// FP64: one array per component.
 template <typename R>
 struct SharedMesh {
   R *s_er, *s_et, *s_ep, *s_br, *s_bt, *s_bp;
   R *s_rn, *s_sn, *s_cn;   // row / column tables of the region
   uint8_t *s_ff;
   int i0, j0, lt;
+  static size_t bytes_per_location() { return 6 * sizeof(R) + 1; }
+  __device__ __forceinline__ unsigned char *carve(unsigned char *base, int area) {
+    R *b = reinterpret_cast<R *>(base);
+    s_er = b; s_et = b + area; s_ep = b + 2 * area; s_br = b + 3 * area; s_bt = b + 4 * area; s_bp = b + 5 * area;
+    return reinterpret_cast<unsigned char *>(b + 6 * area);
+  }
+  __device__ __forceinline__ void put(int k, int, R er, R et, R ep, R br, R bt, R bp) const {
+    s_er[k] = er; s_et[k] = et; s_ep[k] = ep; s_br[k] = br; s_bt[k] = bt; s_bp[k] = bp;
+  }
   __device__ __forceinline__ int o(int i, int j) const { return (i - i0) * lt + (j - j0); }
-  __device__ __forceinline__ R er(int i, int j) const { return s_er[o(i, j)]; }
-  __device__ __forceinline__ R et(int i, int j) const { return s_et[o(i, j)]; }
-  __device__ __forceinline__ R ep(int i, int j) const { return s_ep[o(i, j)]; }
-  __device__ __forceinline__ R br(int i, int j) const { return s_br[o(i, j)]; }
-  __device__ __forceinline__ R bt(int i, int j) const { return s_bt[o(i, j)]; }
-  __device__ __forceinline__ R bp(int i, int j) const { return s_bp[o(i, j)]; }
   __device__ __forceinline__ bool ff(int i, int j) const { return s_ff[o(i, j)] != 0; }
   __device__ __forceinline__ R rn(int i) const { return s_rn[i - i0]; }
   __device__ __forceinline__ R sn(int j) const { return s_sn[j - j0]; }
   __device__ __forceinline__ R cn(int j) const { return s_cn[j - j0]; }
 };
+// FP32: the components that share their locations side by side, and E_ph and
+// B_ph with their right-hand neighbours, so that the gather's corners are
+// 8-byte loads: 12 a particle instead of 24.
+template <>
+struct SharedMesh<float> {
+  float2 *s_a, *s_b;       // (E_r, B_th) and (E_th, B_r)
+  float2 *s_p, *s_q;       // E_ph and B_ph at columns j, j + 1
+  float *s_rn, *s_sn, *s_cn;
+  uint8_t *s_ff;
+  int i0, j0, lt;
+  static size_t bytes_per_location() { return 4 * sizeof(float2) + 1; }
+  __device__ __forceinline__ unsigned char *carve(unsigned char *base, int area) {
+    s_a = reinterpret_cast<float2 *>(base); s_b = s_a + area;
+    s_p = s_b + area; s_q = s_p + area;
+    return reinterpret_cast<unsigned char *>(s_q + area);
+  }
+  // location k, column c of the region: its own slot and the left neighbour's
+  // second half (the last column's second half is never read)
+  __device__ __forceinline__ void put(int k, int c, float er, float et, float ep, float br, float bt, float bp) const {
+    s_a[k] = make_float2(er, bt);
+    s_b[k] = make_float2(et, br);
+    s_p[k].x = ep;
+    s_q[k].x = bp;
+    if (c > 0) {
+      s_p[k - 1].y = ep;
+      s_q[k - 1].y = bp;
+    }
+  }
+  __device__ __forceinline__ int o(int i, int j) const { return (i - i0) * lt + (j - j0); }
+  __device__ __forceinline__ bool ff(int i, int j) const { return s_ff[o(i, j)] != 0; }
+  __device__ __forceinline__ float rn(int i) const { return s_rn[i - i0]; }
+  __device__ __forceinline__ float sn(int j) const { return s_sn[j - j0]; }
+  __device__ __forceinline__ float cn(int j) const { return s_cn[j - j0]; }
+};
 
+// two FP32 values in the packed arithmetic (one issue slot for two additions,
+// multiplications or multiply-adds), used where pairs fall together anyway
+struct F2 {
+  float2 v;
+};
+__device__ __forceinline__ F2 operator-(F2 a, F2 b) { return {__ffma2_rn(b.v, make_float2(-1.f, -1.f), a.v)}; }
+// w a + b
+__device__ __forceinline__ F2 vfma(float w, F2 a, F2 b) { return {__ffma2_rn(make_float2(w, w), a.v, b.v)}; }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
+
+// FP32 reciprocal and reciprocal square root as the single approximate
+// hardware instructions (about 1-2 ulp, denormals flushed): their arguments
+// here are squared norms, radii and ratios of per-step increments, never
+// denormal, and the results enter quantities compared with the FP64 oracle at
+// 1e-5 relative.  FP64 ones from the hardware's approximations (better than
+// 2^-18) by one step of third order: with e = 1 - x y the reciprocal is
+// y / (1 - e) = y (1 + e + e^2 + O(e^3)); with e = 1 - x y^2 the reciprocal
+// square root is y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2 / 8 + O(e^3)); the
+// remainders are below 2^-54.  Three and five FP64 operations instead of the
+// eight to ten of the library's (correctly rounded or nearly so): the FP64
+// push is bound by the FP64 pipe, two operations per clock and SM.  Arguments
+// near the ends of the range go to the library.
+__device__ __forceinline__ float rsq(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rcp(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ unsigned exponent_field(double x) { return ((unsigned)__double2hiint(x) >> 20) & 0x7ffu; }
+__device__ __forceinline__ bool mid_range(double x) { return exponent_field(x) - 32u < 2047u - 64u; }
+__device__ __forceinline__ double rsq(double x) {
+  if (!mid_range(x)) return rsqrt(x);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+__device__ __forceinline__ double rcp(double x) {
+  if (!mid_range(x)) return 1.0 / x;
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+
+// Comparisons of doubles on the integer pipe (a comparison costs the FP64
+// pipe as much as an addition): x >= c for a positive constant c whose lower
+// word is zero, the sign, finiteness, and |a| well below b.
+__device__ __forceinline__ bool at_least(float x, float c) { return x >= c; }
+__device__ __forceinline__ bool at_least(double x, double c) { return __double2hiint(x) >= __double2hiint(c); }
+__device__ __forceinline__ bool below_zero(float x) { return x < 0.f; }
+__device__ __forceinline__ bool below_zero(double x) { return __double2hiint(x) < 0 && ((__double2hiint(x) << 1) | __double2loint(x)) != 0; }
+__device__ __forceinline__ bool finite(float x) { return fabsf(x) <= 3.402823466e38f; }
+__device__ __forceinline__ bool finite(double x) { return exponent_field(x) != 2047u; }
+// inside [0, 1) as an offset that needs no look at the cell: one comparison of
+// the bits (-0 and values outside go the long way)
+__device__ __forceinline__ bool stays(float x) { return (unsigned)__float_as_int(x) < 0x3f800000u; }
+__device__ __forceinline__ bool stays(double x) { return (unsigned)__double2hiint(x) < 0x3ff00000u; }
+__device__ __forceinline__ bool all_finite(float X, float Y, const float u[3]) {
+  return finite((X + Y) + ((u[0] + u[1]) + u[2]));   // a sum is finite unless a term is not (none is near the range's end)
+}
+__device__ __forceinline__ bool all_finite(double X, double Y, const double u[3]) {
+  return finite(X) && finite(Y) && finite(u[0]) && finite(u[1]) && finite(u[2]);
+}
+// |a| < 0.03 b (implies b > 0).  FP64: the high words, read as integers, are
+// piecewise linear in the logarithm (within 0.0861 octaves), so a difference
+// of 5.2 octaves means a ratio below 2^-5.11 = 0.029; ratios between 0.025 and
+// 0.03 may be refused, which only sends the move to its general form.
+constexpr double kSmall = 0.03;
+__device__ __forceinline__ bool well_below(float a, float b) { return fabsf(a) < float(kSmall) * b; }
+__device__ __forceinline__ bool well_below(double a, double b) {
+  const int hb = __double2hiint(b);   // negative for b < 0
+  return hb >= 0 && hb < 0x7ff00000 && hb - (__double2hiint(a) & 0x7fffffff) >= 0x00533333;
+}
+
+// Small-argument Taylor expansions about 0, for the per-step increments that
+// the Courant condition keeps small; callers switch to the library functions
+// outside |x| < kSmall, where every truncation error is below 1e-12 of the
+// value in FP64 and 5e-9 in FP32 (a twelfth of its rounding).
+// c[0] + c[1] x + .. by Horner's rule
+template <typename R, int N>
+__device__ __forceinline__ R poly(R x, const double (&c)[N]) {
+  R t = R(c[N - 1]);
+#pragma unroll
+  for (int k = N - 2; k >= 0; --k) t = vfma(t, x, R(c[k]));
+  return t;
+}
+// sin x / x, (cos x - 1) / x^2 and atan t / t as series in the square,
+// log1p(x) / x and (exp x - 1) / x in x, and for q = tan^2 of an angle
+// (1 - cos) / q = (1 - (1 + q)^(-1/2)) / q and ((1 + q)^(1/2) - 1) / q
+// (binomial series)
+template <typename R> struct Series {
+  static __device__ __forceinline__ R sinc(R x2) { const double c[] = {1.0, -1.0 / 6, 1.0 / 120, -1.0 / 5040}; return poly(x2, c); }
+  static __device__ __forceinline__ R cosm(R x2) { const double c[] = {-0.5, 1.0 / 24, -1.0 / 720}; return poly(x2, c); }
+  static __device__ __forceinline__ R atanc(R t2) { const double c[] = {1.0, -1.0 / 3, 0.2, -1.0 / 7, 1.0 / 9}; return poly(t2, c); }
+  static __device__ __forceinline__ R log1pc(R x) {
+    const double c[] = {1.0, -0.5, 1.0 / 3, -0.25, 0.2, -1.0 / 6, 1.0 / 7};
+    return poly(x, c);
+  }
+  static __device__ __forceinline__ R expm1c(R x) {
+    const double c[] = {1.0, 0.5, 1.0 / 6, 1.0 / 24, 1.0 / 120, 1.0 / 720, 1.0 / 5040};
+    return poly(x, c);
+  }
+  static __device__ __forceinline__ R omc(R q) { const double c[] = {0.5, -3.0 / 8, 5.0 / 16, -35.0 / 128, 63.0 / 256}; return poly(q, c); }
+  static __device__ __forceinline__ R sqm(R q) { const double c[] = {0.5, -1.0 / 8, 1.0 / 16, -5.0 / 128, 7.0 / 256}; return poly(q, c); }
+};
+template <> struct Series<float> {
+  using R = float;
+  static __device__ __forceinline__ R sinc(R x2) { const double c[] = {1.0, -1.0 / 6, 1.0 / 120}; return poly(x2, c); }
+  static __device__ __forceinline__ R cosm(R x2) { const double c[] = {-0.5, 1.0 / 24}; return poly(x2, c); }
+  static __device__ __forceinline__ R atanc(R t2) { const double c[] = {1.0, -1.0 / 3, 0.2}; return poly(t2, c); }
+  static __device__ __forceinline__ R log1pc(R x) { const double c[] = {1.0, -0.5, 1.0 / 3, -0.25, 0.2}; return poly(x, c); }
+  static __device__ __forceinline__ R expm1c(R x) { const double c[] = {1.0, 0.5, 1.0 / 6, 1.0 / 24, 1.0 / 120}; return poly(x, c); }
+  static __device__ __forceinline__ R omc(R q) { const double c[] = {0.5, -3.0 / 8, 5.0 / 16}; return poly(q, c); }
+  static __device__ __forceinline__ R sqm(R q) { const double c[] = {0.5, -1.0 / 8, 1.0 / 16}; return poly(q, c); }
+};
+
+// ------------------------------------------------------------------ gather
 // 1D linear weights for a component at positions k + a (a = 0 or 1/2),
 // k = 0 .. n-1, constant beyond the ends.
 template <typename R>
@@ -73,52 +234,6 @@ __device__ __forceinline__ void stag(int c, R o, bool half, int n, int &k0, R &w
   if (k0 > n - 2) { k0 = n - 2; w = R(1); }
 }
 
-// Small-argument Taylor expansions about 0, for the per-step increments that
-// the Courant condition keeps small; callers switch to the library functions
-// outside |x| < kSmall, where every truncation error is below 1e-12.
-constexpr double kSmall = 0.03;
-template <typename R> __device__ __forceinline__ R sin_small(R x) {
-  const R x2 = x * x;
-  return x * (R(1) - x2 * R(1.0 / 6.0) * (R(1) - x2 * R(1.0 / 20.0) * (R(1) - x2 * R(1.0 / 42.0))));
-}
-template <typename R> __device__ __forceinline__ R cos_small(R x) {
-  const R x2 = x * x;
-  return R(1) - R(0.5) * x2 * (R(1) - x2 * R(1.0 / 12.0) * (R(1) - x2 * R(1.0 / 30.0)));
-}
-template <typename R> __device__ __forceinline__ R atan_small(R t) {
-  const R t2 = t * t;
-  return t * (R(1) - t2 * (R(1.0 / 3.0) - t2 * (R(0.2) - t2 * (R(1.0 / 7.0) - t2 * R(1.0 / 9.0)))));
-}
-template <typename R> __device__ __forceinline__ R log1p_small(R x) {
-  return x * (R(1) - x * (R(0.5) - x * (R(1.0 / 3.0) - x * (R(0.25) - x * (R(0.2) - x * (R(1.0 / 6.0) - x * R(1.0 / 7.0)))))));
-}
-template <typename R> __device__ __forceinline__ R exp_small(R x) {
-  return R(1) + x * (R(1) + x * R(0.5) * (R(1) + x * R(1.0 / 3.0) * (R(1) + x * R(0.25) * (R(1) + x * R(0.2) * (R(1) + x * R(1.0 / 6.0))))));
-}
-// FP32 reciprocal, reciprocal square root and division as the single
-// approximate hardware instructions (about 1-2 ulp, denormals flushed): their
-// arguments here are squared norms, radii and ratios of per-step increments,
-// never denormal, and the results enter quantities compared with the FP64
-// oracle at 1e-5 relative
-__device__ __forceinline__ float rsq(float x) {
-  float y;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
-__device__ __forceinline__ float fdiv(float a, float b) {
-  float y;
-  asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
-  return y;
-}
-__device__ __forceinline__ float rcp(float x) {
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
-__device__ __forceinline__ double fdiv(double a, double b) { return a / b; }
-
 template <typename R, typename M, typename Get>
 __device__ __forceinline__ R interp(const M &m, Get g, int i, R wi, int j, R wj) {
   const R a0 = g(m, i, j), a1 = g(m, i, j + 1), b0 = g(m, i + 1, j), b1 = g(m, i + 1, j + 1);
@@ -126,8 +241,10 @@ __device__ __forceinline__ R interp(const M &m, Get g, int i, R wi, int j, R wj)
   return lo + wi * (hi - lo);
 }
 
-template <typename R, typename M>
-__device__ __forceinline__ void gather(const M &m, int nr, int nt, int i, int j, R xo, R yo, R e[3], R b[3]) {
+template <typename R>
+__device__ __forceinline__ void gather(const GlobalMesh<R> &m, int i, int j, R xo, R yo, R e[3], R b[3]) {
+  using M = GlobalMesh<R>;
+  const int nr = m.p.nr, nt = m.p.nt;
   // the four (node | half) x (node | half) weight sets, each shared by the
   // components that live there
   int kin, kih, kjn, kjh;
@@ -144,24 +261,22 @@ __device__ __forceinline__ void gather(const M &m, int nr, int nt, int i, int j,
   b[2] = interp(m, [](const M &q, int a, int c) { return q.bp(a, c); }, kih, wih, kjh, wjh);
 }
 
-// Shared-memory versions of the gather and the deposit: every access is a
-// constant offset from one base offset per weight set, and the staged
-// region replicates the edge values of each array, which reproduces the
-// constant extrapolation of stag() without clamping.
+// Shared-memory versions of the gather: every access is a constant offset
+// from one base offset per weight set, and the staged region replicates the
+// edge values of each array, which reproduces the constant extrapolation of
+// stag() without clamping.
 template <typename R>
 __device__ __forceinline__ R lerp4(const R *a, int o, int lt, R wi, R wj) {
   const R a0 = a[o], a1 = a[o + 1], b0 = a[o + lt], b1 = a[o + lt + 1];
   const R lo = a0 + wj * (a1 - a0), hi = b0 + wj * (b1 - b0);
   return lo + wi * (hi - lo);
 }
-
-template <typename R>
-__device__ __forceinline__ void gather_sh(const SharedMesh<R> &m, int i, int j, R xo, R yo, R e[3], R b[3]) {
-  const bool hx = xo >= R(0.5), hy = yo >= R(0.5);
-  const int oc = m.o(i, j);
-  const int onn = oc, onh = oc - (hy ? 0 : 1), ohn = oc - (hx ? 0 : m.lt), ohh = ohn - (hy ? 0 : 1);
-  const R win = xo, wjn = yo, wih = hx ? xo - R(0.5) : xo + R(0.5), wjh = hy ? yo - R(0.5) : yo + R(0.5);
-  const int lt = m.lt;
+__device__ __forceinline__ void gather(const SharedMesh<double> &m, int i, int j, double xo, double yo, double e[3],
+                                       double b[3]) {
+  const bool hx = at_least(xo, 0.5), hy = at_least(yo, 0.5);
+  const int oc = m.o(i, j), lt = m.lt;
+  const int onn = oc, onh = oc - (hy ? 0 : 1), ohn = oc - (hx ? 0 : lt), ohh = ohn - (hy ? 0 : 1);
+  const double win = xo, wjn = yo, wih = xo + (hx ? -0.5 : 0.5), wjh = yo + (hy ? -0.5 : 0.5);
   e[0] = lerp4(m.s_er, ohn, lt, wih, wjn);
   b[1] = lerp4(m.s_bt, ohn, lt, wih, wjn);
   e[1] = lerp4(m.s_et, onh, lt, win, wjh);
@@ -169,51 +284,91 @@ __device__ __forceinline__ void gather_sh(const SharedMesh<R> &m, int i, int j, 
   e[2] = lerp4(m.s_ep, onn, lt, win, wjn);
   b[2] = lerp4(m.s_bp, ohh, lt, wih, wjh);
 }
+// (u, v) pairs of two components at the four corners: packed over components
+__device__ __forceinline__ F2 lerp_pair(const float2 *a, int o, int lt, float wi, float wj) {
+  const F2 a0{a[o]}, a1{a[o + 1]}, b0{a[o + lt]}, b1{a[o + lt + 1]};
+  const F2 lo = vfma(wj, a1 - a0, a0), hi = vfma(wj, b1 - b0, b0);
+  return vfma(wi, hi - lo, lo);
+}
+// one component: packed over the columns first
+__device__ __forceinline__ float lerp_one(const float2 *a, int o, int lt, float wi, float wj) {
+  const F2 r0{a[o]}, r1{a[o + lt]}, t = vfma(wi, r1 - r0, r0);
+  return fmaf(wj, t.v.y - t.v.x, t.v.x);
+}
+__device__ __forceinline__ void gather(const SharedMesh<float> &m, int i, int j, float x, float y, float e[3],
+                                       float b[3]) {
+  const bool hx = x >= 0.5f, hy = y >= 0.5f;
+  const int oc = m.o(i, j), lt = m.lt;
+  const int onh = oc - (hy ? 0 : 1), ohn = oc - (hx ? 0 : lt), ohh = ohn - (hy ? 0 : 1);
+  const float wih = x + (hx ? -0.5f : 0.5f), wjh = y + (hy ? -0.5f : 0.5f);
+  const F2 a = lerp_pair(m.s_a, ohn, lt, wih, y), c = lerp_pair(m.s_b, onh, lt, x, wjh);
+  e[0] = a.v.x; b[1] = a.v.y;
+  e[1] = c.v.x; b[0] = c.v.y;
+  e[2] = lerp_one(m.s_p, oc, lt, x, y);
+  b[2] = lerp_one(m.s_q, ohh, lt, wih, wjh);
+}
+
+// ------------------------------------------------------------------- push
+template <typename R> __device__ __forceinline__ R dot3(const R a[3], const R b[3], R c) {
+  return vfma(a[2], b[2], vfma(a[1], b[1], vfma(a[0], b[0], c)));
+}
+template <typename R> __device__ __forceinline__ R dot3(const R a[3], const R b[3]) {
+  return vfma(a[2], b[2], vfma(a[1], b[1], a[0] * b[0]));
+}
+// component k of a x b, plus c
+template <int k, typename R> __device__ __forceinline__ R cross(const R a[3], const R b[3], R c) {
+  constexpr int i = (k + 1) % 3, j = (k + 2) % 3;
+  return vfma(a[i], b[j], vfma(-a[j], b[i], c));
+}
 
 // Modified Boris step (Eqs. 15-17, c = 1): Lorentz Boris gives u_L, the
 // radiation-reaction kick K F_RR is evaluated at the time-centred momentum
 // (u + u_L)/2 and limited to half of |u_L| per step.  Bperp^2 of Eq. 17 is
 // evaluated as |F x beta|^2 + |F|^2 / gamma^2 with F = E + beta x B, which
 // equals |F|^2 - (beta.F)^2 = |F|^2 - (beta.E)^2 without cancellation.
+// Returns 1/gamma of the new momentum; dgam is the energy radiated.
 template <typename R>
-__device__ __forceinline__ void boris_rr(R qm, R krr, R dt, const R u[3], const R e[3], const R b[3],
-                                         R out[3], R &dgam) {
-  const R a = R(0.5) * qm * dt;
-  const R um0 = u[0] + a * e[0], um1 = u[1] + a * e[1], um2 = u[2] + a * e[2];
-  const R ig = rsq(R(1) + um0 * um0 + um1 * um1 + um2 * um2);
-  const R t0 = a * b[0] * ig, t1 = a * b[1] * ig, t2 = a * b[2] * ig;
-  const R sc = R(2) * rcp(R(1) + t0 * t0 + t1 * t1 + t2 * t2);
-  const R s0 = sc * t0, s1 = sc * t1, s2 = sc * t2;
-  const R v0 = um0 + (um1 * t2 - um2 * t1), v1 = um1 + (um2 * t0 - um0 * t2), v2 = um2 + (um0 * t1 - um1 * t0);
-  const R ul0 = um0 + (v1 * s2 - v2 * s1) + a * e[0];
-  const R ul1 = um1 + (v2 * s0 - v0 * s2) + a * e[1];
-  const R ul2 = um2 + (v0 * s1 - v1 * s0) + a * e[2];
-  out[0] = ul0; out[1] = ul1; out[2] = ul2;
-  dgam = R(0);
-  if (krr != R(0)) {
-    const R ub0 = R(0.5) * (u[0] + ul0), ub1 = R(0.5) * (u[1] + ul1), ub2 = R(0.5) * (u[2] + ul2);
-    const R g2 = R(1) + ub0 * ub0 + ub1 * ub1 + ub2 * ub2;
-    const R ig2 = rsq(g2);
-    const R be0 = ub0 * ig2, be1 = ub1 * ig2, be2 = ub2 * ig2;
-    const R f0 = e[0] + (be1 * b[2] - be2 * b[1]);
-    const R f1 = e[1] + (be2 * b[0] - be0 * b[2]);
-    const R f2 = e[2] + (be0 * b[1] - be1 * b[0]);
-    const R c0 = f1 * be2 - f2 * be1, c1 = f2 * be0 - f0 * be2, c2 = f0 * be1 - f1 * be0;
-    const R ff = f0 * f0 + f1 * f1 + f2 * f2;
-    const R bp2 = c0 * c0 + c1 * c1 + c2 * c2 + ff * ig2 * ig2;
-    const R bdot = be0 * e[0] + be1 * e[1] + be2 * e[2];
-    const R k = dt * krr;
-    const R du0 = k * ((f1 * b[2] - f2 * b[1]) + bdot * e[0] - g2 * bp2 * be0);
-    const R du1 = k * ((f2 * b[0] - f0 * b[2]) + bdot * e[1] - g2 * bp2 * be1);
-    const R du2 = k * ((f0 * b[1] - f1 * b[0]) + bdot * e[2] - g2 * bp2 * be2);
-    const R dn2 = du0 * du0 + du1 * du1 + du2 * du2, ul2s = ul0 * ul0 + ul1 * ul1 + ul2 * ul2;
-    const R lim = (dn2 > R(0.25) * ul2s) ? R(0.5) * rsq(dn2 * rcp(ul2s)) : R(1);
-    out[0] = ul0 + lim * du0;
-    out[1] = ul1 + lim * du1;
-    out[2] = ul2 + lim * du2;
-    const R gl = R(1) + ul2s, go = R(1) + out[0] * out[0] + out[1] * out[1] + out[2] * out[2];
-    dgam = gl * rsq(gl) - go * rsq(go);
+__device__ __forceinline__ R boris_rr(R qm, R krr, R dt, const R u[3], const R e[3], const R b[3], R out[3], R &dgam) {
+  const R one = R(1), a = R(0.5) * qm * dt;
+  R um[3], t[3], v[3], w[3], ul[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) um[k] = vfma(a, e[k], u[k]);
+  const R at = a * rsq(dot3(um, um, one));
+#pragma unroll
+  for (int k = 0; k < 3; ++k) t[k] = at * b[k];
+  const R sc = R(2) * rcp(dot3(t, t, one));
+  // u+ = u- + sc (u- + u- x t) x t
+  v[0] = cross<0>(um, t, um[0]); v[1] = cross<1>(um, t, um[1]); v[2] = cross<2>(um, t, um[2]);
+  w[0] = cross<0>(v, t, R(0)); w[1] = cross<1>(v, t, R(0)); w[2] = cross<2>(v, t, R(0));
+#pragma unroll
+  for (int k = 0; k < 3; ++k) ul[k] = vfma(sc, w[k], vfma(a, e[k], um[k]));
+  if (krr == R(0)) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) out[k] = ul[k];
+    dgam = R(0);
+    return rsq(dot3(ul, ul, one));
   }
+  R us[3], be[3], f[3], c[3], du[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) us[k] = u[k] + ul[k];   // twice the centred momentum
+  const R g2 = vfma(R(0.25), dot3(us, us), one), ig = rsq(g2), hb = R(0.5) * ig;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) be[k] = hb * us[k];
+  f[0] = cross<0>(be, b, e[0]); f[1] = cross<1>(be, b, e[1]); f[2] = cross<2>(be, b, e[2]);
+  c[0] = cross<0>(f, be, R(0)); c[1] = cross<1>(f, be, R(0)); c[2] = cross<2>(f, be, R(0));
+  const R bp2 = dot3(c, c, dot3(f, f) * (ig * ig));
+  const R bdot = dot3(be, e), k = dt * krr, gb = -(g2 * bp2);
+  du[0] = k * cross<0>(f, b, vfma(bdot, e[0], gb * be[0]));
+  du[1] = k * cross<1>(f, b, vfma(bdot, e[1], gb * be[1]));
+  du[2] = k * cross<2>(f, b, vfma(bdot, e[2], gb * be[2]));
+  const R dn2 = dot3(du, du), ul2 = dot3(ul, ul);
+  R lim = one;
+  if (dn2 > R(0.25) * ul2) lim = R(0.5) * rsq(dn2 * rcp(ul2));
+#pragma unroll
+  for (int q = 0; q < 3; ++q) out[q] = vfma(lim, du[q], ul[q]);
+  const R gl = one + ul2, go = dot3(out, out, one), rgo = rsq(go);
+  dgam = vfma(gl, rsq(gl), -(go * rgo));
+  return rgo;
 }
 
 // Straight-line move x' = x + (u/gamma) c dt in the local Cartesian frame at
@@ -248,81 +403,54 @@ __device__ __forceinline__ void move_general(R r, R sn, R cs, R dt, const R u[3]
 
 // The same move for the usual case of a displacement much smaller than the
 // distance to the axis (|d_phi| < 0.03 X and |b| < 0.03 a), where both
-// rotation angles are small: with t = tan(angle), cos = 1/sqrt(1+t^2),
-// sin = t cos and 1 - cos = t^2 / (sqrt(1+t^2)(sqrt(1+t^2)+1)) exactly, and
-// the angle itself from the Taylor series of atan.  Returns false (nothing
-// written) when the displacement is not small.
+// rotation angles are small: with t = tan(angle) and q = t^2, 1 - cos and
+// sqrt(1 + q) - 1 are short series in q and sin = t cos.  xr = dr / r.
+// A displacement that is not small takes the general form; `small` says that
+// no particle of the tile can have one (see TileFacts).
 template <typename R>
-__device__ __forceinline__ bool move_small(R r, R sn, R cs, R dt, const R u[3], R &dr, R &dth, R uo[3]) {
-  const R ig = dt * rsq(R(1) + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+__device__ __forceinline__ void move(bool small, R r, R sn, R cs, R ginv, R dt, const R u[3], R &xr, R &dth, R uo[3]) {
+  using P = Series<R>;
+  const R one = R(1), ig = dt * ginv;
   const R d0 = u[0] * ig, d1 = u[1] * ig, d2 = u[2] * ig;
-  const R x = (r + d0) * sn + d1 * cs;
-  if (!(x > R(0)) || fabs(d2) >= R(kSmall) * x) return false;
-  const R tp = fdiv(d2, x), qp = tp * tp;
-  const R cp = rsq(R(1) + qp), sqp = (R(1) + qp) * cp;
-  const R sp = tp * cp, omc = fdiv(qp, sqp * (sqp + R(1)));  // 1 - cos(phi)
-  const R dR = x * omc * sqp;                                // sqrt(x^2+d2^2) - x
-  const R pa = d0 + dR * sn;
-  const R a = r + pa, bb = d1 + dR * cs;
-  if (fabs(bb) >= R(kSmall) * a) return false;
-  const R ta = fdiv(bb, a), qa = ta * ta;
-  const R ca = rsq(R(1) + qa), sqa = (R(1) + qa) * ca, sa = ta * ca;
-  const R rnew = a * sqa;
-  dr = fdiv(pa * (R(2) * r + pa) + bb * bb, rnew + r);
-  dth = atan_small(ta);
-  const R uR = u[0] * sn + u[1] * cs;
-  const R s1 = sn * ca + cs * sa, c1 = cs * ca - sn * sa;
-  const R duR = -uR * omc + u[2] * sp;
-  uo[0] = u[0] * ca + u[1] * sa + duR * s1;
-  uo[1] = -u[0] * sa + u[1] * ca + duR * c1;
-  uo[2] = -uR * sp + u[2] * cp;
-  return true;
+  const R x = vfma(r + d0, sn, d1 * cs);
+  const R tp = d2 * rcp(x), qp = tp * tp;
+  const R omc = qp * P::omc(qp), cp = one - omc, sp = tp * cp;   // 1 - cos, cos and sin of phi
+  const R dR = x * (qp * P::sqm(qp));                             // sqrt(x^2 + d2^2) - x
+  const R pa = vfma(dR, sn, d0), bb = vfma(dR, cs, d1), a = r + pa;
+  const R ta = bb * rcp(a), qa = ta * ta;
+  const R ca = vfma(-qa, P::omc(qa), one), sa = ta * ca;
+  // dr = (pa (2 r + pa) + b^2) / (r' + r) with r' = a sqrt(1 + q)
+  const R ar = a + r, den = r * vfma(a, qa * P::sqm(qa), ar);
+  xr = vfma(pa, ar, bb * bb) * rcp(den);
+  dth = ta * P::atanc(qa);
+  const R uR = vfma(u[0], sn, u[1] * cs);
+  const R s1 = vfma(sn, ca, cs * sa), c1 = vfma(cs, ca, -(sn * sa));
+  const R duR = vfma(u[2], sp, -(uR * omc));
+  uo[0] = vfma(duR, s1, vfma(u[0], ca, u[1] * sa));
+  uo[1] = vfma(duR, c1, vfma(-u[0], sa, u[1] * ca));
+  uo[2] = vfma(u[2], cp, -(uR * sp));
+  if (small || (well_below(d2, x) && well_below(bb, a))) return;
+  R dr;
+  move_general<R>(r, sn, cs, dt, u, dr, dth, uo);
+  xr = dr / r;
 }
 
+// ----------------------------------------------------------------- deposit
 // Charge-conserving deposit for linear shapes (Esirkepov decomposition) in
 // the logical (xi, eta) plane.  (x0, y0) in [0,1) is the start offset in cell
 // (i0, j0) and (X1, Y1) the end point relative to node (i0, j0), in (-1, 2).
-// With S0, S1 the start and end weights on the nodes i0-1 .. i0+2 and
-// dS = S1 - S0, the charge through the radial dual face between nodes a and
-// a+1 in row b is -q (dS_x[0] + .. + dS_x[a]) (S0_y[b] + S1_y[b]) / 2, and
-// likewise in theta; J_ph uses the mid-point weights.  For linear weights the
-// nonzero radial fluxes always lie in a 2-face x 3-row window (and the polar
-// ones in a 3 x 2 window) placed by the direction of any cell crossing; the
-// second face and the third node carry charge only if the particle crosses.
-// The accumulators hold raw charge fluxes (charge x velocity for J_ph);
-// the collection (collect.cuh) applies the face areas, node volumes and dt.
-template <typename R>
-struct Axis {  // weights along one direction
-  R f0, f1;       // prefix-summed dS on the two faces of the window
-  R m0, m1, m2;   // (S0 + S1) / 2 on the three nodes of the window
-  int a0;         // window start relative to node i0 - 1 (0 or 1)
-};
-
-template <typename R>
-__device__ __forceinline__ Axis<R> axis_weights(R x0, R X1) {
-  Axis<R> w;
-  const bool lo = X1 < R(0), hi = X1 >= R(1);
-  // end weights on the nodes -1, 0, 1, 2 (relative to the start node)
-  const R e0 = lo ? -X1 : R(0);
-  const R e1 = lo ? R(1) + X1 : (hi ? R(0) : R(1) - X1);
-  const R e2 = lo ? R(0) : (hi ? R(2) - X1 : X1);
-  const R e3 = hi ? X1 - R(1) : R(0);
-  // prefix sums of dS = e - (0, 1 - x0, x0, 0) on the faces -1/2, 1/2, 3/2;
-  // inside one cell the middle one is -(X1 - x0) exactly
-  const R p0 = e0;
-  const R p1 = (lo || hi) ? e0 + e1 - (R(1) - x0) : x0 - X1;
-  const R p2 = hi ? p1 + e2 - x0 : R(0);  // zero without a crossing (exactly)
-  // weights (S0 + S1)/2 on the nodes -1 .. 2
-  const R n0 = R(0.5) * e0, n1 = R(0.5) * (e1 + R(1) - x0), n2 = R(0.5) * (e2 + x0), n3 = R(0.5) * e3;
-  w.a0 = lo ? 0 : 1;
-  w.f0 = lo ? p0 : p1;
-  w.f1 = lo ? p1 : p2;
-  w.m0 = lo ? n0 : n1;
-  w.m1 = lo ? n1 : n2;
-  w.m2 = lo ? n2 : n3;
-  return w;
-}
-
+// With S0, S1 the start and end weights on the nodes and dS = S1 - S0, the
+// charge through the radial dual face between nodes a and a+1 in row b is
+// -q (dS_x[0] + .. + dS_x[a]) (S0_y[b] + S1_y[b]) / 2, and likewise in theta;
+// J_ph uses the mid-point weights.  For linear weights and a move of less
+// than a cell this has a closed form.  With Xc = X1 clamped to [0, 1], the
+// flux is x0 - Xc through the face of the start cell and Xc - X1 through the
+// face of the cell entered (if any); the mean weights are 1 - m - max(h, 0) and
+// m + min(h, 0) on the start cell's nodes, with m = (x0 + Xc) / 2 and
+// h = (Xc - X1) / 2, and |h| on the far node of the cell entered.
+// The accumulators hold raw charge fluxes (charge x velocity for J_ph); the
+// collection (collect.cuh) applies the face areas, node volumes and dt.
+//
 // FP32: one 32-byte record per cell,
 //   [J_r(i+1/2; j, j+1) | J_th(j+1/2; i, i+1) | J_ph(i,j; i,j+1; i+1,j; i+1,j+1)],
 // so that a particle that stays in its cell (most do: a step moves it by at
@@ -340,41 +468,120 @@ __device__ __forceinline__ void red_add4(float *p, float a, float b, float c, fl
 // FP64: three arrays of (nr+2) x (nt+2) values (the window of a particle next
 // to the outer walls reaches one past the mesh), one scalar reduction each;
 // the L2 adds, not the SM, whose FP64 pipe bounds the FP64 push.
-template <typename R>
-__device__ __forceinline__ void deposit(const Params<R> &p, R qw, int i0, int j0, R x0, R y0, R X1, R Y1, R vphi) {
-  const Axis<R> ax = axis_weights(x0, X1), ay = axis_weights(y0, Y1);
-  const R nq = -qw;
-  const int ib = i0 - 1 + ax.a0, jb = j0 - 1 + ay.a0;
-  const R gx0 = nq * ax.f0, gx1 = nq * ax.f1, gy0 = nq * ay.f0, gy1 = nq * ay.f1;
-  // J_ph at the mid-point
-  const R xm = R(0.5) * (x0 + X1), ym = R(0.5) * (y0 + Y1);
-  const int km = (xm < R(0)) ? -1 : (xm < R(1) ? 0 : 1);
-  const int lm = (ym < R(0)) ? -1 : (ym < R(1) ? 0 : 1);
-  const R wx = xm - R(km), wy = ym - R(lm);
-  const R qv = qw * vphi;
-  const R a0 = qv * (R(1) - wx), a1 = qv * wx;
-  if constexpr (sizeof(R) == 4) {
-    const int n1 = p.nt + 1;
-    float *rec = p.jacc + 8 * ix(ib, jb, n1);
-    red_add4(rec, gx0 * ay.m0, gx0 * ay.m1, gy0 * ax.m0, gy0 * ax.m1);
-    red_add4(p.jacc + 8 * ix(i0 + km, j0 + lm, n1) + 4, a0 * (R(1) - wy), a0 * wy, a1 * (R(1) - wy), a1 * wy);
-    const bool cx = X1 < R(0) || X1 >= R(1), cy = Y1 < R(0) || Y1 >= R(1);
-    if (cx) red_add4(rec + 8 * n1, gx1 * ay.m0, gx1 * ay.m1, R(0), gy0 * ax.m2);
-    if (cy) red_add4(rec + 8, R(0), gx0 * ay.m2, gy1 * ax.m0, gy1 * ax.m1);
-    if (cx && cy) red_add4(rec + 8 * n1 + 8, R(0), gx1 * ay.m2, R(0), gy1 * ax.m2);
-  } else {
-    const int ld = p.nt + 2;
-    const int64_t nn = (int64_t)(p.nr + 2) * ld;
-    R *jr = p.jacc + ix(ib, jb, ld), *jt = jr + nn, *jp = p.jacc + 2 * nn + ix(i0 + km, j0 + lm, ld);
-    auto add = [](R *q, R v) {
-      if (v != R(0)) atomicAdd(q, v);
-    };
-    add(jr, gx0 * ay.m0); add(jr + 1, gx0 * ay.m1); add(jr + 2, gx0 * ay.m2);
-    add(jr + ld, gx1 * ay.m0); add(jr + ld + 1, gx1 * ay.m1); add(jr + ld + 2, gx1 * ay.m2);
-    add(jt, gy0 * ax.m0); add(jt + ld, gy0 * ax.m1); add(jt + 2 * ld, gy0 * ax.m2);
-    add(jt + 1, gy1 * ax.m0); add(jt + ld + 1, gy1 * ax.m1); add(jt + 2 * ld + 1, gy1 * ax.m2);
-    add(jp, a0 * (R(1) - wy)); add(jp + 1, a0 * wy); add(jp + ld, a1 * (R(1) - wy)); add(jp + ld + 1, a1 * wy);
+__device__ __forceinline__ int64_t acc_index(const Params<float> &p, int i, int j) { return 8 * ix(i, j, p.nt + 1); }
+__device__ __forceinline__ int64_t acc_index(const Params<double> &p, int i, int j) { return ix(i, j, p.nt + 2); }
+// fluxes of one cell: J_r through its radial face at its two nodes, J_th
+// through its polar face at its two nodes
+__device__ __forceinline__ void add_faces(const Params<float> &p, int i, int j, float r0, float r1, float t0, float t1) {
+  red_add4(p.jacc + acc_index(p, i, j), r0, r1, t0, t1);
+}
+__device__ __forceinline__ void add_faces(const Params<double> &p, int i, int j, double r0, double r1, double t0,
+                                          double t1) {
+  const int ld = p.nt + 2;
+  double *q = p.jacc + acc_index(p, i, j), *t = q + (int64_t)(p.nr + 2) * ld;
+  atomicAdd(q, r0); atomicAdd(q + 1, r1);
+  atomicAdd(t, t0); atomicAdd(t + ld, t1);
+}
+__device__ __forceinline__ void add_corners(const Params<float> &p, int i, int j, float a, float b, float c, float d) {
+  red_add4(p.jacc + acc_index(p, i, j) + 4, a, b, c, d);
+}
+__device__ __forceinline__ void add_corners(const Params<double> &p, int i, int j, double a, double b, double c, double d) {
+  const int ld = p.nt + 2;
+  double *q = p.jacc + 2 * (int64_t)(p.nr + 2) * ld + acc_index(p, i, j);
+  atomicAdd(q, a); atomicAdd(q + 1, b); atomicAdd(q + ld, c); atomicAdd(q + ld + 1, d);
+}
+
+// Items whose particles fill few cells: lanes of a warp that deposit into the
+// same cell are summed first, wherever they sit in the warp, and one of them
+// issues the reduction.  The record of a full cell then sees a tenth of the
+// additions: fewer in the L2's queue, and a shorter chain of FP32 roundings
+// (3,300 equal contributions added one by one lose 3e-5 of their sum, in the
+// L2 as in any FP32 accumulator).  The sums are the tree reduction by key of
+// E. Westphal ("Voting and Shuffling to Optimize Atomic Operations", NVIDIA
+// developer blog, 2015).  Decided once per work item, from sampled pairs of
+// particles kShareDist apart: equal cells there mean more particles in a cell
+// than an accumulator should take singly; elsewhere the reductions are cheaper
+// alone (2e7 particles in cell order, ten to a cell, on 2048^2: push 0.53 ms
+// alone, 0.60 summed), and left out where fewer than kShareMin lanes of the
+// warp share.
+constexpr int kShareMin = 4;
+constexpr int kShareDist = 64;
+constexpr int kShareItemMin = 16;  // equal cells among 256 sampled pairs of a work item
+// returns whether this lane issues the (summed) values
+template <int N>
+__device__ __forceinline__ bool sum_by_cell(int key, float (&v)[N]) {
+  const unsigned act = __activemask(), peers = __match_any_sync(act, key);
+  const unsigned sharing = __ballot_sync(act, (peers & (peers - 1)) != 0);
+  if (__popc(sharing) < kShareMin) return true;  // the same decision in every lane of act
+  const int lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
+  unsigned rest = peers & ~below & ~(1u << lane);   // members after this lane still holding a partial sum
+  int rank = __popc(peers & below);
+  const bool first = rank == 0;
+  while (__any_sync(act, rest != 0)) {
+    const int next = __ffs(rest);
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      const float y = __shfl_sync(act, v[k], next ? next - 1 : lane);
+      if (next) v[k] += y;
+    }
+    // members of odd rank have been taken; the others meet the next of theirs
+    rest &= __ballot_sync(act, (rank & 1) == 0);
+    rank >>= 1;
   }
+  return first;
+}
+__device__ __forceinline__ void add_faces_shared(const Params<float> &p, int i, int j, float r0, float r1, float t0,
+                                                 float t1) {
+  float v[4] = {r0, r1, t0, t1};
+  if (sum_by_cell((int)ix(i, j, p.nt + 1), v)) add_faces(p, i, j, v[0], v[1], v[2], v[3]);
+}
+
+// sx, sy: the cell entered in either direction (-1, 0, 1)
+template <bool kShare, typename R>
+__device__ __forceinline__ void deposit(const Params<R> &p, R qw, int i, int j, int sx, int sy, R x0, R y0, R X1,
+                                        R Y1, R vphi) {
+  const R nq = -qw;
+  R gx = nq * (x0 - X1), gy = nq * (y0 - Y1);
+  R mx1 = R(0.5) * (x0 + X1), my1 = R(0.5) * (y0 + Y1), mx0 = R(1) - mx1, my0 = R(1) - my1;
+  R wx = mx1, wy = my1;          // J_ph: mid-point weights in the cell (ic, jc)
+  int ic = i, jc = j;
+  if ((sx | sy) != 0) {
+    const R Xc = sx == 0 ? X1 : (sx < 0 ? R(0) : R(1)), Yc = sy == 0 ? Y1 : (sy < 0 ? R(0) : R(1));
+    const R hx = R(0.5) * (Xc - X1), hy = R(0.5) * (Yc - Y1);
+    const R ax0 = sx < 0 ? hx : R(0), ax1 = sx > 0 ? -hx : R(0);   // far-node weights of the cell entered
+    const R ay0 = sy < 0 ? hy : R(0), ay1 = sy > 0 ? -hy : R(0);
+    const R gxo = nq * (Xc - X1), gyo = nq * (Yc - Y1);
+    const R mxc = R(0.5) * (x0 + Xc), myc = R(0.5) * (y0 + Yc);
+    gx = nq * (x0 - Xc); gy = nq * (y0 - Yc);
+    mx0 = R(1) - mxc - ax0; mx1 = mxc - ax1; my0 = R(1) - myc - ay0; my1 = myc - ay1;
+    if constexpr (kShare) {
+      if (sx) add_faces_shared(p, i + sx, j, gxo * my0, gxo * my1, gy * ax0, gy * ax1);
+      if (sy) add_faces_shared(p, i, j + sy, gx * ay0, gx * ay1, gyo * mx0, gyo * mx1);
+      if (sx && sy) add_faces_shared(p, i + sx, j + sy, gxo * ay0, gxo * ay1, gyo * ax0, gyo * ax1);
+    } else {
+      if (sx) add_faces(p, i + sx, j, gxo * my0, gxo * my1, gy * ax0, gy * ax1);
+      if (sy) add_faces(p, i, j + sy, gx * ay0, gx * ay1, gyo * mx0, gyo * mx1);
+      if (sx && sy) add_faces(p, i + sx, j + sy, gxo * ay0, gxo * ay1, gyo * ax0, gyo * ax1);
+    }
+    if (sx && (below_zero(wx) || at_least(wx, R(1)))) { ic += sx; wx -= R(sx); }
+    if (sy && (below_zero(wy) || at_least(wy, R(1)))) { jc += sy; wy -= R(sy); }
+  }
+  const R qv = qw * vphi, a1 = qv * wx, a0 = qv - a1, a01 = a0 * wy, a11 = a1 * wy;
+  if constexpr (kShare) {
+    float v[8] = {gx * my0, gx * my1, gy * mx0, gy * mx1, a0 - a01, a01, a1 - a11, a11};
+    if (ic != i || jc != j) {   // mid-point in the cell entered: on its own
+      add_corners(p, ic, jc, v[4], v[5], v[6], v[7]);
+      v[4] = v[5] = v[6] = v[7] = 0.f;
+    }
+    if (sum_by_cell(i * p.nt + j, v)) {
+      add_faces(p, i, j, v[0], v[1], v[2], v[3]);
+      add_corners(p, i, j, v[4], v[5], v[6], v[7]);
+    }
+    return;
+  }
+  add_faces(p, i, j, gx * my0, gx * my1, gy * mx0, gy * mx1);
+  add_corners(p, ic, jc, a0 - a01, a01, a1 - a11, a11);
 }
 
 template <typename R> __device__ __forceinline__ R one_minus_ulp();
@@ -388,22 +595,34 @@ struct Tally {
   R killed, radiated;
   unsigned nonfinite;
   unsigned pushed;
+  __device__ __forceinline__ void add(const Tally &t) {
+    killed += t.killed; radiated += t.radiated;
+    nonfinite += t.nonfinite; pushed += t.pushed;
+  }
 };
 
-// per-species constants of a push, loaded once per work item.  In (read)
-// and S (written) are the same arrays, except in the first push after a sort,
-// which reads the unsorted parity through the sorted order sidx.
+// per-species constants of a push, loaded once per work item.  The arrays
+// read (in) and written (out) are the same, except in the first push after a
+// sort, which reads the unsorted parity through the sorted order sidx.  xo,
+// yo, ur, ut, up, w of a species lie p.pstride elements apart, so that one
+// address serves all six.
 template <typename R>
 struct SpeciesConst {
-  Species<R> S, In;
+  const int32_t *cell_in;
+  int32_t *cell_out;
+  const R *x_in;
+  R *x_out;
+  int64_t stride;
   const uint32_t *sidx;
   R qm, krr, q, m;
   uint32_t key_hi;   // species in the top bit of a pair-creation event key
   bool creates;      // a lepton of a run with pair creation
   __device__ __forceinline__ SpeciesConst(const Params<R> &p, int s, bool gather = false)
-      : S(p.sp[s]), In(gather ? p.src[s] : p.sp[s]), sidx(p.sidx[s]), qm(p.qm[s]),
-        krr(p.krr[s] * (R)(*p.rr_scale)), q(p.q[s]), m(p.m[s]), key_hi((uint32_t)s << 31),
-        creates(p.pairs != 0 && s < 2) {}
+      : cell_in(gather ? p.src[s].cell : p.sp[s].cell), cell_out(p.sp[s].cell), x_in(gather ? p.src[s].xo : p.sp[s].xo),
+        x_out(p.sp[s].xo), stride(p.pstride), sidx(p.sidx[s]), qm(p.qm[s]), krr(p.krr[s] * (R)(*p.rr_scale)), q(p.q[s]),
+        m(p.m[s]), key_hi((uint32_t)s << 31), creates(p.pairs != 0 && s < 2) {}
+  __device__ __forceinline__ R in(int k, int q) const { return x_in[q + k * stride]; }
+  __device__ __forceinline__ R &out(int k, int q) const { return x_out[q + k * stride]; }
 };
 
 // Sect. 5.1: a lepton above the threshold Lorentz factor creates a pair at
@@ -425,93 +644,120 @@ __device__ __forceinline__ void record_pair(const Params<R> &p, const SpeciesCon
   p.ev_w[e] = w;
 }
 
-// One particle: gather, push, move, kill rules, deposit, store.  Reads
-// particle qi of K.In and writes slot q of K.S (the same particle unless the
-// push also performs a sort's payload gather, kGather, which writes w too).
-template <typename R, bool kGather, typename M>
-__device__ __forceinline__ void push_one(const M &m, const Params<R> &p, const SpeciesConst<R> &K, int q,
-                                         int qi, int i, int j, Tally<R> &tl) {
-  constexpr bool kShared = std::is_same<M, SharedMesh<R>>::value;
-  const Species<R> &S = K.S;
-  const Species<R> &In = K.In;
-  const int nt = p.nt, nr = p.nr;
-  const R xo = In.xo[qi], yo = In.yo[qi], w = In.w[qi];
-  R u[3] = {In.ur[qi], In.ut[qi], In.up[qi]};
-  R e[3], b[3], un[3], dg;
+// What holds for every particle of a work item (or, outside the tiles, what
+// cannot be assumed), so that most particles skip the tests:
+//   small  a step's displacement is small against the distance to the axis:
+//          |d_phi|, |b| <= dt < 0.028 (r sin(theta) - 2 dt) over the region;
+//   shell  some may lie inside shell_r;
+//   edge   some may reach a wall, the axis or the absorber.
+struct TileFacts {
+  bool small, shell, edge;
+};
+
+// One particle in cell (i, j): gather, push, move, kill rules, deposit, and
+// its new state in slot q (the slot it came from, unless the push also
+// performs a sort's payload gather, kGather, which writes w too).
+template <typename R, bool kGather, bool kShare, typename M>
+__device__ __forceinline__ void push_one(const M &m, const TileFacts &F, const Params<R> &p, const SpeciesConst<R> &K,
+                                         int q, int i, int j, R xo, R yo, R w, const R u[3], Tally<R> &tl) {
+  using P = Series<R>;
+  const int nt = p.nt;
+  R e[3], b[3], un[3], uo[3], dg;
+  gather(m, i, j, xo, yo, e, b);
+  R ginv = boris_rr<R>(K.qm, K.krr, p.dt, u, e, b, un, dg);
   tl.pushed += 1;
-  if constexpr (kShared) gather_sh<R>(m, i, j, xo, yo, e, b);
-  else gather<R>(m, nr, nt, i, j, xo, yo, e, b);
-  boris_rr<R>(K.qm, K.krr, p.dt, u, e, b, un, dg);
-  tl.radiated += w * K.m * dg;
+  if (K.krr != R(0)) tl.radiated += w * K.m * dg;
   // position of the particle: r = r_i exp(xo D), theta = theta_j + yo dtheta
   const R xl = xo * p.dlog, ya = yo * p.dth;
   R ex, sa0, ca0;
   if (p.small_grid) {
-    ex = exp_small(xl);
-    sa0 = sin_small(ya);
-    ca0 = cos_small(ya);
+    const R y2 = ya * ya;
+    sa0 = ya * P::sinc(y2);
+    ca0 = vfma(y2, P::cosm(y2), R(1));
+    ex = vfma(xl, P::expm1c(xl), R(1));
   } else {
-    ex = exp(xl);
     sincos(ya, &sa0, &ca0);
+    ex = exp(xl);
   }
-  const R r = m.rn(i) * ex;
-  const R snj = m.sn(j), cnj = m.cn(j);
-  const R sn = snj * ca0 + cnj * sa0, cs = cnj * ca0 - snj * sa0;
-  if (r * r < p.shell_r2) {  // Sect. 5.1: no momentum across B near the star
-    const R b2 = b[0] * b[0] + b[1] * b[1] + b[2] * b[2];
+  const R r = m.rn(i) * ex, snj = m.sn(j), cnj = m.cn(j);
+  const R sn = vfma(snj, ca0, cnj * sa0), cs = vfma(cnj, ca0, -(snj * sa0));
+  if (F.shell && r * r < p.shell_r2) {  // Sect. 5.1: no momentum across B near the star
+    const R b2 = dot3(b, b);
     if (b2 > R(1e-30)) {
-      const R ub = (un[0] * b[0] + un[1] * b[1] + un[2] * b[2]) * rcp(b2);
-      un[0] = ub * b[0]; un[1] = ub * b[1]; un[2] = ub * b[2];
+      const R ub = dot3(un, b) * rcp(b2);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) un[k] = ub * b[k];
+      ginv = rsq(dot3(un, un, R(1)));
     }
   }
-  R dr, dth, uo[3];
-  if (!move_small<R>(r, sn, cs, p.dt, un, dr, dth, uo)) move_general<R>(r, sn, cs, p.dt, un, dr, dth, uo);
-  const R ginv = rsq(R(1) + un[0] * un[0] + un[1] * un[1] + un[2] * un[2]);
-  const R xr = dr * rcp(r);
-  R X1 = xo + ((fabs(xr) < R(kSmall)) ? log1p_small(xr) : log1p(xr)) * p.inv_dlog;
-  R Y1 = yo + dth * p.inv_dth;
-  if (!isfinite(X1) || !isfinite(Y1) || !isfinite(uo[0] + uo[1] + uo[2])) {
-    S.cell[q] = -1;
+  R xr, dth;
+  move<R>(F.small, r, sn, cs, ginv, p.dt, un, xr, dth, uo);
+  const R lg = (F.small || !at_least(fabs(xr), R(0.03125))) ? xr * P::log1pc(xr) : R(log1p(xr));
+  R X1 = vfma(lg, p.inv_dlog, xo), Y1 = vfma(dth, p.inv_dth, yo);
+  if (!all_finite(X1, Y1, uo)) {
+    K.cell_out[q] = -1;
     tl.nonfinite += 1;
     return;
   }
-  if (R(j) + Y1 < R(0)) Y1 = R(-2 * j) - Y1;
-  if (R(j) + Y1 > R(nt)) Y1 = R(2 * (nt - j)) - Y1;
-  bool dead = false;
-  if (R(i) + X1 < R(0)) { X1 = -R(i); dead = true; }
-  else if (R(i) + X1 > p.xi_abs) dead = true;
-  int di = (int)floor(X1), dj = (int)floor(Y1);
-  R xn = X1 - R(di), yn = Y1 - R(dj);
-  if (xn >= R(1)) { xn -= R(1); di += 1; }
-  if (yn >= R(1)) { yn -= R(1); dj += 1; }
-  const int i1 = i + di;
-  int j1 = j + dj;
-  if (j1 >= nt) { j1 = nt - 1; yn = one_minus_ulp<R>(); }
-  if (!dead && (i1 >= nr || m.ff(i1, j1))) dead = true;  // off the mesh (no absorber), or force-free
-  deposit<R>(p, K.q * w, i, j, xo, yo, X1, Y1, un[2] * ginv);
+  bool dead = F.edge && i >= p.i_abs && R(i) + X1 > p.xi_abs;
+  int sx = 0, sy = 0, i1 = i, j1 = j;
+  R xn = X1, yn = Y1;
+  // A step moves a particle by less than a cell in either direction (Courant
+  // number <= 0.9 at the innermost cells, the smallest; at most 0.965 cells
+  // over all grids with nt >= 8), so the entered cell is a neighbour.
+  if (!(stays(X1) && stays(Y1))) {
+    bool lo = below_zero(X1), yl = below_zero(Y1), yh = at_least(Y1, R(1));
+    const bool hi = at_least(X1, R(1));
+    if (F.edge) {
+      if (j == 0 && yl) { Y1 = -Y1; yl = false; }
+      if (j == nt - 1 && yh && Y1 > R(1)) { Y1 = R(2) - Y1; yh = false; }
+      if (i == 0 && lo) { X1 = R(0); lo = false; dead = true; }
+    }
+    sx = lo ? -1 : (hi ? 1 : 0);
+    sy = yl ? -1 : (yh ? 1 : 0);
+    xn = X1 - R(sx);
+    yn = Y1 - R(sy);
+    // a tiny step below the node, rounded back to it, stays in the cell
+    if (lo && at_least(xn, R(1))) { xn = R(0); sx = 0; }
+    if (yl && at_least(yn, R(1))) { yn = R(0); sy = 0; }
+    i1 += sx;
+    j1 += sy;
+    if (j1 >= nt) { j1 = nt - 1; yn = one_minus_ulp<R>(); sy = 0; }
+    // the deposit ends where the particle is stored (its offset was rounded
+    // on the way down; these sums are exact), or Gauss's law would drift
+    X1 = xn + R(sx);
+    Y1 = yn + R(sy);
+  }
+  // off the mesh (no absorber), or force-free
+  if (!dead) dead = (F.edge && i1 >= p.nr) || m.ff(i1, j1);
+  deposit<kShare, R>(p, K.q * w, i, j, sx, sy, xo, yo, X1, Y1, un[2] * ginv);
   if (dead) {
-    S.cell[q] = -1;
+    K.cell_out[q] = -1;
     tl.killed += w;
     return;
   }
-  S.cell[q] = i1 * nt + j1;
-  S.xo[q] = xn; S.yo[q] = yn;
-  S.ur[q] = uo[0]; S.ut[q] = uo[1]; S.up[q] = uo[2];
-  if constexpr (kGather) S.w[q] = w;
-  if (i1 == 0 && p.inject) atomicAdd(&p.surf[j1], 1);
+  K.cell_out[q] = i1 * nt + j1;
+  K.out(0, q) = xn; K.out(1, q) = yn;
+  K.out(2, q) = uo[0]; K.out(3, q) = uo[1]; K.out(4, q) = uo[2];
+  if constexpr (kGather) K.out(5, q) = w;
+  if (F.edge && i1 == 0 && p.inject) atomicAdd(&p.surf[j1], 1);
   if (K.creates) record_pair(p, K, q, i1 * nt + j1, xn, yn, uo, w);
 }
 
-// out-of-region fallback of the tiled kernel.  It returns its counts by
+// one particle outside the tiles (appended since the sort, drifted out of the
+// staged region, or the no-sort configuration).  It returns its counts by
 // value and takes the species index rather than the species constants:
 // arguments passed by reference to an out-of-line call would have to live
 // in local memory for the whole work item.
 template <typename R, bool kGather>
-__device__ __forceinline__ Tally<R> push_one_global(const Params<R> &p, int s, int q, int qi, int i, int j) {
+__device__ __noinline__ Tally<R> push_one_global(const Params<R> &p, int s, int slot, int from, int cell) {
   const SpeciesConst<R> K(p, s, kGather);
   GlobalMesh<R> g(p);
   Tally<R> tl{R(0), R(0), 0u, 0u};
-  push_one<R, kGather>(g, p, K, q, qi, i, j, tl);
+  int i, j;
+  decode_cell(p, cell, i, j);
+  const R u[3] = {K.in(2, from), K.in(3, from), K.in(4, from)};
+  push_one<R, kGather, false>(g, TileFacts{false, true, true}, p, K, slot, i, j, K.in(0, from), K.in(1, from), K.in(5, from), u, tl);
   return tl;
 }
 
@@ -539,19 +785,13 @@ __device__ __forceinline__ void flush_tally(const Tally<R> &tl, double *acc, uns
 // from its last block (which the tiled kernel gives a work item last)
 template <typename R>
 __device__ __forceinline__ Tally<R> push_tail(const Params<R> &p) {
-  GlobalMesh<R> m(p);
   Tally<R> tl{R(0), R(0), 0u, 0u};
   for (int s = 0; s < p.n_species; ++s) {
     const int64_t n0 = p.count_sorted[s], n1 = p.count[s];
-    int64_t q = n0 + (gridDim.x - 1 - blockIdx.x) * (int64_t)blockDim.x + threadIdx.x;
-    if (q >= n1) continue;
-    const SpeciesConst<R> K(p, s);
-    for (; q < n1; q += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t q = n0 + (gridDim.x - 1 - blockIdx.x) * (int64_t)blockDim.x + threadIdx.x; q < n1;
+         q += (int64_t)gridDim.x * blockDim.x) {
       const int c = p.sp[s].cell[q];
-      if (c < 0) continue;
-      int i, j;
-      decode_cell(p, c, i, j);
-      push_one<R, false>(m, p, K, (int)q, (int)q, i, j, tl);
+      if (c >= 0) tl.add(push_one_global<R, false>(p, s, (int)q, (int)q, c));
     }
   }
   return tl;
@@ -562,22 +802,102 @@ __global__ void __launch_bounds__(256) k_push_tail(const __grid_constant__ Param
 }
 
 // ---------------------------------------------------------- tiled kernel
-// Region of a tile: cells [ti*TR - H, (ti+1)*TR + H) (and likewise in theta)
+static_assert(kPushThreads * 32 >= kMaxItem, "one bit per round of a work item");
+// The next round's particles are copied to shared memory while this round's
+// are pushed (one slot per thread and array, read back by the thread that
+// copied it): the loads' latency, lengthened by the reductions in the L2's
+// queues, was the largest stall, and registers have no room for them.
+template <int B> __device__ __forceinline__ void copy_async(void *dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "n"(B)
+               : "memory");
+}
+template <typename R>
+struct Prefetch {
+  R *slot;   // 7 arrays of kPushThreads slots (the first holds the cells)
+  __device__ __forceinline__ void start(const SpeciesConst<R> &K, int q, bool any) const {
+    if (any) {
+      R *d = slot + threadIdx.x;
+      copy_async<4>(d, K.cell_in + q);
+      const R *a = K.x_in + q;
+#pragma unroll
+      for (int k = 1; k < 7; ++k, a += K.stride) copy_async<sizeof(R)>(d + k * kPushThreads, a);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  __device__ __forceinline__ void wait() const { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+  __device__ __forceinline__ int cell() const { return *reinterpret_cast<const int *>(slot + threadIdx.x); }
+  __device__ __forceinline__ R get(int k) const { return slot[(k + 1) * kPushThreads + threadIdx.x]; }
+};
+
+// particles of slots q0 .. q1 of a work item, one per thread and round
+template <typename R, bool kGather, bool kShare>
+__device__ __forceinline__ void push_item(const SharedMesh<R> &m, const TileFacts &F, const Params<R> &p,
+                                          const SpeciesConst<R> &K, const Prefetch<R> &pre, int s, int q0, int q1, int lr,
+                                          Tally<R> &tl) {
+  // rounds whose particle was left for the global path: an item has at most
+  // kMaxItem particles, 32 rounds
+  unsigned left = 0, bit = 1;
+  for (int slot = q0 + (int)threadIdx.x; slot < q1; slot += kPushThreads, bit <<= 1) {
+    int c;
+    R x, y, w, u[3];
+    if constexpr (kGather) {
+      const int from = (int)K.sidx[slot];
+      c = K.cell_in[from];
+      if (c < 0) K.cell_out[slot] = -1;
+      x = K.in(0, from); y = K.in(1, from); w = K.in(5, from);
+      u[0] = K.in(2, from); u[1] = K.in(3, from); u[2] = K.in(4, from);
+    } else {
+      pre.wait();
+      c = pre.cell();
+      x = pre.get(0); y = pre.get(1); u[0] = pre.get(2); u[1] = pre.get(3); u[2] = pre.get(4); w = pre.get(5);
+      pre.start(K, slot + kPushThreads, slot + kPushThreads < q1);
+    }
+    if (c < 0) continue;
+    int i, j;
+    decode_cell(p, c, i, j);
+    // a particle is handled in shared memory when its gather stencil and the
+    // cells it can reach (start cell -1 .. +1) lie inside the region
+    if ((unsigned)(i - m.i0 - 1) < (unsigned)(lr - 2) && (unsigned)(j - m.j0 - 1) < (unsigned)(m.lt - 2))
+      push_one<R, kGather, kShare>(m, F, p, K, slot, i, j, x, y, w, u, tl);
+    else
+      left |= bit;
+  }
+  for (; left; left &= left - 1) {
+    const int slot = q0 + (int)threadIdx.x + kPushThreads * (__ffs(left) - 1);
+    const int from = kGather ? (int)K.sidx[slot] : slot;
+    tl.add(push_one_global<R, kGather>(p, s, slot, from, K.cell_in[from]));
+  }
+}
+
+// Order of the work items: the list is by species and tile, so a tile with
+// many particles (the current sheet: 36 items on the 1024^2 workload) would
+// be pushed by many blocks at once, whose reductions then queue at the few
+// records of its cells.  Within windows of kOrderWindow items an odd stride
+// (a permutation of the window) spreads them; the window keeps the tiles at
+// work, and their fields in the L2, close together.  Push of 5e7 particles on
+// 1024^2: 1.07 ms in list order, 1.03 with 2048 or 4096, 1.05 unlimited.
+constexpr int kOrderWindow = 2048, kOrderStride = 1013;
+__device__ __forceinline__ int item_order(int it, int n) {
+  const int w = it & ~(kOrderWindow - 1);
+  return w + kOrderWindow <= n ? w + ((it * kOrderStride) & (kOrderWindow - 1)) : it;
+}
+
+// Region of a tile: cells [ti*TR - H, ti*TR + TR + H) (and likewise in theta)
 // widened by the gather's stencil: one node on either side.
-// Register budget: five blocks of 256 per SM in FP32 (48 registers, a few
-// spilled values in L1; the region of a 16 x 24 tile fits five times in
-// shared memory), three in FP64, whose doubled region leaves room for no more.
-template <typename R> constexpr int push_tiled_min_blocks() { return sizeof(R) == 4 ? 5 : 3; }
+// Blocks of 256 per SM, measured on 2e7 FP32 particles (2048^2) and 4.6e6
+// FP64 ones (512^2): FP32 with 3, 4, 5 blocks (80, 64, 48 registers) 0.486,
+// 0.478, 0.53 ms; FP64 with 2, 3 (128, 80 registers) 2.93, 2.98 ms.
+template <typename R> constexpr int push_tiled_min_blocks() { return sizeof(R) == 4 ? 4 : 2; }
 template <typename R, bool kGather>
-__global__ void __launch_bounds__(256, push_tiled_min_blocks<R>())
+__global__ void __launch_bounds__(kPushThreads, push_tiled_min_blocks<R>())
     k_push_tiled(const __grid_constant__ Params<R> p, WorkList wl, int halo) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int lr = p.tile_r + 2 * halo + 2, lt = p.tile_t + 2 * halo + 2, area = lr * lt;
-  R *base = reinterpret_cast<R *>(smem);
   SharedMesh<R> m;
-  m.s_er = base; m.s_et = base + area; m.s_ep = base + 2 * area;
-  m.s_br = base + 3 * area; m.s_bt = base + 4 * area; m.s_bp = base + 5 * area;
-  m.s_rn = base + 6 * area; m.s_sn = m.s_rn + lr; m.s_cn = m.s_sn + lt;
+  Prefetch<R> pre;
+  pre.slot = reinterpret_cast<R *>(smem);
+  m.s_rn = reinterpret_cast<R *>(m.carve(smem + 7 * kPushThreads * sizeof(R), area));
+  m.s_sn = m.s_rn + lr; m.s_cn = m.s_sn + lt;
   m.s_ff = reinterpret_cast<uint8_t *>(m.s_cn + lt);
   m.lt = lt;
   __shared__ int s_item;
@@ -586,26 +906,33 @@ __global__ void __launch_bounds__(256, push_tiled_min_blocks<R>())
   for (;;) {
     if (threadIdx.x == 0) s_item = atomicAdd(wl.next, 1);
     __syncthreads();
-    const int it = s_item;
-    if (it >= *wl.n_items) break;
-    const int4 item = wl.items[it];
+    const int it = s_item, ni = *wl.n_items;
+    if (it >= ni) break;
+    const int4 item = wl.items[item_order(it, ni)];
     const int s = item.x, tile = item.y;
     const int ti = tile / p.ntt, tj = tile - ti * p.ntt;
     m.i0 = ti * p.tile_r - halo - 1;
     m.j0 = tj * p.tile_t - halo - 1;
+    const SpeciesConst<R> K(p, s, kGather);
+    int ca = -1, cb = -2;   // cells of a sampled pair of particles (read here, behind the staging too)
+    if constexpr (sizeof(R) == 4) {
+      const int qa = item.z + kShareDist + (int)threadIdx.x * max(1, (item.w - kShareDist) / kPushThreads);
+      if (qa < item.z + item.w) {
+        ca = K.cell_in[kGather ? (int)K.sidx[qa] : qa];
+        cb = K.cell_in[kGather ? (int)K.sidx[qa - kShareDist] : qa - kShareDist];
+      }
+    }
+    if constexpr (!kGather)   // the first round's particles, behind the staging
+      pre.start(K, item.z + (int)threadIdx.x, (int)threadIdx.x < item.w);
     // stage E, B, flags (edge values replicated outside each array)
     for (int k = threadIdx.x; k < area; k += blockDim.x) {
       const int a = k / lt, c = k - a * lt;
       const int gi = m.i0 + a, gj = m.j0 + c;
       const int in = min(max(gi, 0), nr), ih = min(max(gi, 0), nr - 1);   // node / half rows
       const int jn = min(max(gj, 0), nt), jh = min(max(gj, 0), nt - 1);   // node / half columns
-      m.s_er[k] = p.f.er[ix(ih, jn, n1)];
-      m.s_et[k] = p.f.et[ix(in, jh, nt)];
-      m.s_ep[k] = p.f.ep[ix(in, jn, n1)];
-      const int64_t kb = ix(in, jh, nt), kt = ix(ih, jn, n1), kp = ix(ih, jh, nt);
-      m.s_br[k] = p.f.br0[kb] + p.f.br[kb];   // B = B_0 + dB
-      m.s_bt[k] = p.f.bt0[kt] + p.f.bt[kt];
-      m.s_bp[k] = p.f.bp0[kp] + p.f.bp[kp];
+      const int64_t kb = ix(in, jh, nt), kt = ix(ih, jn, n1), kp = ix(ih, jh, nt), kn = ix(in, jn, n1);
+      m.put(k, c, p.f.er[kt], p.f.et[kb], p.f.ep[kn], p.f.br0[kb] + p.f.br[kb],   // B = B_0 + dB
+            p.f.bt0[kt] + p.f.bt[kt], p.f.bp0[kp] + p.f.bp[kp]);
       m.s_ff[k] = (gi >= 0 && gj >= 0 && gi < nr && gj < nt) ? p.f.ffcell[ix(gi, gj, nt)] : 1;
     }
     for (int k = threadIdx.x; k < lr; k += blockDim.x) {
@@ -617,28 +944,21 @@ __global__ void __launch_bounds__(256, push_tiled_min_blocks<R>())
       m.s_sn[k] = (gj >= 0 && gj <= nt) ? p.t.sn[gj] : R(0);
       m.s_cn[k] = (gj >= 0 && gj <= nt) ? p.t.cn[gj] : R(1);
     }
-    const SpeciesConst<R> K(p, s, kGather);
-    const int q0 = item.z, q1 = item.z + item.w;
-    __syncthreads();
-    // a particle is handled in shared memory when its gather stencil and the
-    // cells it can reach (start cell -1 .. +1) lie inside the region
-    for (int q = q0 + (int)threadIdx.x; q < q1; q += (int)blockDim.x) {
-      const int qi = kGather ? (int)K.sidx[q] : q;
-      const int c = K.In.cell[qi];
-      if (c < 0) {
-        if (kGather) K.S.cell[q] = -1;
-        continue;
-      }
-      int i, j;
-      decode_cell(p, c, i, j);
-      if (i - 1 >= m.i0 && i + 1 < m.i0 + lr && j - 1 >= m.j0 && j + 1 < m.j0 + lt)
-        push_one<R, kGather>(m, p, K, q, qi, i, j, tl);
-      else {
-        const Tally<R> t = push_one_global<R, kGather>(p, s, q, qi, i, j);
-        tl.killed += t.killed; tl.radiated += t.radiated;
-        tl.nonfinite += t.nonfinite; tl.pushed += t.pushed;
-      }
+    TileFacts F;
+    // many particles in few cells?  (the barrier also completes the staged region)
+    const bool share = __syncthreads_count(ca == cb && ca >= 0) >= kShareItemMin;
+    {
+      // over the region's nodes inside the mesh
+      const int ra = max(m.i0, 0), rb = min(m.i0 + lr, nr), ca = max(m.j0, 0), cb = min(m.j0 + lt - 1, nt);
+      const R r0 = p.t.rn[ra], sm = min(p.t.sn[ca], p.t.sn[cb]);
+      F.small = p.dt < R(0.028) * (r0 * sm - R(2) * p.dt);
+      F.shell = r0 * r0 < p.shell_r2 * R(1.001);
+      F.edge = ra == 0 || rb == nr || ca == 0 || cb == nt || rb >= p.i_abs;
     }
+    if constexpr (sizeof(R) == 4) {
+      if (share) push_item<R, kGather, true>(m, F, p, K, pre, s, item.z, item.z + item.w, lr, tl);
+    }
+    if (sizeof(R) != 4 || !share) push_item<R, kGather, false>(m, F, p, K, pre, s, item.z, item.z + item.w, lr, tl);
     __syncthreads();
   }
   flush_tally(tl, p.acc, p.status, &p.pushed[0]);
@@ -653,7 +973,8 @@ __global__ void __launch_bounds__(256, push_tiled_min_blocks<R>())
 
 template <typename R> size_t push_tiled_smem(const Params<R> &p, int halo) {
   const size_t lr = p.tile_r + 2 * halo + 2, lt = p.tile_t + 2 * halo + 2, area = lr * lt;
-  return area * (6 * sizeof(R) + 1) + (lr + 2 * lt) * sizeof(R);
+  return 7 * kPushThreads * sizeof(R) + area * SharedMesh<R>::bytes_per_location() +
+         (lr + 2 * lt) * sizeof(R);
 }
 
 // The tiles and cadences that hff_init accepts: those whose region, two
@@ -680,8 +1001,8 @@ template <typename R> void launch_push_tail(const Params<R> &p, cudaStream_t s, 
 }
 template <typename R> void launch_push_tiled(const Params<R> &p, const WorkList &wl, int halo,
                                              cudaStream_t s, int grid, bool gather) {
-  if (gather) k_push_tiled<R, true><<<grid, 256, push_tiled_smem(p, halo), s>>>(p, wl, halo);
-  else k_push_tiled<R, false><<<grid, 256, push_tiled_smem(p, halo), s>>>(p, wl, halo);
+  if (gather) k_push_tiled<R, true><<<grid, kPushThreads, push_tiled_smem(p, halo), s>>>(p, wl, halo);
+  else k_push_tiled<R, false><<<grid, kPushThreads, push_tiled_smem(p, halo), s>>>(p, wl, halo);
 }
 
 // ------------------------------------------------------------- injection
@@ -855,8 +1176,8 @@ template <typename R> cudaError_t set_push_smem(size_t bytes) {
 // (registers and shared memory both counted); 0 on error
 template <typename R> int push_tiled_blocks_per_sm(size_t bytes) {
   int a = 0, b = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_push_tiled<R, false>, 256, bytes) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_push_tiled<R, true>, 256, bytes) != cudaSuccess)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_push_tiled<R, false>, kPushThreads, bytes) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_push_tiled<R, true>, kPushThreads, bytes) != cudaSuccess)
     return 0;
   return a < b ? a : b;
 }
