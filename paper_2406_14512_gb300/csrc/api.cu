@@ -189,7 +189,8 @@ struct Offsets {
   size_t part[2][kMaxSpecies][7];
   size_t small;          // counters block
   size_t surf, target, inj_prefix;
-  size_t keys_a, keys_b, idx_a, idx_b, hist, spart, tstart, tend;
+  size_t keys, idx, hist, spart, bounds, nsort;
+  int64_t sort_stride, hist_stride, part_stride;  // words per species
   size_t sidx[kMaxSpecies];  // sorted order of the last sort, per species
   size_t items;
   size_t qnode, rows, psi64;
@@ -263,12 +264,16 @@ void layout(const hff_config &c, Offsets &o) {
   o.max_items = c.n_species * (o.ntiles + (int)((cap + kChunkMin - 1) / kChunkMin)) + 1;
   if (c.sort_every > 0) {
     for (int s = 0; s < c.n_species; ++s) o.sidx[s] = L.take(cap * 4);
-    o.keys_a = L.take(cap * 4); o.keys_b = L.take(cap * 4);
-    o.idx_a = L.take(cap * 4); o.idx_b = L.take(cap * 4);
-    o.hist = L.take((size_t)o.nb * 256 * 4 + 4);
-    o.spart = L.take((size_t)o.nparts * 4 + 4);
-    o.tstart = L.take(((size_t)o.ntiles + 1) * 4);
-    o.tend = L.take(((size_t)o.ntiles + 1) * 4);
+    const size_t ns = c.n_species;
+    o.sort_stride = ((int64_t)cap + 63) & ~int64_t(63);
+    o.hist_stride = (int64_t)o.nb * 256 + 64;
+    o.part_stride = (o.nparts + 64) & ~63;
+    o.keys = L.take(ns * 2 * o.sort_stride * 4);
+    o.idx = L.take(ns * 2 * o.sort_stride * 4);
+    o.hist = L.take(ns * o.hist_stride * 4);
+    o.spart = L.take(ns * o.part_stride * 4);
+    o.bounds = L.take(ns * 2 * ((size_t)o.ntiles + 1) * 4);
+    o.nsort = L.take((kMaxSpecies + 1) * 8);  // and the unsettled flag
     o.items = L.take((size_t)o.max_items * sizeof(int4));
   }
   // pair-creation events of one step (bounded; overflow is latched)
@@ -696,11 +701,10 @@ template <typename R>
 int enqueue_sort(hff_handle *h, int par, cudaStream_t s, bool gather) {
   if (h->c.capacity <= 0) return HFF_OK;  // nothing to sort
   Params<R> &p = params<R>(h)[par];
-  Params<R> &q = params<R>(h)[par ^ 1];
-  for (int sp = 0; sp < h->c.n_species; ++sp) {
-    launch_sort_species<R>(p, sp, q.sp[sp], h->ss, s, gather);
-    launch_worklist<R>(p, &h->ss, h->wl, sp, sp == 0 ? 1 : 0, s);
-  }
+  launch_sort<R>(p, h->ss, s);
+  launch_worklist<R>(p, h->ss, h->wl, s);
+  if (gather)
+    for (int sp = 0; sp < h->c.n_species; ++sp) launch_materialize<R>(params<R>(h)[par ^ 1], sp, s);
   CK(cudaGetLastError());
   return HFF_OK;
 }
@@ -1143,14 +1147,16 @@ static int init_one(const hff_config *cfg, void *dev_mem, size_t bytes, void *st
   h->wl.done = &h->small->done;
   h->wl.max_items = h->o.max_items;
   h->wl.chunk = chunk_of(*cfg);
-  h->ss.keys_a = reinterpret_cast<uint32_t *>(h->base + h->o.keys_a);
-  h->ss.keys_b = reinterpret_cast<uint32_t *>(h->base + h->o.keys_b);
-  h->ss.idx_a = reinterpret_cast<uint32_t *>(h->base + h->o.idx_a);
-  h->ss.idx_b = reinterpret_cast<uint32_t *>(h->base + h->o.idx_b);
+  h->ss.keys = reinterpret_cast<uint32_t *>(h->base + h->o.keys);
+  h->ss.idx = reinterpret_cast<uint32_t *>(h->base + h->o.idx);
   h->ss.hist = reinterpret_cast<uint32_t *>(h->base + h->o.hist);
   h->ss.part = reinterpret_cast<uint32_t *>(h->base + h->o.spart);
-  h->ss.tile_start = reinterpret_cast<int *>(h->base + h->o.tstart);
-  h->ss.tile_end = reinterpret_cast<int *>(h->base + h->o.tend);
+  h->ss.bounds = reinterpret_cast<int *>(h->base + h->o.bounds);
+  h->ss.n_sort = reinterpret_cast<long long *>(h->base + h->o.nsort);
+  h->ss.unsettled = reinterpret_cast<int *>(h->ss.n_sort + kMaxSpecies);
+  h->ss.stride = h->o.sort_stride;
+  h->ss.hist_stride = h->o.hist_stride;
+  h->ss.part_stride = h->o.part_stride;
   h->ss.cap = cfg->capacity;
   h->ss.ntiles = h->o.ntiles;
   int dev = 0, nsm = 0;
@@ -1164,6 +1170,7 @@ static int init_one(const hff_config *cfg, void *dev_mem, size_t bytes, void *st
     if (e != cudaSuccess) return bail(fail(HFF_ERR_CUDA, "cannot set the flux-prefix shared memory size"));
     const cudaError_t e2 = cfg->precision == HFF_FP64 ? set_field_fused_smem<double>(field_fused_smem<double>())
                                                       : set_field_fused_smem<float>(field_fused_smem<float>());
+    if (set_sort_smem() != cudaSuccess) return bail(fail(HFF_ERR_CUDA, "cannot set the sort's shared memory size"));
     if (e2 != cudaSuccess) return bail(fail(HFF_ERR_CUDA, "cannot set the fused field update's shared memory size"));
     h->fused = fused_fields(*cfg);
     // one wave of the fused field update at its occupancy on this device
@@ -1195,6 +1202,78 @@ static int init_one(const hff_config *cfg, void *dev_mem, size_t bytes, void *st
   return HFF_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+// the arrays of a species in buffer parity pp, or the caller's
+template <typename R>
+Species<R> species_of(const void *const src[7]) {
+  Species<R> s;
+  s.cell = const_cast<int32_t *>(static_cast<const int32_t *>(src[0]));
+  R **q[6] = {&s.xo, &s.yo, &s.ur, &s.ut, &s.up, &s.w};
+  for (int k = 0; k < 6; ++k) *q[k] = const_cast<R *>(static_cast<const R *>(src[k + 1]));
+  return s;
+}
+
+// A load with sorting: the species' particles go straight from the caller's
+// device arrays (or, from the host, from its slots of the current buffer)
+// into sorted order there; the other species stay where they are, unless they
+// are not as a sort leaves them (particles removed or appended since): then
+// all are sorted, as on the cadence.
+template <typename R>
+int load_sorted(hff_handle *h, int species, int64_t n, const void *const src[7], int where, bool *bad) {
+  char *mine[2][7];
+  for (int par = 0; par < 2; ++par)
+    for (int k = 0; k < 7; ++k) mine[par][k] = h->base + h->o.part[par][species][k];
+  const int pp = h->parity;
+  const void *from[7];
+  bool inside = false;   // device arrays inside the instance's own memory
+  for (int k = 0; k < 7; ++k) {
+    from[k] = src[k];
+    const char *c = static_cast<const char *>(src[k]);
+    const size_t b = (size_t)n * (k == 0 ? 4 : sizeof(R));
+    if (where == HFF_DEVICE && n > 0 && c < h->base + h->o.total && c + b > h->base) inside = true;
+  }
+  // records fit the other parity's arrays of two or more species
+  void *rec = h->c.n_species >= 2 ? (void *)(h->base + h->o.part[pp ^ 1][0][0]) : nullptr;
+  if (where == HFF_HOST || inside) {
+    // staged in the current buffer (read by the packing before the sorted
+    // particles overwrite it), or in the other one where there is no packing
+    const int to = rec && !inside ? pp : pp ^ 1;
+    if (inside) rec = nullptr;
+    for (int k = 0; k < 7; ++k) {
+      const cudaMemcpyKind kind = where == HFF_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
+      if (n > 0) CK(cudaMemcpyAsync(mine[to][k], src[k], (size_t)n * (k == 0 ? 4 : sizeof(R)), kind, h->st));
+      from[k] = mine[to][k];
+    }
+  }
+  Params<R> &p = params<R>(h)[pp];
+  launch_load_sorted<R>(p, species, species_of<R>(from), n, rec, h->ss, h->ss.unsettled, h->st);
+  launch_worklist<R>(p, h->ss, h->wl, h->st);
+  CK(cudaGetLastError());
+  unsigned st = 0;
+  int unsettled = 0;
+  CK(cudaMemcpyAsync(&st, &h->small->status, sizeof(st), cudaMemcpyDeviceToHost, h->st));
+  CK(cudaMemcpyAsync(&unsettled, h->ss.unsettled, sizeof(int), cudaMemcpyDeviceToHost, h->st));
+  CK(cudaStreamSynchronize(h->st));
+  *bad = (st & kStBadCell) != 0;
+  if (*bad) {  // clear this bit only; other latched errors stay for hff_status
+    const unsigned rest = st & ~kStBadCell;
+    CK(cudaMemcpyAsync(&h->small->status, &rest, sizeof(rest), cudaMemcpyHostToDevice, h->st));
+  }
+  if (unsettled) {
+    const int rc = run_sort_now<R>(h, h->st);
+    if (rc != HFF_OK) return rc;
+  }
+  if (*bad || unsettled) CK(cudaStreamSynchronize(h->st));
+  return HFF_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
 int hff_load_particles(hff_handle *h, int inst, int species, int64_t n, const int32_t *cell, const void *xo,
                        const void *yo, const void *ur, const void *ut, const void *up, const void *w, int where) {
   h = member(h, inst);
@@ -1206,37 +1285,37 @@ int hff_load_particles(hff_handle *h, int inst, int species, int64_t n, const in
     if (rc != HFF_OK) return rc;
   }
   if (n > h->c.capacity) return fail(HFF_ERR_CAPACITY, "more particles than capacity");
-  const size_t R = h->c.precision == HFF_FP64 ? 8 : 4;
-  const int pp = (h->c.sort_every > 0) ? h->parity : 0;
-  const cudaMemcpyKind kind = where == HFF_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
   const void *src[7] = {cell, xo, yo, ur, ut, up, w};
-  for (int k = 0; k < 7; ++k) {
+  for (int k = 0; k < 7; ++k)
     if (n > 0 && !src[k]) return fail(HFF_ERR_ARG, "null particle array");
-    if (n > 0) CK(cudaMemcpyAsync(h->base + h->o.part[pp][species][k], src[k], n * (k == 0 ? 4 : R), kind, h->st));
-  }
-  if (h->c.capacity > n)
-    CK(cudaMemsetAsync(h->base + h->o.part[pp][species][0] + n * 4, 0xFF, (h->c.capacity - n) * 4, h->st));
-  // a cell index at or past nr * nt is invalid input: that particle is
-  // removed (cell = -1) and the load reports HFF_ERR_ARG after completing
-  launch_check_cells(reinterpret_cast<int32_t *>(h->base + h->o.part[pp][species][0]), n,
-                     (int64_t)h->c.nr * h->c.nt, &h->small->status, h->st);
-  const long long nn = n, zero = 0;
-  CK(cudaMemcpyAsync(&h->small->count[species], &nn, sizeof(nn), cudaMemcpyHostToDevice, h->st));
-  CK(cudaMemcpyAsync(&h->small->count_sorted[species], &zero, sizeof(zero), cudaMemcpyHostToDevice, h->st));
-  unsigned st = 0;
-  CK(cudaMemcpyAsync(&st, &h->small->status, sizeof(st), cudaMemcpyDeviceToHost, h->st));
-  CK(cudaStreamSynchronize(h->st));
-  if (st & kStBadCell) {  // clear this bit only; other latched errors stay for hff_status
-    const unsigned rest = st & ~kStBadCell;
-    CK(cudaMemcpyAsync(&h->small->status, &rest, sizeof(rest), cudaMemcpyHostToDevice, h->st));
-  }
-  if (h->c.sort_every > 0) {
-    const int rc = h->c.precision == HFF_FP64 ? run_sort_now<double>(h, h->st) : run_sort_now<float>(h, h->st);
+  bool bad = false;
+  if (h->c.sort_every > 0 && h->c.capacity > 0) {
+    const int rc = h->c.precision == HFF_FP64 ? load_sorted<double>(h, species, n, src, where, &bad)
+                                              : load_sorted<float>(h, species, n, src, where, &bad);
     if (rc != HFF_OK) return rc;
+  } else {
+    const size_t R = h->c.precision == HFF_FP64 ? 8 : 4;
+    const cudaMemcpyKind kind = where == HFF_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
+    for (int k = 0; k < 7; ++k)
+      if (n > 0) CK(cudaMemcpyAsync(h->base + h->o.part[0][species][k], src[k], n * (k == 0 ? 4 : R), kind, h->st));
+    // a cell index at or past nr * nt is invalid input: that particle is
+    // removed (cell = -1) and the load reports HFF_ERR_ARG after completing
+    launch_check_cells(reinterpret_cast<int32_t *>(h->base + h->o.part[0][species][0]), n,
+                       (int64_t)h->c.nr * h->c.nt, &h->small->status, h->st);
+    const long long nn = n, zero = 0;
+    CK(cudaMemcpyAsync(&h->small->count[species], &nn, sizeof(nn), cudaMemcpyHostToDevice, h->st));
+    CK(cudaMemcpyAsync(&h->small->count_sorted[species], &zero, sizeof(zero), cudaMemcpyHostToDevice, h->st));
+    unsigned st = 0;
+    CK(cudaMemcpyAsync(&st, &h->small->status, sizeof(st), cudaMemcpyDeviceToHost, h->st));
+    CK(cudaStreamSynchronize(h->st));
+    bad = (st & kStBadCell) != 0;
+    if (bad) {
+      const unsigned rest = st & ~kStBadCell;
+      CK(cudaMemcpyAsync(&h->small->status, &rest, sizeof(rest), cudaMemcpyHostToDevice, h->st));
+      CK(cudaStreamSynchronize(h->st));
+    }
   }
-  CK(cudaStreamSynchronize(h->st));
-  if (st & kStBadCell)
-    return fail(HFF_ERR_ARG, "a particle cell index is at or past nr * nt; such particles were removed");
+  if (bad) return fail(HFF_ERR_ARG, "a particle cell index is at or past nr * nt; such particles were removed");
   return HFF_OK;
 }
 
@@ -1796,9 +1875,6 @@ int hff_checkpoint_load(hff_handle *h, int inst, const void *src, size_t bytes) 
       if (n) CK(cudaMemcpyAsync(h->base + h->o.part[pp][s][k], in, n, cudaMemcpyHostToDevice, h->st));
       in += n;
     }
-    if (h->c.capacity > hd.count[s])
-      CK(cudaMemsetAsync(h->base + h->o.part[pp][s][0] + hd.count[s] * 4, 0xFF,
-                         (size_t)(h->c.capacity - hd.count[s]) * 4, h->st));
   }
   // counters: the saved state was sorted, so the sorted prefix is everything
   Small sm;

@@ -103,11 +103,12 @@ __device__ __forceinline__ uint32_t fastdiv(const FastDiv &q, uint32_t n) {
 }
 
 // the radix sort's blocks: kSortItems rounds of kSortThreads slots each, one
-// 256-bin histogram column per block (the histogram matrix the scans pass
-// over shrinks as the blocks grow), scanned in kScanBlock pieces
+// 256-bin histogram column per block, scanned in kScanBlock pieces (with 16
+// rounds the scatter's registers leave 4 blocks per SM and it takes 1.35 times
+// as long, more than the halved histogram matrix saves)
 constexpr int kSortThreads = 256;
-constexpr int kSortItems = 16;
-constexpr int kSortBlock = kSortThreads * kSortItems;  // 4096 slots
+constexpr int kSortItems = 8;
+constexpr int kSortBlock = kSortThreads * kSortItems;  // 2048 slots
 constexpr int kScanBlock = 4096;
 
 template <typename R>
@@ -320,29 +321,33 @@ template <typename R> cudaError_t set_push_smem(size_t bytes);
 template <typename R> int push_tiled_blocks_per_sm(size_t bytes);
 
 struct SortScratch {
-  uint32_t *keys_a, *keys_b;   // cap
-  uint32_t *idx_a, *idx_b;     // cap
-  uint32_t *hist;              // 256 * max_blocks
-  uint32_t *part;              // block sums of the scan
-  int *tile_start;             // [ntiles + 1] first sorted slot of each tile
-  int *tile_end;               // [ntiles + 1] one past its last slot
-  int64_t cap;
-  int64_t pstride;          // elements from one real array of a species to the next (xo .. w)
+  uint32_t *keys, *idx;        // two buffers per species, `stride` words apart
+  uint32_t *hist;              // per species: 256 words per block
+  uint32_t *part;              // per species: block sums of the scan
+  long long *n_sort;           // per species: slots the sort under way runs over
+  int *bounds;                 // per species: first sorted slot of each tile, then one past its last
+  int *unsettled;              // set by launch_load_sorted (see there)
+  int64_t cap, stride, hist_stride, part_stride;
   int ntiles;
 };
 
-// Sort one species of parity p into the other parity dst.  The sorted order
-// is left in p.sidx[species]; with gather the payload moves now, otherwise
-// only the count and the removed slots of dst are set and the next push moves
-// the payload (launch_materialize does it eagerly).
-template <typename R> void launch_sort_species(const Params<R> &p, int species, Species<R> dst,
-                                               const SortScratch &ss, cudaStream_t s, bool gather);
+// Sort every species of parity p: the sorted order is left in p.sidx, the
+// counts are compacted and the tile bounds taken; the payload moves with the
+// next push (or launch_materialize) into the other parity.
+template <typename R> void launch_sort(const Params<R> &p, const SortScratch &ss, cudaStream_t s);
+// Particles src (n, in any order) of one species into parity p, sorted; src is
+// outside p's arrays, or, with `records` (n records of load_record_bytes, in
+// neither), may be them.  The other species are left alone; their tile bounds
+// are taken afresh, and *unsettled is set if one is not as a sort leaves it.
+template <typename R> void launch_load_sorted(const Params<R> &p, int species, const Species<R> &src, int64_t n,
+                                              void *records, const SortScratch &ss, int *unsettled, cudaStream_t s);
+template <typename R> size_t load_record_bytes();
+cudaError_t set_sort_smem();
 // the deferred payload gather of a species, src -> sp by sidx (slots < count)
 template <typename R> void launch_materialize(const Params<R> &p, int species, cudaStream_t s);
 // loaded cells at or past ncells become removed particles; kStBadCell latched
 void launch_check_cells(int32_t *cell, int64_t n, int64_t ncells, unsigned *status, cudaStream_t s);
-template <typename R> void launch_worklist(const Params<R> &p, const SortScratch *ss,
-                                           const WorkList &wl, int species, int first,
-                                           cudaStream_t s);
+// the work list of the tiled push from the tile bounds of all species
+template <typename R> void launch_worklist(const Params<R> &p, const SortScratch &ss, const WorkList &wl, cudaStream_t s);
 
 }  // namespace hff
