@@ -18,6 +18,7 @@
 #include <type_traits>
 
 #include "collect.cuh"
+#include "fastmath.cuh"
 #include "hff_common.cuh"
 
 namespace hff {
@@ -110,45 +111,6 @@ __device__ __forceinline__ F2 operator-(F2 a, F2 b) { return {__ffma2_rn(b.v, ma
 __device__ __forceinline__ F2 vfma(float w, F2 a, F2 b) { return {__ffma2_rn(make_float2(w, w), a.v, b.v)}; }
 __device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
-
-// FP32 reciprocal and reciprocal square root as the single approximate
-// hardware instructions (about 1-2 ulp, denormals flushed): their arguments
-// here are squared norms, radii and ratios of per-step increments, never
-// denormal, and the results enter quantities compared with the FP64 oracle at
-// 1e-5 relative.  FP64 ones from the hardware's approximations (better than
-// 2^-18) by one step of third order: with e = 1 - x y the reciprocal is
-// y / (1 - e) = y (1 + e + e^2 + O(e^3)); with e = 1 - x y^2 the reciprocal
-// square root is y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2 / 8 + O(e^3)); the
-// remainders are below 2^-54.  Three and five FP64 operations instead of the
-// eight to ten of the library's (correctly rounded or nearly so): the FP64
-// push is bound by the FP64 pipe, two operations per clock and SM.  Arguments
-// near the ends of the range go to the library.
-__device__ __forceinline__ float rsq(float x) {
-  float y;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ float rcp(float x) {
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ unsigned exponent_field(double x) { return ((unsigned)__double2hiint(x) >> 20) & 0x7ffu; }
-__device__ __forceinline__ bool mid_range(double x) { return exponent_field(x) - 32u < 2047u - 64u; }
-__device__ __forceinline__ double rsq(double x) {
-  if (!mid_range(x)) return rsqrt(x);
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-(x * y), y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
-}
-__device__ __forceinline__ double rcp(double x) {
-  if (!mid_range(x)) return 1.0 / x;
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);
-}
 
 // Comparisons of doubles on the integer pipe (a comparison costs the FP64
 // pipe as much as an addition): x >= c for a positive constant c whose lower
