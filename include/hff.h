@@ -188,17 +188,18 @@ typedef struct hff_config {
                                pass over theta strips and row segments after
                                the push, which computes J_perp itself and reads
                                E and dB once (it needs a halo snapshot of E and
-                               dB, about 14% of their size on a 4096^2 grid);
+                               dB, about 6% of their size on a 4096^2 grid);
                                HFF_FIELDS_SPLIT = J_perp at the nodes before
                                the push, then four kernels after it (Faraday
                                half step, Ampere, renormalisation and return,
                                Faraday half step with the absorber), each over
                                every row at once; HFF_FIELDS_AUTO (0) = fused
-                               when segments of 32 rows give at least one wave
-                               of its blocks on a GB300 (six per SM in FP32,
-                               three in FP64, on 152 SMs), else split: on
-                               smaller grids the fused pass's row chains run
-                               on too few blocks                               */
+                               in FP32 on grids of at least 500 areas of 32
+                               rows by 120 columns (about 1340^2), else split:
+                               on smaller grids the fused pass's row chains
+                               run on too few warps, and in FP64 its halos,
+                               computed twice, cost more than the traffic that
+                               it saves                                       */
 } hff_config;
 
 typedef struct hff_info {

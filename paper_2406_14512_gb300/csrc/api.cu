@@ -153,19 +153,25 @@ int validate(const hff_config *c) {
 }
 
 // The field update of a configuration: HFF_FIELDS_AUTO takes the fused pass
-// when segments of 32 rows give at least one wave of its blocks (six per SM
-// in FP32, three in FP64, on the 152 SMs of a GB300: a property of the grid,
-// so that hff_plan needs no GPU); on smaller grids its row chains run on too
-// few blocks and the separate passes, each over every row at once, are
-// faster (1024^2: 1.92 against 2.00 ms per step; a 32-instance ensemble of
-// grids up to 1024 x 512: 2.01 against 2.31 ms).
+// in FP32 on grids of at least 500 areas of 32 rows by 120 columns (about
+// 1340^2; a property of the grid, so that hff_plan needs no GPU).  On smaller
+// grids its row chains run on too few warps and the separate passes, each
+// over every row at once, are faster; in FP64 they always are, because both
+// are bound by the FP64 pipe and the fused pass computes its halos twice.
+// A step of the fields alone, fused against separate: FP32 115 / 80 us at
+// 1024^2, 134 / 168 at 1448^2, 232 / 321 at 2048^2, 756 / 1203 at 4096^2;
+// FP64 0.71 / 0.54 ms at 1024^2, 2.2 / 2.0 at 2048^2, 10.1 / 8.0 at 4096^2.
 static bool fused_fields(const hff_config &c) {
   if (c.field_pass != HFF_FIELDS_AUTO) return c.field_pass == HFF_FIELDS_FUSED;
   if (c.ff_delta_only == 2) return false;  // the stellar-row return exists in the separate passes only
-  const bool fp64 = c.precision == HFF_FP64;
-  const int own = fuse_own_cols(fp64 ? sizeof(double) : sizeof(float));
-  const int64_t strips = (c.nt + 1 + own - 1) / own, segs = (c.nr + 1 + 31) / 32;
-  return strips * segs >= 152 * (fp64 ? 3 : 6);
+  if (c.precision == HFF_FP64) return false;
+  const int64_t strips = (c.nt + 1 + 119) / 120, segs = (c.nr + 1 + 31) / 32;
+  return strips * segs >= 500;
+}
+
+// whether the theta filter's weight is nonzero in the run's precision
+static bool filtered(const hff_config &c) {
+  return c.precision == HFF_FP64 ? c.ff_filter / 16.0 != 0.0 : (float)(c.ff_filter / 16.0) != 0.0f;
 }
 
 // ----------------------------------------------------------- memory layout
@@ -284,12 +290,10 @@ void layout(const hff_config &c, Offsets &o) {
   o.qnode = L.take(nn * 8);
   o.rows = L.take((nr + 1) * 8 * 8);
   o.psi64 = L.take(nn * 8);
-  // the fused field update's snapshot is sized for its shortest segments:
-  // one wave of up to eight blocks on each of the 152 SMs of a GB300 (a
-  // property of the grid, not of the device, so that hff_plan needs no GPU);
-  // hff_init lengthens them to the measured occupancy
-  o.seg_rows = fuse_seg_rows(c.nr, c.nt, 152 * 8, R);
-  o.fsnap = fused_fields(c) ? L.take(fuse_snap_bytes(c.nr, c.nt, o.seg_rows, R)) : 0;
+  // segments of the fused field update: one wave of its blocks on the 152 SMs
+  // of a GB300 (a property of the grid, so that hff_plan needs no GPU)
+  o.seg_rows = fuse_seg_rows(c.nr, c.nt, 152 * kFuseBlocksPerSm, R, filtered(c));
+  o.fsnap = fused_fields(c) ? L.take(fuse_snap_bytes(c.nr, c.nt, o.seg_rows, R, filtered(c))) : 0;
   o.total = (L.off + 255) & ~size_t(255);
 }
 
@@ -307,7 +311,6 @@ struct hff_handle {
   double dt = 0, psi_unit = 0, xi_abs = 0;
   int halo = 0, push_grid = 0, tail_grid = 0;
   bool fused = false;  // the field update runs as the fused pass (fused_fields)
-  int seg_rows = 0;    // rows per segment of the fused field update (>= o.seg_rows)
   Params<float> pf[2];
   Params<double> pd[2];
   WorkList wl{};
@@ -658,8 +661,8 @@ int enqueue_step(hff_handle *h, int par, int stages, cudaStream_t s, int parts =
   const bool fused = h->fused && (stages & kFieldStages) == kFieldStages;
   if ((parts & 1) && (stages & HFF_ST_NODE)) {
     launch_psi<R>(p, s);
-    if (fused) launch_ffcell<R>(p, s);
-    else launch_node_a<R>(p, s);
+    if (!fused) launch_node_a<R>(p, s);
+    else if (h->c.capacity > 0) launch_ffcell<R>(p, s);  // read by the push
   }
   if ((parts & 1) && (stages & HFF_ST_PUSH) && h->c.gamma_th > 0)  // events of this step only
     CK(cudaMemsetAsync(&h->small->pe_count, 0, sizeof(unsigned), s));
@@ -680,11 +683,9 @@ int enqueue_step(hff_handle *h, int par, int stages, cudaStream_t s, int parts =
   }
   if (fused) {
     // the whole field update in one pass; J_PIC cleared for the next deposit
-    launch_field_fused<R>(p, h->seg_rows, h->base + h->o.fsnap, collect, s);
-    const int64_t nr = h->c.nr, nt = h->c.nt;
-    CK(cudaMemsetAsync(p.f.jr, 0, (size_t)(nr * (nt + 1)) * sizeof(R), s));
-    CK(cudaMemsetAsync(p.f.jt, 0, (size_t)((nr + 1) * nt) * sizeof(R), s));
-    CK(cudaMemsetAsync(p.f.jp, 0, (size_t)((nr + 1) * (nt + 1)) * sizeof(R), s));
+    launch_field_fused<R>(p, h->o.seg_rows, h->base + h->o.fsnap, collect, s);
+    // J_r, J_th, J_ph lie one after the other (see layout)
+    CK(cudaMemsetAsync(p.f.jr, 0, (size_t)(h->o.f[12] - h->o.f[9]), s));
   } else {
     if (stages & HFF_ST_FARADAY1) launch_faraday<R>(p, R(0.5), false, collect, s);
     if (stages & HFF_ST_AMPERE) launch_ampere<R>(p, s);
@@ -1168,15 +1169,12 @@ static int init_one(const hff_config *cfg, void *dev_mem, size_t bytes, void *st
     const size_t psm = cfg->precision == HFF_FP64 ? psi_smem<double>(cfg->nt) : psi_smem<float>(cfg->nt);
     const cudaError_t e = cfg->precision == HFF_FP64 ? set_psi_smem<double>(psm) : set_psi_smem<float>(psm);
     if (e != cudaSuccess) return bail(fail(HFF_ERR_CUDA, "cannot set the flux-prefix shared memory size"));
-    const cudaError_t e2 = cfg->precision == HFF_FP64 ? set_field_fused_smem<double>(field_fused_smem<double>())
-                                                      : set_field_fused_smem<float>(field_fused_smem<float>());
+    const cudaError_t e2 = cfg->precision == HFF_FP64
+                               ? set_field_fused_smem<double>(field_fused_smem<double>(h->o.seg_rows))
+                               : set_field_fused_smem<float>(field_fused_smem<float>(h->o.seg_rows));
     if (set_sort_smem() != cudaSuccess) return bail(fail(HFF_ERR_CUDA, "cannot set the sort's shared memory size"));
     if (e2 != cudaSuccess) return bail(fail(HFF_ERR_CUDA, "cannot set the fused field update's shared memory size"));
     h->fused = fused_fields(*cfg);
-    // one wave of the fused field update at its occupancy on this device
-    const int occ = cfg->precision == HFF_FP64 ? field_fused_blocks_per_sm<double>() : field_fused_blocks_per_sm<float>();
-    h->seg_rows = std::max(h->o.seg_rows, fuse_seg_rows(cfg->nr, cfg->nt, std::max(1, occ) * nsm,
-                                                         cfg->precision == HFF_FP64 ? sizeof(double) : sizeof(float)));
   }
   if (cfg->precision == HFF_FP32) {
     fill_params<float>(h);

@@ -422,73 +422,76 @@ __global__ void __launch_bounds__(kRowThreads) k_correct(Params<R> p) {
 // (Eq. 18), Ampere's law with the blended current (Eqs. 19, 28) and the
 // boundaries, the renormalisation at the nodes (Eqs. 25-26), the return to
 // the edges with the blend weights, and Faraday's second half step with the
-// absorber -- as one pass.  A block owns a strip of theta columns (with
-// kFuseHalo columns recomputed on each side) and a segment of rows (with
-// kFuseWarm rows of warm-up below it), and walks the rows upward.  Row step
-// k has four phases separated by barriers:
-//   0: F2, dB^{n+1} at node row k-4 (B_r) and half row k-5 (B_th, B_ph);
-//      node row k and half row k (k+1/2) of E^n, dB^n, B_0, Psi and the
-//      radial tables, loaded one step earlier, go to shared-memory rings,
-//      and the loads of row k+1 are issued (they complete behind phases
-//      1-3);
-//   1: F1, B^{n+1/2} at node row k (B_r) and half row k-1 (B_th, B_ph), and
-//      J_perp at node row k;
-//   2: A, E^{n+1} at half row k-1 (E_r) and node row k-1 (E_th, E_ph), with
-//      the blend weights f kept in registers for phase 3 two steps later;
-//      N, Delta E (or E'') at node row k-2, and the filter terms;
-//   3: C, the corrected E at half row k-3 and node row k-3.
-// Every stage reads only what earlier phases produced, so E^n and dB^n are
-// read once and every output written once; the arithmetic is that of
-// k_node_a, k_faraday, k_ampere, k_node_b and k_correct, location by
-// location.  Column and row ranges: F2 needs the corrected E at columns c,
-// c+1; C (with the theta filter) the uncorrected E at c-2 .. c+2 and Delta E
-// at c, c+1; N and A one column to the left, F1 and J_perp one more on
-// either side, so three columns of halo suffice on each side, and likewise
-// three rows of warm-up (C's radial filter reaches two rows down, A and F1
-// one more each).
+// absorber -- as one pass.  A warp owns a strip of theta columns, one per
+// lane, with a halo recomputed on each side, and a segment of rows (with
+// kFuseWarm rows of warm-up below it), and walks the rows upward.  Everything
+// a column has in flight sits in registers, and what the stencils need of the
+// columns beside it comes by shuffles (16 a row), so warps neither share
+// memory nor wait for each other at every row.  Row step k does
+//   F1  B^{n+1/2} at node row k (B_r) and half row k-1 (B_th, B_ph), and
+//       J_perp at node row k;
+//   A   E^{n+1} at half row k-1 (E_r) and node row k-1 (E_th, E_ph), with the
+//       blend weights f kept for C;
+//   N   Delta E (or E'') at node row k-2;
+//   C   the corrected E at half row k-3 and node row k-3;
+//   F2  dB^{n+1} at node row k-3 (B_r) and half row k-4 (B_th, B_ph);
+// after issuing the copies of row k+2.
+// E^n and dB^n are read once and every output written once; the arithmetic is
+// that of k_node_a, k_faraday, k_ampere, k_node_b and k_correct, location by
+// location.  F2 needs the corrected E at columns c, c+1; C Delta E at c, c+1
+// (and with the theta filter the uncorrected E at c-2 .. c+2); N and A one
+// column to the left, F1 and J_perp one more on either side: two columns of
+// halo on each side, three with the filter, and likewise three or four rows
+// of warm-up.
 //
-// The update is in place, and a block's halo columns and warm-up / trailing
-// rows belong to its neighbours, which overwrite them during the same
-// launch; so a block reads E^n and dB^n live only inside its own area (which
-// no other block writes, and which it overwrites only rows below the one it
-// is reading), and everywhere else from a snapshot of those regions taken
-// just before (k_fuse_prepare).  J_PIC is only read, and
-// the caller clears it after the launch.
-constexpr int kFuseThreads = 128;     // columns of a strip, halo included
-constexpr int kFuseHalo = 4;          // columns recomputed on each side
+// Bound by issue and dependent-instruction latency (640 instructions per warp
+// and row at 4 warps per scheduler, 60% of the issue slots; DRAM at 45%): FP32
+// 0.16 ms at 2048^2 and 0.57 at 4096^2, FP64 1.78 ms at 2048^2 (FP64 pipe).
+// With the rows in shared-memory rings of a 128-thread block, four barriers a
+// row and 1,050 instructions, it took 0.24, 0.81 and 1.96 ms.  10 warps a
+// block at 96 registers: the same at 2048^2, 0.64 ms at 4096^2; blocks of 4 or
+// 5 warps: 0.18 - 0.19 and 0.72 - 0.76 ms, for their snapshot columns.
+//
+// The update is in place.  Within a block, whose warps own neighbouring
+// strips, a barrier every four rows keeps them close enough that the neighbours'
+// copies of a row r are complete (at step r) before its owner overwrites it
+// (from step r+3).  A block's outer halo columns and its warm-up / trailing rows belong
+// to other blocks, which overwrite them during the same launch; those are read
+// from a snapshot of them taken just before (k_fuse_prepare).  J_PIC is only
+// read, and the caller clears it after the launch.
+constexpr int kFuseHalo = 3;          // snapshot columns on each side of a block boundary
 constexpr int kFuseWarm = 4;          // rows recomputed below a segment
-constexpr int kFuseTrail = 5;         // rows above a segment the pipeline loads (up to i_e + 3)
-constexpr int kFuseOwn = kFuseThreads - 2 * kFuseHalo;
+constexpr int kFuseTrail = 4;         // rows above a segment the pipeline reads (up to i_e + 3)
+constexpr int kFuseMaxRows = 384;     // rows of a segment
 constexpr int kFuseArrays = 6;        // E_r E_th E_ph dB_r dB_th dB_ph
-// ring depths: rows live at once (see the phase order above)
-constexpr int kDEn = 2, kDDbr = 1, kDDbn = 2, kDB0r = 3, kDB0h = 4, kDJp = 2, kDPsi = 2, kDBr = 4, kDBh = 4,
-              kDE1r = 5, kDE1n = 3, kDD = 2, kDEc = 2, kDTab = 8;
-constexpr int kFuseRingRows = 3 * kDEn + kDDbr + 2 * kDDbn + kDB0r + 2 * kDB0h + 3 * kDJp + kDBr + 2 * kDBh + kDE1r +
-                              2 * kDE1n + 3 * kDD + 3 * kDEc;
-// radial tables of a row, staged in shared memory by the first threads
+// FP32: 8 warps a block, two blocks per SM at 128 registers; FP64 4 warps
+__host__ __device__ constexpr int fuse_warps(size_t real) { return real == 4 ? 8 : 4; }
+__host__ __device__ constexpr int fuse_halo(bool filt) { return filt ? 3 : 2; }
+// theta columns a block owns
+__host__ __device__ constexpr int fuse_cols(size_t real, bool filt) {
+  return fuse_warps(real) * (32 - 2 * fuse_halo(filt));
+}
+// radial tables of a row, staged in shared memory for the whole segment
 enum FuseTab { TB_RN, TB_INV_RN, TB_C_E2, TB_C_EP2, TB_SIG_N, TB_RHO_A, TB_RHO_B, TB_RH, TB_INV_RH, TB_C_B2,
                TB_C_BP2, TB_SIG_H, TB_RH2, TB_COUNT };
 constexpr int kTabN = 16;
-static_assert(TB_COUNT <= kTabN && TB_COUNT <= kFuseThreads, "table row");
+static_assert(TB_COUNT <= kTabN, "table row");
+// rows of the table of a segment: from five below it (k - 4 of the first
+// step) to its last step
+__host__ __device__ constexpr int fuse_tab_rows(int seg_rows) { return seg_rows + kFuseWarm + kFuseTrail + 8; }
 
-template <typename R>
-size_t fuse_smem_bytes() {
-  return ((size_t)kFuseRingRows * kFuseThreads + (size_t)kDTab * kTabN) * sizeof(R) +
-         (size_t)kDPsi * kFuseThreads * sizeof(typename PsiOf<R>::T) + 16;
-}
-
-// Geometry of a launch: strips of kFuseOwn owned columns, segments of
-// seg_rows owned rows.  Snapshot of E^n and dB^n (six arrays, every array
-// addressed as (nr+1) x (nt+1)): for every strip boundary b = 1 .. strips-1
-// the 2 kFuseHalo columns around column b kFuseOwn over all rows, and for
-// every segment boundary b = 1 .. segs-1 the rows from b seg_rows - kFuseWarm
-// to b seg_rows + kFuseTrail - 1 over all columns.
+// Geometry of a launch: strips of `cols` owned columns, segments of seg_rows
+// owned rows.  Snapshot of E^n and dB^n (six arrays, every array addressed as
+// (nr+1) x (nt+1)): for every strip boundary b = 1 .. strips-1 the 2 kFuseHalo
+// columns around column b cols over all rows, and for every segment boundary
+// b = 1 .. segs-1 the rows from b seg_rows - kFuseWarm to b seg_rows +
+// kFuseTrail - 1 over all columns.
 struct FuseGeom {
   int strips, segs, seg_rows;
 };
-__host__ __device__ inline FuseGeom fuse_geom(int nr, int nt, int seg_rows) {
+__host__ __device__ inline FuseGeom fuse_geom(int nr, int nt, int seg_rows, int cols) {
   FuseGeom g;
-  g.strips = (nt + 1 + kFuseOwn - 1) / kFuseOwn;
+  g.strips = (nt + 1 + cols - 1) / cols;
   g.seg_rows = seg_rows;
   g.segs = (nr + 1 + seg_rows - 1) / seg_rows;
   return g;
@@ -513,26 +516,34 @@ __device__ __forceinline__ const R *fuse_array(const Params<R> &p, int a, int &l
   }
 }
 
-// The snapshot in one launch: the first `nc` blocks copy halo columns (one
-// array of one boundary over kSnapThreads / (2 kFuseHalo) rows each), the next
-// `nw` blocks copy warm-up / trailing rows (kSnapThreads columns of one row of
-// one array of one boundary each), and the rest collect the push's current.
+// The snapshot in one launch: the first `nc` blocks copy halo columns (those
+// of one boundary over kSnapRows rows each), the next `nw` blocks copy warm-up
+// / trailing rows (kSnapThreads columns of one row of one boundary each), and
+// the rest collect the push's current.  A thread copies its element of all six
+// arrays, loads first: bound by latency, 8.9 us at 2048^2 without a collection
+// (18.4 with an array per thread).
 constexpr int kSnapThreads = kCollectThreads;
 constexpr int kSnapRows = kSnapThreads / (2 * kFuseHalo);
 template <typename R>
 __global__ void __launch_bounds__(kSnapThreads) k_fuse_prepare(const __grid_constant__ Params<R> p, R *snap_c,
-                                                               R *snap_r, int seg_rows, int nc, int nw) {
+                                                               R *snap_r, int seg_rows, int own_cols, int nc, int nw) {
   int blk = blockIdx.x;
   int ld, rows, cols;
   if (blk < nc) {
     const int per = (p.nr + kSnapRows) / kSnapRows, ba = blk / per;
-    const int cc = threadIdx.x % (2 * kFuseHalo), row = (blk - ba * per) * kSnapRows + threadIdx.x / (2 * kFuseHalo);
-    if (row > p.nr) return;
-    const int a = ba % kFuseArrays, b = ba / kFuseArrays + 1;
-    const int col = b * kFuseOwn - kFuseHalo + cc;
-    const R *src = fuse_array(p, a, ld, rows, cols);
-    const R v = (row < rows && col >= 0 && col < cols) ? src[(int64_t)row * ld + col] : R(0);
-    snap_c[((int64_t)ba * (p.nr + 1) + row) * (2 * kFuseHalo) + cc] = v;
+    const int rr = threadIdx.x / (2 * kFuseHalo), cc = threadIdx.x - rr * (2 * kFuseHalo);
+    const int row = (blk - ba * per) * kSnapRows + rr;
+    if (row > p.nr || rr >= kSnapRows) return;
+    const int col = (ba + 1) * own_cols - kFuseHalo + cc;
+    R v[kFuseArrays];
+#pragma unroll
+    for (int a = 0; a < kFuseArrays; ++a) {
+      const R *src = fuse_array(p, a, ld, rows, cols);
+      v[a] = (row < rows && col >= 0 && col < cols) ? src[(int64_t)row * ld + col] : R(0);
+    }
+#pragma unroll
+    for (int a = 0; a < kFuseArrays; ++a)
+      snap_c[((int64_t)(ba * kFuseArrays + a) * (p.nr + 1) + row) * (2 * kFuseHalo) + cc] = v[a];
     return;
   }
   blk -= nc;
@@ -541,11 +552,16 @@ __global__ void __launch_bounds__(kSnapThreads) k_fuse_prepare(const __grid_cons
     const int col = (blk - w * per) * kSnapThreads + threadIdx.x;
     if (col > p.nt) return;
     const int rr = w % (kFuseWarm + kFuseTrail), ba = w / (kFuseWarm + kFuseTrail);
-    const int a = ba % kFuseArrays, b = ba / kFuseArrays + 1;
-    const int row = b * seg_rows - kFuseWarm + rr;
-    const R *src = fuse_array(p, a, ld, rows, cols);
-    const R v = (row >= 0 && row < rows && col < cols) ? src[(int64_t)row * ld + col] : R(0);
-    snap_r[(int64_t)w * (p.nt + 1) + col] = v;
+    const int row = (ba + 1) * seg_rows - kFuseWarm + rr;
+    R v[kFuseArrays];
+#pragma unroll
+    for (int a = 0; a < kFuseArrays; ++a) {
+      const R *src = fuse_array(p, a, ld, rows, cols);
+      v[a] = (row >= 0 && row < rows && col < cols) ? src[(int64_t)row * ld + col] : R(0);
+    }
+#pragma unroll
+    for (int a = 0; a < kFuseArrays; ++a)
+      snap_r[((int64_t)(ba * kFuseArrays + a) * (kFuseWarm + kFuseTrail) + rr) * (p.nt + 1) + col] = v[a];
     return;
   }
   blk -= nw;
@@ -553,451 +569,442 @@ __global__ void __launch_bounds__(kSnapThreads) k_fuse_prepare(const __grid_cons
   collect_block(p, blk % cx, blk / cx);
 }
 
-// a ring of rows in shared memory, one element per column of the strip
-template <typename T, int D>
-struct FRing {
-  T *p;
-  __device__ __forceinline__ T &operator()(int row, int c) const {
-    return p[((unsigned)row % (unsigned)D) * kFuseThreads + c];
-  }
+// a value of the column to the right / left
+template <typename T> __device__ __forceinline__ T right(T v) { return __shfl_down_sync(0xffffffffu, v, 1); }
+template <typename T> __device__ __forceinline__ T left(T v) { return __shfl_up_sync(0xffffffffu, v, 1); }
+__device__ __forceinline__ float2 right(float2 v) { return make_float2(right(v.x), right(v.y)); }
+
+// What a row step reads, staged in shared memory by its own lane: E^n, dB^n,
+// B_0 of the row (half rows: the half row above the node row), J_PIC and
+// curl B_0 at the E locations of the row below, Psi of the row.
+enum FuseInput { IN_ER, IN_ET, IN_EP, IN_BR, IN_BT, IN_BP, IN_B0R, IN_B0T, IN_B0P, IN_JR, IN_SR, IN_JT, IN_ST, IN_JP,
+               IN_SP, IN_COUNT };
+constexpr int kFuseStages = 4;        // rows staged: the two in use and two in flight
+template <typename R> __host__ __device__ constexpr size_t fuse_stage_bytes() {
+  return 32 * (IN_COUNT * sizeof(R) + 8);
+}
+
+// whether a step's rows (a warp's columns) are known to be interior
+template <bool ROWS, bool COLS>
+struct FuseTag {
+  static constexpr bool rows = ROWS, cols = COLS;
 };
 
-// node row k and half row k of one column, in flight between phase 0 of
-// step k-1 and phase 0 of step k
-template <typename R>
-struct FuseRow {
-  R er, et, ep, br, bt, bp, b0r, b0t, b0p, tab;
-  typename PsiOf<R>::T psi;
-};
-// J_PIC and curl B_0 of one column at the E locations of row k (half row
-// for E_r, node row for E_th and E_ph), used by phase 2 of step k+1
-template <typename R>
-struct FuseSrc {
-  R jr, sr, jt, st, jp, sp;
-};
-
-template <typename R>
-__global__ void __launch_bounds__(kFuseThreads) k_field_fused(Params<R> p, R hdt, FuseGeom fg, const R *snap_c,
-                                                              const R *snap_r) {
+template <typename R, bool FILT>
+__global__ void __launch_bounds__(32 * fuse_warps(sizeof(R)), sizeof(R) == 4 ? 2 : 1)
+    k_field_fused(const __grid_constant__ Params<R> p, R hdt, FuseGeom fg, const R *snap_c, const R *snap_r) {
   using P = typename PsiOf<R>::T;
-  constexpr int NC = kFuseThreads, H = kFuseHalo, W = kFuseWarm;
+  constexpr int H = fuse_halo(FILT), OWN = 32 - 2 * H, COLS = fuse_warps(sizeof(R)) * OWN, W = kFuseWarm;
   extern __shared__ __align__(16) unsigned char fsmem[];
+  R *tab = reinterpret_cast<R *>(fsmem);
   const int nr = p.nr, nt = p.nt, n1 = nt + 1, seg_rows = fg.seg_rows;
-  const int c = threadIdx.x, sx = blockIdx.x, sy = blockIdx.y;
-  const int j = sx * kFuseOwn - H + c;                                 // global column of this thread
-  const bool jn = j >= 0 && j <= nt, jh = j >= 0 && j < nt;           // node / half column exists
-  const bool own = c >= H && c < NC - H;                              // column written by this block
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sx = blockIdx.x, sy = blockIdx.y;
+  const int j = sx * COLS + warp * OWN - H + lane;                     // global column of this lane
+  const bool jn_ = j >= 0 && j <= nt, jh_ = j >= 0 && j < nt;         // node / half column exists
+  const bool own = lane >= H && lane < 32 - H && jn_;                 // column written by this lane
+  const unsigned ju = jn_ ? j : 0;
+  const bool mine = j >= sx * COLS && j < (sx + 1) * COLS;            // column of this block
+  const int j0 = j - lane;                                            // first column of this warp
+  const bool cin = j0 >= 2 && j0 + 31 <= nt - 3;                      // all columns away from the axis
+  const bool live = __all_sync(0xffffffffu, mine);                    // all columns of this block
   const int i_s = sy * seg_rows;                                      // first output row
   if (i_s > nr) return;
   const int i_e = min(i_s + seg_rows, nr + 1);                        // one past the last output node row
-  const int k0 = max(0, i_s - W), kl = min(nr, i_e) + 3;              // row steps with phases 1-3
+  const int k0 = max(0, i_s - W), kl = min(nr, i_e) + 3;              // row steps
   const Fields<R> &f = p.f;
   const Tables<R> &t = p.t;
-  // snapshot offset of a halo column (array 0, row 0); unused where the
-  // column is outside the grid (the first strip's left and the last
-  // strip's right halo)
-  int64_t sc0 = 0;
-  if (!own) {
-    const int b = (c < H) ? sx : sx + 1;
-    sc0 = (int64_t)(b - 1) * kFuseArrays * (nr + 1) * (2 * H) + (j - (b * kFuseOwn - H));
+  const int t0 = k0 - 4;                                              // first row of the staged table
+  {
+    const R *src[TB_COUNT] = {t.rn, t.inv_rn, t.c_e2, t.c_ep2, t.sig_n, t.rho_a, t.rho_b, t.rh, t.inv_rh, t.c_b2,
+                              t.c_bp2, t.sig_h, t.rh2};
+    for (int w = 0; w < TB_COUNT; ++w) {
+      const int last = w < TB_RH ? nr : nr - 1;
+      for (int r = threadIdx.x; r <= kl - t0; r += blockDim.x) {
+        const int row = t0 + r;
+        tab[r * kTabN + w] = (row >= 0 && row <= last) ? src[w][row] : R(0);
+      }
+    }
   }
-  // the radial table this thread stages (threads 0 .. TB_COUNT-1)
-  const R *tp = nullptr;
-  int tlim = -1;
-  switch (c) {
-    case TB_RN: tp = t.rn; tlim = nr; break;
-    case TB_INV_RN: tp = t.inv_rn; tlim = nr; break;
-    case TB_C_E2: tp = t.c_e2; tlim = nr; break;
-    case TB_C_EP2: tp = t.c_ep2; tlim = nr; break;
-    case TB_SIG_N: tp = t.sig_n; tlim = nr; break;
-    case TB_RHO_A: tp = t.rho_a; tlim = nr; break;
-    case TB_RHO_B: tp = t.rho_b; tlim = nr; break;
-    case TB_RH: tp = t.rh; tlim = nr - 1; break;
-    case TB_INV_RH: tp = t.inv_rh; tlim = nr - 1; break;
-    case TB_C_B2: tp = t.c_b2; tlim = nr - 1; break;
-    case TB_C_BP2: tp = t.c_bp2; tlim = nr - 1; break;
-    case TB_SIG_H: tp = t.sig_h; tlim = nr - 1; break;
-    case TB_RH2: tp = t.rh2; tlim = nr - 1; break;
-    default: break;
-  }
-  // Row steps come in two versions: interior steps, whose rows k-5 .. k+1
-  // all lie inside this block's own rows and inside rows 2 .. nr-3 (every
-  // row condition below holds), and the general one.  IN is true in the
-  // former, where the compiler drops the row conditions.
-  //
+  __syncthreads();
+  auto T = [&](int row, int w) -> R { return tab[(row - t0) * kTabN + w]; };
   // E^n and dB^n of node row k and half row k: live inside this block's own
-  // area, from the snapshot in the halo columns and the warm-up / trailing
-  // rows; then B_0, Psi and the radial table of the row
-  auto fetch = [&](int k, FuseRow<R> &x, auto tag) {
-    constexpr bool IN = decltype(tag)::value;
+  // area, from the snapshot in its outer halo columns and its warm-up /
+  // trailing rows; then B_0 and Psi.  Steps come in versions for rows (and
+  // columns) known to be in the grid's interior, where every condition on the
+  // row (column) holds and the compiler drops it.
+  int64_t sc0 = 0;
+  if (!mine) {   // unused where the column is outside the grid
+    const int b = (j < sx * COLS) ? sx : sx + 1;
+    sc0 = (int64_t)(b - 1) * kFuseArrays * (nr + 1) * (2 * kFuseHalo) + (j - (b * COLS - kFuseHalo));
+  }
+  auto fetch = [&](int k, unsigned char *st, auto tag) {
+    constexpr bool IN = decltype(tag)::rows, CI = decltype(tag)::cols, ALL = IN && CI;
+    const bool jn = CI || jn_, jh = CI || jh_;
     const bool node = IN || k <= nr, half = IN || k < nr;
+    const int64_t kn = (int64_t)k * n1, kh = (int64_t)k * nt;
+    R *d = reinterpret_cast<R *>(st) + lane;
+    auto get = [&](int a, const R *src, bool ok) {
+      if constexpr (ALL) copy_async<sizeof(R)>(d + a * 32, src);
+      else copy_async<sizeof(R)>(d + a * 32, ok ? src : f.ep, ok);
+    };
     const bool cer = half && jn, cet = node && jh, cep = node && jn, cbr = node && jh, cbt = half && jn,
                cbp = half && jh;
-    const int64_t kn = (int64_t)k * n1 + j, kh = (int64_t)k * nt + j;
-    if (own && (IN || (k >= i_s && k < i_e))) {
-      x.er = cer ? f.er[kn] : R(0);
-      x.et = cet ? f.et[kh] : R(0);
-      x.ep = cep ? f.ep[kn] : R(0);
-      x.br = cbr ? f.br[kh] : R(0);
-      x.bt = cbt ? f.bt[kn] : R(0);
-      x.bp = cbp ? f.bp[kh] : R(0);
+    if ((live || mine) && k >= i_s && k < i_e) {
+      get(IN_ER, f.er + kn + ju, cer);
+      get(IN_ET, f.et + kh + ju, cet);
+      get(IN_EP, f.ep + kn + ju, cep);
+      get(IN_BR, f.br + kh + ju, cbr);
+      get(IN_BT, f.bt + kn + ju, cbt);
+      get(IN_BP, f.bp + kh + ju, cbp);
     } else {
       // array a of the snapshot at s + a as (see k_fuse_prepare)
       const R *s;
       int64_t as;
-      if (own) {
+      if (mine) {
         const int b = (k < i_s) ? sy : sy + 1;
-        s = snap_r + ((int64_t)(b - 1) * kFuseArrays * (W + kFuseTrail) + (k - (b * seg_rows - W))) * n1 + j;
+        s = snap_r + ((int64_t)(b - 1) * kFuseArrays * (W + kFuseTrail) + (k - (b * seg_rows - W))) * n1 + ju;
         as = (int64_t)(W + kFuseTrail) * n1;
       } else {
-        s = snap_c + sc0 + (int64_t)k * (2 * H);
-        as = (int64_t)(nr + 1) * (2 * H);
+        s = snap_c + sc0 + (int64_t)k * (2 * kFuseHalo);
+        as = (int64_t)(nr + 1) * (2 * kFuseHalo);
       }
-      x.er = cer ? s[0] : R(0);
-      x.et = cet ? s[as] : R(0);
-      x.ep = cep ? s[2 * as] : R(0);
-      x.br = cbr ? s[3 * as] : R(0);
-      x.bt = cbt ? s[4 * as] : R(0);
-      x.bp = cbp ? s[5 * as] : R(0);
+      get(IN_ER, s, cer);
+      get(IN_ET, s + as, cet);
+      get(IN_EP, s + 2 * as, cep);
+      get(IN_BR, s + 3 * as, cbr);
+      get(IN_BT, s + 4 * as, cbt);
+      get(IN_BP, s + 5 * as, cbp);
     }
-    x.b0r = cbr ? __ldg(f.br0 + kh) : R(0);
-    x.b0t = cbt ? __ldg(f.bt0 + kn) : R(0);
-    x.b0p = cbp ? __ldg(f.bp0 + kh) : R(0);
-    x.psi = cep ? __ldg(f.psi + kn) : P{};
-    x.tab = (k <= tlim) ? __ldg(tp + k) : R(0);
+    get(IN_B0R, f.br0 + kh + ju, cbr);
+    get(IN_B0T, f.bt0 + kn + ju, cbt);
+    get(IN_B0P, f.bp0 + kh + ju, cbp);
+    {
+      const bool up = IN || k >= 1, node1 = up && (IN || k - 1 <= nr), half1 = up && (IN || k - 1 < nr);
+      const int64_t ln = kn - n1, lh = kh - nt;
+      get(IN_JR, f.jr + ln + ju, half1 && jn);
+      get(IN_SR, f.sr + ln + ju, half1 && jn);
+      get(IN_JT, f.jt + lh + ju, node1 && jh);
+      get(IN_ST, f.st + lh + ju, node1 && jh);
+      get(IN_JP, f.jp + ln + ju, node1 && jn);
+      get(IN_SP, f.sp + ln + ju, node1 && jn);
+    }
+    unsigned char *ps = st + 32 * IN_COUNT * sizeof(R) + lane * sizeof(P);
+    const P *psi = f.psi + kn + ju;
+    if constexpr (ALL) copy_async<sizeof(P)>(ps, psi);
+    else copy_async<sizeof(P)>(ps, cep ? psi : f.psi, cep);
   };
-  auto fetch_src = [&](int k, FuseSrc<R> &y, auto tag) {
-    constexpr bool IN = decltype(tag)::value;
-    const bool node = IN || k <= nr, half = IN || k < nr;
-    const int64_t kn = (int64_t)k * n1 + j, kh = (int64_t)k * nt + j;
-    y.jr = (half && jn) ? __ldg(f.jr + kn) : R(0);
-    y.sr = (half && jn) ? __ldg(f.sr + kn) : R(0);
-    y.jt = (node && jh) ? __ldg(f.jt + kh) : R(0);
-    y.st = (node && jh) ? __ldg(f.st + kh) : R(0);
-    y.jp = (node && jn) ? __ldg(f.jp + kn) : R(0);
-    y.sp = (node && jn) ? __ldg(f.sp + kn) : R(0);
-  };
-  // carve the rings
-  FRing<R, kDEn> en_r, en_t, en_p;      // E^n            (half, node, node)
-  FRing<R, kDDbr> dbr;                  // dB_r^n         (node)
-  FRing<R, kDDbn> dbn_t, dbn_p;         // dB_th^n, dB_ph^n (half)
-  FRing<R, kDB0r> b0_r;                 // B_0,r          (node)
-  FRing<R, kDB0h> b0_t, b0_p;           // B_0,th, B_0,ph (half)
-  FRing<R, kDJp> jp_r, jp_t, jp_p;      // J_perp         (node)
-  FRing<R, kDBr> bh_r;                  // dB_r^{n+1/2}   (node)
-  FRing<R, kDBh> bh_t, bh_p;            // dB^{n+1/2}     (half)
-  FRing<R, kDE1r> e1_r;                 // E^{n+1} before the correction (half)
-  FRing<R, kDE1n> e1_t, e1_p;           //                                (node)
-  FRing<R, kDD> d_r, d_t, d_p;          // Delta E or E'' (node)
-  FRing<R, kDEc> ec_r, ec_t, ec_p;      // corrected E    (half, node, node)
-  FRing<P, kDPsi> psi;                  // Psi            (node)
-  R *tab;                               // radial tables, kDTab rows of kTabN
-  {
-    R *q = reinterpret_cast<R *>(fsmem);
-    auto take = [&](int rows) { R *r = q; q += rows * NC; return r; };
-    en_r.p = take(kDEn); en_t.p = take(kDEn); en_p.p = take(kDEn);
-    dbr.p = take(kDDbr); dbn_t.p = take(kDDbn); dbn_p.p = take(kDDbn);
-    b0_r.p = take(kDB0r); b0_t.p = take(kDB0h); b0_p.p = take(kDB0h);
-    jp_r.p = take(kDJp); jp_t.p = take(kDJp); jp_p.p = take(kDJp);
-    bh_r.p = take(kDBr); bh_t.p = take(kDBh); bh_p.p = take(kDBh);
-    e1_r.p = take(kDE1r); e1_t.p = take(kDE1n); e1_p.p = take(kDE1n);
-    d_r.p = take(kDD); d_t.p = take(kDD); d_p.p = take(kDD);
-    ec_r.p = take(kDEc); ec_t.p = take(kDEc); ec_p.p = take(kDEc);
-    tab = q;
-    q += kDTab * kTabN;
-    uintptr_t a = reinterpret_cast<uintptr_t>(q);
-    a = (a + 15) & ~uintptr_t(15);
-    psi.p = reinterpret_cast<P *>(a);
-  }
-  auto T = [&](int row, int w) -> R { return tab[((unsigned)row % (unsigned)kDTab) * kTabN + w]; };
+  auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
   // theta tables of this column
-  const R sn0 = jn ? t.sn[j] : R(0), sn1 = jh ? t.sn[j + 1] : R(0), idcp = jh ? t.inv_dcp[j] : R(0);
-  const R sh0 = jh ? t.sh[j] : R(0), shm = (j >= 1 && j <= nt) ? t.sh[j - 1] : R(0);
-  const R idch = jn ? t.inv_dch[j] : R(0);
+  const R sn0 = jn_ ? t.sn[j] : R(0), sn1 = jh_ ? t.sn[j + 1] : R(0), idcp = jh_ ? t.inv_dcp[j] : R(0);
+  const R sh0 = jh_ ? t.sh[j] : R(0), shm = (j >= 1 && j <= nt) ? t.sh[j - 1] : R(0);
+  const R idch = jn_ ? t.inv_dch[j] : R(0);
   const R dt = p.dt, fp4 = R(4.0 * kPi) * p.dt;
-  const bool lit = p.ff_interp_e == 1, filt = p.ff_sigma16 != R(0);
-  const bool axis = (j == 0 || j == nt);
-  unsigned long long nclamp = 0;
-  // blend weights of rows k-1, k-2, k-3 (E_r edge, E_th edge, node)
-  R fr1 = 0, fr2 = 0, fr3 = 0, ft1 = 0, ft2 = 0, ft3 = 0, fn1 = 0, fn2 = 0, fn3 = 0;
-  FuseRow<R> nx{};
-  FuseSrc<R> js{}, jsn{};
-  // F2: dB^{n+1} at node row k-4 and half row k-5 (own columns and rows)
-  auto f2 = [&](int k, auto tag) {
-    constexpr bool IN = decltype(tag)::value;
-    if (!own) return;
-    const int i = k - 4;  // B_r(i, j+1/2)
-    if ((IN || (i >= i_s && i < i_e)) && jh) {
-      const R cu = T(i, TB_INV_RN) * (sn1 * ec_p(i, c + 1) - sn0 * ec_p(i, c)) * idcp;
-      R v = bh_r(i, c) - hdt * cu;
-      const R sg = T(i, TB_SIG_N);
-      if (sg > R(0)) v -= sg * v;
-      f.br[(int64_t)i * nt + j] = v;
+  const bool lit = p.ff_interp_e == 1;
+  unsigned nclamp = 0;
+  // The blend weights are uniform where every Psi of the warp's two rows lies
+  // on one side of all breakpoints by more than the rounding of a mean: the
+  // usual case, and a mean in pairs with its search costs 35 instructions a
+  // weight.
+  R psi_lo = R(0), psi_hi = R(0), f_lo = R(0), f_hi = R(0);
+  if (p.n_breaks > 0) {   // else f = 0 everywhere
+    const R eps = R(1e-6), tiny = R(1e-30);
+    psi_lo = psi_lead(p.psi_bk[0]);
+    psi_lo -= eps * fabs(psi_lo) + tiny;
+    f_lo = p.f_break[0];
+    psi_hi = psi_lo;
+    for (int q = 0; q < p.n_breaks; ++q) {
+      const R b = psi_lead(p.psi_bk[q]);
+      psi_hi = max(psi_hi, b + (eps * fabs(b) + tiny));
     }
-    const int h = k - 5;  // B_th(h+1/2, j), B_ph(h+1/2, j+1/2)
-    if (IN || (h >= i_s && h < i_e && h < nr)) {
-      const R sg = T(h, TB_SIG_H), cb2 = T(h, TB_C_B2), rn0 = T(h, TB_RN), rn1 = T(h + 1, TB_RN);
-      if (jn) {
-        R v = R(0);
-        if (j > 0 && j < nt) {
-          v = bh_t(h, c) + hdt * cb2 * (rn1 * ec_p(h + 1, c) - rn0 * ec_p(h, c));
-          if (sg > R(0)) v -= sg * v;
-        }
-        f.bt[(int64_t)h * n1 + j] = v;
-      }
-      if (jh) {
-        const R cu = cb2 * (rn1 * ec_t(h + 1, c) - rn0 * ec_t(h, c)) - T(h, TB_C_BP2) * (ec_r(h, c + 1) - ec_r(h, c));
-        R w = bh_p(h, c) - hdt * cu;
-        if (sg > R(0)) w -= sg * w;
-        f.bp[(int64_t)h * nt + j] = w;
-      }
-    }
-  };
-  auto step = [&](int k, auto tag) {
-    constexpr bool IN = decltype(tag)::value;
-    // ------------------------------------------------------------ phase 0
-    f2(k, tag);
-    en_r(k, c) = nx.er; en_t(k, c) = nx.et; en_p(k, c) = nx.ep;
-    dbr(k, c) = nx.br; dbn_t(k, c) = nx.bt; dbn_p(k, c) = nx.bp;
-    b0_r(k, c) = nx.b0r; b0_t(k, c) = nx.b0t; b0_p(k, c) = nx.b0p;
-    psi(k, c) = nx.psi;
-    if (c < TB_COUNT) tab[((unsigned)k % (unsigned)kDTab) * kTabN + c] = nx.tab;
-    js = jsn;
-    fetch_src(k, jsn, tag);
-    if (IN || k + 1 <= kl) fetch(k + 1, nx, tag);
-    __syncthreads();
-    // ------------------------------------------------------------ phase 1
-    if (IN || k <= nr) {
-      // B_r(k, j+1/2)
-      R v = dbr(k, c);
-      if (jh && c < NC - 1) v -= hdt * (T(k, TB_INV_RN) * (sn1 * en_p(k, c + 1) - sn0 * en_p(k, c)) * idcp);
-      bh_r(k, c) = v;
-      // J_perp(k, j) = rho E x B / B^2 from E^n, B^n
-      R jx = 0, jy = 0, jz = 0;
-      if ((IN || (k >= 1 && k < nr)) && jn && c >= 1) {
-        R e[3], b[3];
-        e[0] = R(0.5) * (en_r(k - 1, c) + en_r(k, c));
-        e[1] = axis ? R(0) : R(0.5) * (en_t(k, c - 1) + en_t(k, c));
-        e[2] = axis ? R(0) : en_p(k, c);
-        auto br = [&](int dc) { return b0_r(k, c + dc) + dbr(k, c + dc); };
-        auto bt = [&](int row) { return b0_t(row, c) + dbn_t(row, c); };
-        auto bp = [&](int row, int dc) { return b0_p(row, c + dc) + dbn_p(row, c + dc); };
-        b[0] = (j == 0) ? br(0) : (j == nt) ? br(-1) : R(0.5) * (br(-1) + br(0));
-        b[1] = axis ? R(0) : R(0.5) * (bt(k - 1) + bt(k));
-        b[2] = axis ? R(0) : R(0.25) * (bp(k - 1, -1) + bp(k - 1, 0) + bp(k, -1) + bp(k, 0));
-        const R div = T(k, TB_RHO_A) * (T(k, TB_RH2) * en_r(k, c) - T(k - 1, TB_RH2) * en_r(k - 1, c));
-        R dth = 0;
-        if (j < nt) dth += sh0 * en_t(k, c);
-        if (j > 0) dth -= shm * en_t(k, c - 1);
-        const R rho = div + T(k, TB_RHO_B) * dth * idch;
-        const R b2 = b[0] * b[0] + b[1] * b[1] + b[2] * b[2];
-        if (b2 > b2min<R>()) {
-          const R s = rho / b2;
-          jx = s * (e[1] * b[2] - e[2] * b[1]);
-          jy = s * (e[2] * b[0] - e[0] * b[2]);
-          jz = s * (e[0] * b[1] - e[1] * b[0]);
-        }
-      }
-      jp_r(k, c) = jx; jp_t(k, c) = jy; jp_p(k, c) = jz;
-      if (own && jn && (IN || (k >= i_s && k < i_e))) {
-        const int64_t kk = (int64_t)k * n1 + j;
-        f.jpr[kk] = jx; f.jpt[kk] = jy; f.jpp[kk] = jz;
-      }
-    }
-    if (IN || (k >= 1 && k - 1 < nr)) {
-      const int i = k - 1;
-      const R cb2 = T(i, TB_C_B2), rn0 = T(i, TB_RN), rn1 = T(k, TB_RN);
-      R v = R(0);  // B_th(i+1/2, j): zero on the axis
-      if (j > 0 && j < nt) v = dbn_t(i, c) + hdt * cb2 * (rn1 * en_p(k, c) - rn0 * en_p(i, c));
-      bh_t(i, c) = v;
-      if (jh && c < NC - 1) {  // B_ph(i+1/2, j+1/2)
-        const R cu = cb2 * (rn1 * en_t(k, c) - rn0 * en_t(i, c)) - T(i, TB_C_BP2) * (en_r(i, c + 1) - en_r(i, c));
-        bh_p(i, c) = dbn_p(i, c) - hdt * cu;
-      }
-    }
-    __syncthreads();
-    // ------------------------------------------------------------ phase 2
-    fr3 = fr2; fr2 = fr1; ft3 = ft2; ft2 = ft1; fn3 = fn2; fn2 = fn1;
-    fr1 = 0; ft1 = 0; fn1 = 0;
-    if ((IN || (k >= 1 && k - 1 <= nr)) && c >= 1 && c < NC - 1) {  // A at row i = k-1
-      const int i = k - 1;
-      if ((IN || i < nr) && jn) {  // E_r(i+1/2, j)
-        R cu = R(0);
-        if (j < nt) cu += sh0 * bh_p(i, c);
-        if (j > 0) cu -= shm * bh_p(i, c - 1);
-        cu *= T(i, TB_INV_RH) * idch;
-        const R fb = blend(p, psi_mean2(psi(i, c), psi(i + 1, c)));
-        fr1 = fb;
-        const bool lo = IN || i >= 1, hi = IN || i + 1 <= nr - 1;
-        R jm = R(0);
-        if (lo) jm += jp_r(i, c);
-        if (hi) jm += jp_r(i + 1, c);
-        if (lo && hi) jm *= R(0.5);
-        const R jt = (R(1) - fb) * js.jr + fb * jm;
-        e1_r(i, c) = (en_r(i, c) + dt * (cu + js.sr) - fp4 * jt) * (R(1) - T(i, TB_SIG_H));
-      }
-      if (jh) {  // E_th(i, j+1/2)
-        R v;
-        if (!IN && i == 0) {
-          v = -p.omega * T(0, TB_RN) * sh0 * (b0_r(0, c) + bh_r(0, c));
-        } else if (!IN && i == nr) {
-          v = R(0);
-        } else {
-          const R cu = -T(i, TB_C_E2) * (T(i, TB_RH) * bh_p(i, c) - T(i - 1, TB_RH) * bh_p(i - 1, c));
-          const R fb = blend(p, psi_mean2(psi(i, c), psi(i, c + 1)));
-          ft1 = fb;
-          const R jt = (R(1) - fb) * js.jt + fb * R(0.5) * (jp_t(i, c) + jp_t(i, c + 1));
-          v = (en_t(i, c) + dt * (cu + js.st) - fp4 * jt) * (R(1) - T(i, TB_SIG_N));
-        }
-        e1_t(i, c) = v;
-      }
-      if (jn) {  // E_ph(i, j)
-        R v = R(0);
-        if ((IN || (i >= 1 && i < nr)) && j >= 1 && j < nt) {
-          const R cu = T(i, TB_C_E2) * (T(i, TB_RH) * bh_t(i, c) - T(i - 1, TB_RH) * bh_t(i - 1, c)) -
-                       T(i, TB_C_EP2) * (bh_r(i, c) - bh_r(i, c - 1));
-          const R fb = blend(p, psi(i, c));
-          fn1 = fb;
-          const R jt = (R(1) - fb) * js.jp + fb * jp_p(i, c);
-          v = (en_p(i, c) + dt * (cu + js.sp) - fp4 * jt) * (R(1) - T(i, TB_SIG_N));
-        }
-        e1_p(i, c) = v;
-      }
-    }
-    if ((IN || (k >= 2 && k - 2 <= nr)) && c >= 1) {  // N at node row i = k-2
-      const int i = k - 2;
-      const bool orow = IN || (i >= i_s && i < i_e);
-      R d0 = 0, d1 = 0, d2 = 0;
-      if ((IN || (i >= 1 && i < nr)) && jn) {
-        R e[3], b[3];
-        e[0] = R(0.5) * (e1_r(i - 1, c) + e1_r(i, c));
-        e[1] = axis ? R(0) : R(0.5) * (e1_t(i, c - 1) + e1_t(i, c));
-        e[2] = axis ? R(0) : e1_p(i, c);
-        auto br = [&](int dc) { return b0_r(i, c + dc) + bh_r(i, c + dc); };
-        auto bt = [&](int row) { return b0_t(row, c) + bh_t(row, c); };
-        auto bp = [&](int row, int dc) { return b0_p(row, c + dc) + bh_p(row, c + dc); };
-        b[0] = (j == 0) ? br(0) : (j == nt) ? br(-1) : R(0.5) * (br(-1) + br(0));
-        b[1] = axis ? R(0) : R(0.5) * (bt(i - 1) + bt(i));
-        b[2] = axis ? R(0) : R(0.25) * (bp(i - 1, -1) + bp(i - 1, 0) + bp(i, -1) + bp(i, 0));
-        const R b2 = b[0] * b[0] + b[1] * b[1] + b[2] * b[2];
-        if (b2 > b2min<R>()) {
-          const R sdot = (e[0] * b[0] + e[1] * b[1] + e[2] * b[2]) / b2;
-          const R x = e[0] - sdot * b[0], y = e[1] - sdot * b[1], z = e[2] - sdot * b[2];
-          const R e2 = x * x + y * y + z * z;
-          const R sc = (e2 > b2) ? sqrt(b2 / e2) : R(1);
-          d0 = sc * x - e[0];
-          d1 = sc * y - e[1];
-          d2 = sc * z - e[2];
-          if (e2 > b2 && own && orow) ++nclamp;
-        }
-        if (lit) { d0 += e[0]; d1 += e[1]; d2 += e[2]; }
-      }
-      d_r(i, c) = d0; d_t(i, c) = d1; d_p(i, c) = d2;
-      if (own && jn && orow) {
-        const int64_t kk = (int64_t)i * n1 + j;
-        f.der[kk] = d0; f.det[kk] = d1; f.dep[kk] = d2;
-      }
-    }
-    __syncthreads();
-    // ------------------------------------------------------------ phase 3
-    if ((IN || (k >= 3 && k - 3 <= nr)) && c >= 2 && c < NC - 2) {  // C at row i = k-3
-      const int i = k - 3;
-      const bool out = own && (IN || (i >= i_s && i < i_e));
-      if ((IN || i < nr) && jn) {  // E_r(i+1/2, j)
-        R v = e1_r(i, c);
-        const R fb = fr3;
-        if (fb != R(0)) {
-          const bool lo = IN || i >= 1, hi = IN || i + 1 <= nr - 1;
-          R m = R(0);
-          if (lo) m += d_r(i, c);
-          if (hi) m += d_r(i + 1, c);
-          if (lo && hi) m *= R(0.5);
-          if (filt && (IN || (i >= 2 && i <= nr - 3)))
-            m -= p.ff_sigma16 * (e1_r(i - 2, c) - R(4) * e1_r(i - 1, c) + R(6) * v - R(4) * e1_r(i + 1, c) +
-                                 e1_r(i + 2, c));
-          v += fb * (lit ? m - v : m);
-        }
-        ec_r(i, c) = v;
-        if (out) f.er[(int64_t)i * n1 + j] = v;
-      }
-      if (jh) {  // E_th(i, j+1/2)
-        R v = e1_t(i, c);
-        if (IN || (i >= 1 && i < nr)) {
-          const R fb = ft3;
-          if (fb != R(0)) {
-            R m = R(0.5) * (d_t(i, c) + d_t(i, c + 1));
-            if (filt && j >= 2 && j <= nt - 3)
-              m -= p.ff_sigma16 * (e1_t(i, c - 2) - R(4) * e1_t(i, c - 1) + R(6) * v - R(4) * e1_t(i, c + 1) +
-                                   e1_t(i, c + 2));
-            v += fb * (lit ? m - v : m);
-          }
-        }
-        ec_t(i, c) = v;
-        if (out) f.et[(int64_t)i * nt + j] = v;
-      }
-      if (jn) {  // E_ph(i, j)
-        R v = e1_p(i, c);
-        if ((IN || (i >= 1 && i < nr)) && j >= 1 && j < nt) {
-          const R fb = fn3;
-          if (fb != R(0)) {
-            const R m = d_p(i, c);
-            v += fb * (lit ? m - v : m);
-          }
-        }
-        ec_p(i, c) = v;
-        if (out) f.ep[(int64_t)i * n1 + j] = v;
-      }
-    }
-    __syncthreads();
-  };
-  // interior steps: rows k-5 .. k+1 own (k-5 >= i_s, k+1 < i_e) and inside
-  // rows 2 .. nr-3 (k >= 7, k+4 <= nr)
-  const int kin0 = max(i_s + 5, 7), kin1 = min(i_e - 2, nr - 4);
-  fetch(k0, nx, std::false_type{});
-  for (int k = k0; k <= kl; ++k) {
-    if (k >= kin0 && k <= kin1) step(k, std::true_type{});
-    else step(k, std::false_type{});
+    f_hi = p.f_break[p.n_breaks - 1];
   }
-  f2(kl + 1, std::false_type{});
+  bool lo1 = false, hi1 = false;   // every Psi of row k-1 below / above the breakpoints
+  // the pipeline: suffix = rows behind k at the beginning of a step (half
+  // rows: the half row above that node row)
+  R tbt1 = 0, tbp1 = 0;                                  // B^n: B_th; B_ph, sum of two columns
+  R jr1 = 0, jt1 = 0, jp1 = 0;                           // J_perp of row k-1
+  R br1 = 0, br2 = 0, br3 = 0, ht2 = 0, ht3 = 0, ht4 = 0, hp2 = 0, hp3 = 0, hp4 = 0;   // dB^{n+1/2}
+  R nb1 = 0, nb2 = 0, bb2 = 0, bb3 = 0, pp2 = 0, pp3 = 0;   // B^{n+1/2}: B_r at the node; B_th; B_ph, two columns
+  R fr2 = 0, fr3 = 0, ft2 = 0, ft3 = 0, fn2 = 0, fn3 = 0;   // blend weights
+  R ar2 = 0, ar3 = 0, ar4 = 0, ar5 = 0, at2 = 0, at3 = 0, ap2 = 0, ap3 = 0;   // E^{n+1} before the correction
+  R dr3 = 0, mt3 = 0, dp3 = 0;                           // Delta E or E'': E_r, E_th (mean of two columns), E_ph
+  R cd4 = 0, ct4 = 0, cp4 = 0;                           // corrected E: E_r (difference to the right), E_th, E_ph
+  // step k: row k is staged at `at`, row k-1 at `below`, and `next` is free
+  auto step = [&](int k, const unsigned char *at, const unsigned char *below, unsigned char *next, auto tag) {
+    constexpr bool IN = decltype(tag)::rows, CI = decltype(tag)::cols;
+    const bool jn = CI || jn_, jh = CI || jh_;
+    const bool south = !CI && j == 0, north = !CI && j == nt, axis = south || north, inner = CI || (j > 0 && j < nt);
+    if (k + kFuseStages - 2 <= kl) fetch(k + kFuseStages - 2, next, tag);
+    commit();
+    auto in = [&](int a) -> R { return reinterpret_cast<const R *>(at)[a * 32 + lane]; };
+    auto in1 = [&](int a) -> R { return reinterpret_cast<const R *>(below)[a * 32 + lane]; };
+    const R er = in(IN_ER), et = in(IN_ET), ep = in(IN_EP), dbr = in(IN_BR), dbt = in(IN_BT), dbp = in(IN_BP),
+            b0r = in(IN_B0R), b0t = in(IN_B0T), b0p = in(IN_B0P);
+    const P psi = reinterpret_cast<const P *>(at + 32 * IN_COUNT * sizeof(R))[lane];
+    // row k-1
+    const R er1 = in1(IN_ER), et1 = in1(IN_ET), ep1 = in1(IN_EP), bt1 = in1(IN_BT), bp1 = in1(IN_BP),
+            b0r1 = in1(IN_B0R), b0t1 = in1(IN_B0T), b0p1 = in1(IN_B0P);
+    const P psi1 = reinterpret_cast<const P *>(below + 32 * IN_COUNT * sizeof(R))[lane];
+    // --------------------------------------------------------- F1, J_perp
+    const R ep_r = right(ep);
+    R bhr = dbr;   // B_r(k, j+1/2)
+    if (jh) bhr -= hdt * (T(k, TB_INV_RN) * (sn1 * ep_r - sn0 * ep) * idcp);
+    const R tbr = b0r + dbr, tbr_l = left(tbr), tbt = b0t + dbt, bpk = b0p + dbp, tbp = left(bpk) + bpk;
+    const R et_l = left(et);
+    R jx = 0, jy = 0, jz = 0;
+    if ((IN || (k >= 1 && k < nr)) && jn) {
+      const R e0 = R(0.5) * (er1 + er), e1 = axis ? R(0) : R(0.5) * (et_l + et), e2 = axis ? R(0) : ep;
+      const R b0 = south ? tbr : north ? tbr_l : R(0.5) * (tbr_l + tbr);
+      const R b1 = axis ? R(0) : R(0.5) * (tbt1 + tbt), b2 = axis ? R(0) : R(0.25) * (tbp1 + tbp);
+      const R div = T(k, TB_RHO_A) * (T(k, TB_RH2) * er - T(k - 1, TB_RH2) * er1);
+      R dth = 0;
+      if (CI || j < nt) dth += sh0 * et;
+      if (CI || j > 0) dth -= shm * et_l;
+      const R rho = div + T(k, TB_RHO_B) * dth * idch;
+      const R bsq = b0 * b0 + b1 * b1 + b2 * b2;
+      if (bsq > b2min<R>()) {
+        const R s = rho / bsq;
+        jx = s * (e1 * b2 - e2 * b1);
+        jy = s * (e2 * b0 - e0 * b2);
+        jz = s * (e0 * b1 - e1 * b0);
+      }
+    }
+    if (own && k >= i_s && k < i_e) {
+      const int64_t kk = (int64_t)k * n1;
+      (f.jpr + kk)[ju] = jx; (f.jpt + kk)[ju] = jy; (f.jpp + kk)[ju] = jz;
+    }
+    // half row k-1
+    const int i1 = k - 1;
+    R bht = R(0), bhp = R(0);
+    const R er1_r = right(er1);
+    if (IN || (k >= 1 && i1 < nr)) {
+      const R cb2 = T(i1, TB_C_B2), rn0 = T(i1, TB_RN), rn1 = T(k, TB_RN);
+      if (inner) bht = bt1 + hdt * cb2 * (rn1 * ep - rn0 * ep1);   // zero on the axis
+      if (jh) {
+        const R cu = cb2 * (rn1 * et - rn0 * et1) - T(i1, TB_C_BP2) * (er1_r - er1);
+        bhp = bp1 - hdt * cu;
+      }
+    }
+    // B^{n+1/2} for N: B_r at node row k, half row k-1
+    const R hr = b0r + bhr, hr_l = left(hr);
+    const R nb = south ? hr : north ? hr_l : R(0.5) * (hr_l + hr);
+    const R bb1 = b0t1 + bht, hpk = b0p1 + bhp, pp1 = left(hpk) + hpk;
+    // ------------------------------------------------------ A at row k-1
+    const R bhp_l = left(bhp), br1_l = left(br1), jt1_r = right(jt1);
+    const P psi1_r = right(psi1);
+    R wr = f_lo, wt = f_lo, wn = f_lo;   // f at the E_r edge, the E_th edge and the node
+    const bool lo0 = __all_sync(0xffffffffu, psi_lead(psi) < psi_lo);
+    const bool hi0 = __all_sync(0xffffffffu, psi_lead(psi) > psi_hi);
+    if (hi0 && hi1) {
+      wr = wt = wn = f_hi;
+    } else if (!(lo0 && lo1)) {
+      wr = blend(p, psi_mean2(psi1, psi));
+      wt = blend(p, psi_mean2(psi1, psi1_r));
+      wn = blend(p, psi1);
+    }
+    lo1 = lo0;
+    hi1 = hi0;
+    R fr1 = 0, ft1 = 0, fn1 = 0, ar1 = 0, at1 = 0, ap1 = 0;
+    if (IN || (k >= 1 && i1 <= nr)) {
+      if ((IN || i1 < nr) && jn) {  // E_r(i+1/2, j)
+        R cu = R(0);
+        if (CI || j < nt) cu += sh0 * bhp;
+        if (CI || j > 0) cu -= shm * bhp_l;
+        cu *= T(i1, TB_INV_RH) * idch;
+        fr1 = wr;
+        const bool lo = IN || i1 >= 1, hi = IN || i1 + 1 <= nr - 1;
+        R jm = R(0);
+        if (lo) jm += jr1;
+        if (hi) jm += jx;
+        if (lo && hi) jm *= R(0.5);
+        const R jt = (R(1) - fr1) * in(IN_JR) + fr1 * jm;
+        ar1 = (er1 + dt * (cu + in(IN_SR)) - fp4 * jt) * (R(1) - T(i1, TB_SIG_H));
+      }
+      if (jh) {  // E_th(i, j+1/2)
+        if (!IN && i1 == 0) {
+          at1 = -p.omega * T(0, TB_RN) * sh0 * (b0r1 + br1);
+        } else if (!IN && i1 == nr) {
+          at1 = R(0);
+        } else {
+          const R cu = -T(i1, TB_C_E2) * (T(i1, TB_RH) * bhp - T(i1 - 1, TB_RH) * hp2);
+          ft1 = wt;
+          const R jt = (R(1) - ft1) * in(IN_JT) + ft1 * R(0.5) * (jt1 + jt1_r);
+          at1 = (et1 + dt * (cu + in(IN_ST)) - fp4 * jt) * (R(1) - T(i1, TB_SIG_N));
+        }
+      }
+      if ((IN || (i1 >= 1 && i1 < nr)) && inner) {  // E_ph(i, j)
+        const R cu = T(i1, TB_C_E2) * (T(i1, TB_RH) * bht - T(i1 - 1, TB_RH) * ht2) - T(i1, TB_C_EP2) * (br1 - br1_l);
+        fn1 = wn;
+        const R jt = (R(1) - fn1) * in(IN_JP) + fn1 * jp1;
+        ap1 = (ep1 + dt * (cu + in(IN_SP)) - fp4 * jt) * (R(1) - T(i1, TB_SIG_N));
+      }
+    }
+    // ------------------------------------------------------ N at row k-2
+    const int i2 = k - 2;
+    const R at2_l = left(at2);
+    R d0 = 0, d1 = 0, d2 = 0;
+    if ((IN || (i2 >= 1 && i2 < nr)) && jn) {
+      const R e0 = R(0.5) * (ar3 + ar2), e1 = axis ? R(0) : R(0.5) * (at2_l + at2), e2 = axis ? R(0) : ap2;
+      const R b0 = nb2, b1 = axis ? R(0) : R(0.5) * (bb3 + bb2), b2 = axis ? R(0) : R(0.25) * (pp3 + pp2);
+      const R bsq = b0 * b0 + b1 * b1 + b2 * b2;
+      if (bsq > b2min<R>()) {
+        const R sdot = (e0 * b0 + e1 * b1 + e2 * b2) / bsq;
+        const R x = e0 - sdot * b0, y = e1 - sdot * b1, z = e2 - sdot * b2;
+        const R esq = x * x + y * y + z * z;
+        R sc = R(1);
+        if (esq > bsq) {
+          sc = sqrt(bsq / esq);
+          if (own && i2 >= i_s && i2 < i_e) ++nclamp;
+        }
+        d0 = sc * x - e0;
+        d1 = sc * y - e1;
+        d2 = sc * z - e2;
+      }
+      if (lit) { d0 += e0; d1 += e1; d2 += e2; }
+    }
+    if (own && i2 >= i_s && i2 < i_e) {
+      const int64_t kk = (int64_t)i2 * n1;
+      (f.der + kk)[ju] = d0; (f.det + kk)[ju] = d1; (f.dep + kk)[ju] = d2;
+    }
+    const R mt2 = R(0.5) * (d1 + right(d1));
+    // ------------------------------------------------------ C at row k-3
+    const int i3 = k - 3;
+    const bool out = own && i3 >= i_s && i3 < i_e;
+    R f4 = R(0);
+    if constexpr (FILT) {   // fourth difference of E_th along theta
+      const R l1 = left(at3), l2 = __shfl_up_sync(0xffffffffu, at3, 2), r1 = right(at3),
+              r2 = __shfl_down_sync(0xffffffffu, at3, 2);
+      f4 = l2 - R(4) * l1 + R(6) * at3 - R(4) * r1 + r2;
+    }
+    R cr = ar3, ct = at3, cp = ap3;
+    if (IN || (i3 >= 0 && i3 <= nr)) {
+      if ((IN || i3 < nr) && jn) {  // E_r(i+1/2, j)
+        if (fr3 != R(0)) {
+          const bool lo = IN || i3 >= 1, hi = IN || i3 + 1 <= nr - 1;
+          R m = R(0);
+          if (lo) m += dr3;
+          if (hi) m += d0;
+          if (lo && hi) m *= R(0.5);
+          if constexpr (FILT) {
+            if (IN || (i3 >= 2 && i3 <= nr - 3))
+              m -= p.ff_sigma16 * (ar5 - R(4) * ar4 + R(6) * ar3 - R(4) * ar2 + ar1);
+          }
+          cr += fr3 * (lit ? m - ar3 : m);
+        }
+        if (out) (f.er + (int64_t)i3 * n1)[ju] = cr;
+      }
+      if (jh) {  // E_th(i, j+1/2)
+        if ((IN || (i3 >= 1 && i3 < nr)) && ft3 != R(0)) {
+          R m = mt3;
+          if (FILT && (CI || (j >= 2 && j <= nt - 3))) m -= p.ff_sigma16 * f4;
+          ct += ft3 * (lit ? m - at3 : m);
+        }
+        if (out) (f.et + (int64_t)i3 * nt)[ju] = ct;
+      }
+      if (jn) {  // E_ph(i, j)
+        if ((IN || (i3 >= 1 && i3 < nr)) && inner && fn3 != R(0)) cp += fn3 * (lit ? dp3 - ap3 : dp3);
+        if (out) (f.ep + (int64_t)i3 * n1)[ju] = cp;
+      }
+    }
+    // ----------------------------------- F2 at node row k-3, half row k-4
+    const R cp_r = right(cp), cd = right(cr) - cr;
+    if (out && jh) {
+      const R cu = T(i3, TB_INV_RN) * (sn1 * cp_r - sn0 * cp) * idcp;
+      R v = br3 - hdt * cu;
+      const R sg = T(i3, TB_SIG_N);
+      if (sg > R(0)) v -= sg * v;
+      (f.br + (int64_t)i3 * nt)[ju] = v;
+    }
+    const int h = k - 4;
+    if (own && h >= i_s && h < i_e && (IN || h < nr)) {
+      const R sg = T(h, TB_SIG_H), cb2 = T(h, TB_C_B2), rn0 = T(h, TB_RN), rn1 = T(h + 1, TB_RN);
+      R v = R(0);
+      if (inner) {
+        v = ht4 + hdt * cb2 * (rn1 * cp - rn0 * cp4);
+        if (sg > R(0)) v -= sg * v;
+      }
+      (f.bt + (int64_t)h * n1)[ju] = v;
+      if (jh) {
+        const R cu = cb2 * (rn1 * ct - rn0 * ct4) - T(h, TB_C_BP2) * cd4;
+        R w = hp4 - hdt * cu;
+        if (sg > R(0)) w -= sg * w;
+        (f.bp + (int64_t)h * nt)[ju] = w;
+      }
+    }
+    // ------------------------------------------------------- one row on
+    tbt1 = tbt; tbp1 = tbp; jr1 = jx; jt1 = jy; jp1 = jz;
+    br3 = br2; br2 = br1; br1 = bhr; ht4 = ht3; ht3 = ht2; ht2 = bht; hp4 = hp3; hp3 = hp2; hp2 = bhp;
+    nb2 = nb1; nb1 = nb; bb3 = bb2; bb2 = bb1; pp3 = pp2; pp2 = pp1;
+    fr3 = fr2; fr2 = fr1; ft3 = ft2; ft2 = ft1; fn3 = fn2; fn2 = fn1;
+    if constexpr (FILT) { ar5 = ar4; ar4 = ar3; }
+    ar3 = ar2; ar2 = ar1; at3 = at2; at2 = at1; ap3 = ap2; ap2 = ap1;
+    dr3 = d0; mt3 = mt2; dp3 = d2; cd4 = cd; ct4 = ct; cp4 = cp;
+  };
+  // interior steps: rows k-4 .. k+2 inside rows 2 .. nr-3
+  const int kin0 = 6, kin1 = nr - 5;
+  const bool some = j0 + H <= nt;   // this warp owns columns of the grid
+  constexpr int kStage = (int)fuse_stage_bytes<R>();
+  unsigned char *ring = fsmem + fuse_tab_rows(seg_rows) * kTabN * sizeof(R) + warp * (kFuseStages * kStage);
+  static_assert((kFuseStages & (kFuseStages - 1)) == 0, "ring");
+  auto slot = [&](int k) { return ring + (k & (kFuseStages - 1)) * kStage; };
+  for (int w = lane; w < kStage / 4; w += 32) reinterpret_cast<int *>(slot(k0 - 1))[w] = 0;   // the row before the first
+  __syncwarp();
+  for (int k = k0; k < k0 + kFuseStages - 2; ++k) {
+    if (some) fetch(k, slot(k), FuseTag<false, false>{});
+    commit();
+  }
+  for (int k = k0; k <= kl; ++k) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kFuseStages - 3) : "memory");
+    if (((k - k0) & 3) == 3) __syncthreads();   // see above: neighbours' reads before this warp's writes
+    if (!some) continue;
+    const unsigned char *at = slot(k), *below = slot(k - 1);
+    unsigned char *next = slot(k + kFuseStages - 2);
+    if (k < kin0 || k > kin1) step(k, at, below, next, FuseTag<false, false>{});
+    else if (cin) step(k, at, below, next, FuseTag<true, true>{});
+    else step(k, at, below, next, FuseTag<true, false>{});
+  }
   // running count of Eq. 26 activations (see k_node_b)
-  unsigned long long tot = nclamp;
+  unsigned tot = nclamp;
   for (int o = 16; o > 0; o >>= 1) tot += __shfl_down_sync(0xffffffffu, tot, o);
-  if ((threadIdx.x & 31) == 0 && tot) atomicAdd(p.clamps, tot);
+  if (lane == 0 && tot) atomicAdd(p.clamps, (unsigned long long)tot);
 }
 
-template <typename R> size_t field_fused_smem() { return fuse_smem_bytes<R>(); }
-template <typename R> const void *field_fused_fn() { return reinterpret_cast<const void *>(&k_field_fused<R>); }
-template <typename R> cudaError_t set_field_fused_smem(size_t bytes) { return raise_smem_limit<field_fused_fn<R>>(bytes); }
+template <typename R> size_t field_fused_smem(int seg_rows) {
+  return (size_t)fuse_tab_rows(seg_rows) * kTabN * sizeof(R) + fuse_warps(sizeof(R)) * kFuseStages * fuse_stage_bytes<R>();
+}
+template <typename R, bool F> const void *field_fused_fn() { return reinterpret_cast<const void *>(&k_field_fused<R, F>); }
+template <typename R> cudaError_t set_field_fused_smem(size_t bytes) {
+  const cudaError_t e = raise_smem_limit<field_fused_fn<R, false>>(bytes);
+  return e != cudaSuccess ? e : raise_smem_limit<field_fused_fn<R, true>>(bytes);
+}
 // rows per segment: as many segments as fit the strips into wave_blocks
 // resident blocks (one wave: every block walks its rows once, none waits
 // for a second wave), at least 32 rows so that the warm-up stays a small
-// share
-int fuse_seg_rows(int nr, int nt, int wave_blocks, size_t) {
-  const int strips = (nt + 1 + kFuseOwn - 1) / kFuseOwn;
+// share, and at most kFuseMaxRows (the staged radial tables)
+int fuse_seg_rows(int nr, int nt, int wave_blocks, size_t real, bool filt) {
+  const int cols = fuse_cols(real, filt), strips = (nt + 1 + cols - 1) / cols;
   const int segs = std::max(1, wave_blocks / strips);
-  return std::max(32, (nr + 1 + segs - 1) / segs);
+  return std::min(kFuseMaxRows, std::max(32, (nr + 1 + segs - 1) / segs));
 }
-template <typename R> int field_fused_blocks_per_sm() {
-  int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_field_fused<R>, kFuseThreads, fuse_smem_bytes<R>()) !=
-      cudaSuccess)
-    return 0;
-  return n;
-}
-int fuse_own_cols(size_t) { return kFuseOwn; }
-size_t fuse_snap_bytes(int nr, int nt, int seg_rows, size_t real) {
-  const FuseGeom fg = fuse_geom(nr, nt, seg_rows);
+size_t fuse_snap_bytes(int nr, int nt, int seg_rows, size_t real, bool filt) {
+  const FuseGeom fg = fuse_geom(nr, nt, seg_rows, fuse_cols(real, filt));
   return (size_t)(fuse_snap_cols(nr, fg.strips) + fuse_snap_rows(nt, fg.segs)) * real;
 }
 template <typename R> void launch_field_fused(const Params<R> &p, int seg_rows, void *snap, bool collect, cudaStream_t s) {
-  const FuseGeom fg = fuse_geom(p.nr, p.nt, seg_rows);
+  const bool filt = p.ff_sigma16 != R(0);
+  const int cols = fuse_cols(sizeof(R), filt);
+  const FuseGeom fg = fuse_geom(p.nr, p.nt, seg_rows, cols);
   R *sc = reinterpret_cast<R *>(snap);
   R *sr = sc + fuse_snap_cols(p.nr, fg.strips);
-  const int nc = (fg.strips - 1) * kFuseArrays * ((p.nr + kSnapRows) / kSnapRows);
-  const int nw = (fg.segs - 1) * kFuseArrays * (kFuseWarm + kFuseTrail) * (p.nt / kSnapThreads + 1);
+  const int nc = (fg.strips - 1) * ((p.nr + kSnapRows) / kSnapRows);
+  const int nw = (fg.segs - 1) * (kFuseWarm + kFuseTrail) * (p.nt / kSnapThreads + 1);
   const int nj = collect ? collect_blocks_x(p) * collect_blocks_y(p) : 0;
-  if (nc + nw + nj > 0) k_fuse_prepare<R><<<nc + nw + nj, kSnapThreads, 0, s>>>(p, sc, sr, seg_rows, nc, nw);
-  k_field_fused<R><<<dim3(fg.strips, fg.segs), kFuseThreads, fuse_smem_bytes<R>(), s>>>(p, R(0.5) * p.dt, fg, sc, sr);
+  if (nc + nw + nj > 0) k_fuse_prepare<R><<<nc + nw + nj, kSnapThreads, 0, s>>>(p, sc, sr, seg_rows, cols, nc, nw);
+  const dim3 grid(fg.strips, fg.segs);
+  const int threads = 32 * fuse_warps(sizeof(R));
+  const size_t smem = field_fused_smem<R>(seg_rows);
+  if (filt) k_field_fused<R, true><<<grid, threads, smem, s>>>(p, R(0.5) * p.dt, fg, sc, sr);
+  else k_field_fused<R, false><<<grid, threads, smem, s>>>(p, R(0.5) * p.dt, fg, sc, sr);
 }
 
 // The per-cell pure force-free flag f(Psi_cell) >= 1 (used to remove
@@ -1098,9 +1105,8 @@ template <typename R> void launch_combine(R *dst, const R *a, const R *b, int64_
   template void launch_correct<R>(const Params<R> &, cudaStream_t);            \
   template void launch_blend_out<R>(const Params<R> &, R *, R *, R *, uint8_t *, cudaStream_t); \
   template void launch_field_fused<R>(const Params<R> &, int, void *, bool, cudaStream_t);      \
-  template size_t field_fused_smem<R>();                                                         \
-  template cudaError_t set_field_fused_smem<R>(size_t);                                          \
-  template int field_fused_blocks_per_sm<R>();
+  template size_t field_fused_smem<R>(int);                                                         \
+  template cudaError_t set_field_fused_smem<R>(size_t);
 HFF_INST(float)
 HFF_INST(double)
 #undef HFF_INST

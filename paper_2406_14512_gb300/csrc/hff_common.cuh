@@ -32,6 +32,20 @@ inline cudaError_t raise_smem_limit(size_t bytes) {
   return e;
 }
 
+// copies of B bytes from global to shared memory behind the program's back
+// (completed by wait_group); the second form writes zeros where !ok
+template <int B>
+__device__ __forceinline__ void copy_async(void *dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "n"(B)
+               : "memory");
+}
+template <int B>
+__device__ __forceinline__ void copy_async(void *dst, const void *src, bool ok) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+               "n"(B), "r"(ok ? B : 0)
+               : "memory");
+}
+
 // status bits latched on the device
 constexpr unsigned kStCapacity = 1u;
 constexpr unsigned kStNonfinite = 2u;
@@ -68,6 +82,9 @@ __host__ __device__ __forceinline__ bool psi_lt(float2 a, float2 b) { return a.x
 __host__ __device__ __forceinline__ bool psi_lt(double a, double b) { return a < b; }
 __host__ __device__ __forceinline__ float psi_diff(float2 a, float2 b) { return (a.x - b.x) + (a.y - b.y); }
 __host__ __device__ __forceinline__ double psi_diff(double a, double b) { return a - b; }
+// the leading part: the value to 6e-8 (FP32) or exactly
+__host__ __device__ __forceinline__ float psi_lead(float2 a) { return a.x; }
+__host__ __device__ __forceinline__ double psi_lead(double a) { return a; }
 // Psi at an edge is the mean of its two nodes, at a cell the mean of four
 template <typename P> __device__ __forceinline__ P psi_mean2(P a, P b) { return psi_scale(psi_add(a, b), 0.5f); }
 template <typename P> __device__ __forceinline__ P psi_mean4(P a, P b, P c, P d) {
@@ -285,11 +302,10 @@ template <typename R> void launch_blend_out(const Params<R> &p, R *fr, R *ft, R 
 // Ampere, renormalisation, return, Faraday half with absorber) in one pass
 // over row segments of seg_rows rows
 template <typename R> void launch_field_fused(const Params<R> &p, int seg_rows, void *snap, bool collect, cudaStream_t s);
-int fuse_own_cols(size_t real);                                     // theta columns a strip owns
-int fuse_seg_rows(int nr, int nt, int wave_blocks, size_t real);    // rows per segment of the launch
-template <typename R> int field_fused_blocks_per_sm();              // its occupancy (0 = unknown)
-size_t fuse_snap_bytes(int nr, int nt, int seg_rows, size_t real);  // its halo snapshot
-template <typename R> size_t field_fused_smem();
+constexpr int kFuseBlocksPerSm = 2;                                 // its resident blocks
+int fuse_seg_rows(int nr, int nt, int wave_blocks, size_t real, bool filt);    // rows per segment of the launch
+size_t fuse_snap_bytes(int nr, int nt, int seg_rows, size_t real, bool filt);  // its halo snapshot
+template <typename R> size_t field_fused_smem(int seg_rows);
 template <typename R> cudaError_t set_field_fused_smem(size_t bytes);
 // dst[k] = a[k] + sign * b[k], k < n (B <-> B - B_0 at the ABI)
 template <typename R> void launch_combine(R *dst, const R *a, const R *b, int64_t n, int sign, cudaStream_t s);

@@ -769,10 +769,6 @@ static_assert(kPushThreads * 32 >= kMaxItem, "one bit per round of a work item")
 // are pushed (one slot per thread and array, read back by the thread that
 // copied it): the loads' latency, lengthened by the reductions in the L2's
 // queues, was the largest stall, and registers have no room for them.
-template <int B> __device__ __forceinline__ void copy_async(void *dst, const void *src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "n"(B)
-               : "memory");
-}
 template <typename R>
 struct Prefetch {
   R *slot;   // 7 arrays of kPushThreads slots (the first holds the cells)
