@@ -47,6 +47,32 @@ def test_particles_that_drifted_out_of_their_tile(tile, prec, tol, err):
     assert sim.info().pushed_tiled >= 12 * live and sim.status() == 0
 
 
+@pytest.mark.parametrize("prec,err", [("fp32", 1e-5), ("fp64", 1e-11)])
+@pytest.mark.parametrize("n", [(0, 1), (1, 0), (31, 33), (0, 0), (7, 160_000), (160_000, 5)])
+def test_tail_is_one_list_over_the_species(n, prec, err):
+    """Particles outside the tiles are handed out as one list over the species,
+    a warp at a time: empty species, lists that end inside a warp, and more
+    particles than the launch has threads (152 x 4 x 256), one push without
+    sorting (the tolerances of the one-step parity tests)."""
+    hff, workloads, oracle = _libs()
+    cfg = workloads.config("small_rr")
+    cfg.update(capacity=170_000, precision=prec, sort_every=0, inject=False)
+    ps = workloads.particles(cfg, n_pairs=max(*n, 1), seed=23)
+    sim, ref = hff.Sim(cfg), oracle.Oracle(cfg)
+    shared_initial_state(sim, ref, seed=7)
+    for s in range(2):
+        part = {k: v[:n[s]] for k, v in ps[s].items()}
+        sim.load(s, part)
+        ref.set_particles(s, part)
+    sim.step_stages(1, ST["node"] | ST["push"])
+    ref.step(1, ST["node"] | ST["push"])
+    for s in range(2):
+        bad, _, e = particle_mismatches(sim.particles(s), ref.particles(s), cfg["nt"])
+        assert bad == 0 and e < err, (s, bad, e)
+    info = sim.info()
+    assert (info.pushed_tiled, info.pushed_tail) == (0, sum(n)) and sim.status() == 0
+
+
 def test_fp64_momentum_whose_square_overflows():
     """|u| = 1e160: u^2 is infinite, 1/gamma zero, and the particle neither
     moves nor is removed (the reciprocal square root at the end of its range)."""
