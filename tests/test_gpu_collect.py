@@ -1,6 +1,6 @@
 """J_PIC out of the push's flux accumulators, against the FP64 oracle, on grids
 around the widths of the collection (warps of 32 columns, blocks of 128,
-segments of 16 rows) with particles in every cell inside the absorber, from
+segments of rows, odd and even row counts) with particles in every cell inside the absorber, from
 the star and up to the axis: each location must get the parts of all the cells that meet there.
 
 Tolerances: the tiled FP32 deposit's and the FP64 one's of the parity tests
