@@ -446,9 +446,10 @@ __global__ void __launch_bounds__(kRowThreads) k_correct(Params<R> p) {
 //
 // Bound by issue and dependent-instruction latency (640 instructions per warp
 // and row at 4 warps per scheduler, 60% of the issue slots; DRAM at 45%): FP32
-// 0.16 ms at 2048^2 and 0.57 at 4096^2, FP64 1.78 ms at 2048^2 (FP64 pipe).
+// 0.16 ms at 2048^2 and 0.57 at 4096^2 (0.19 and 0.68 where many nodes are
+// mixed or clamped), FP64 1.78 ms at 2048^2 (FP64 pipe).
 // With the rows in shared-memory rings of a 128-thread block, four barriers a
-// row and 1,050 instructions, it took 0.24, 0.81 and 1.96 ms.  10 warps a
+// row and 1,050 instructions, it took 0.24, 0.81 (0.25, 0.85) and 1.96 ms.  10 warps a
 // block at 96 registers: the same at 2048^2, 0.64 ms at 4096^2; blocks of 4 or
 // 5 warps: 0.18 - 0.19 and 0.72 - 0.76 ms, for their snapshot columns.
 //
