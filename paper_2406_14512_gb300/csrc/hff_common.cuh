@@ -363,7 +363,9 @@ cudaError_t set_sort_smem();
 template <typename R> void launch_materialize(const Params<R> &p, int species, cudaStream_t s);
 // loaded cells at or past ncells become removed particles; kStBadCell latched
 void launch_check_cells(int32_t *cell, int64_t n, int64_t ncells, unsigned *status, cudaStream_t s);
-// the work list of the tiled push from the tile bounds of all species
-template <typename R> void launch_worklist(const Params<R> &p, const SortScratch &ss, const WorkList &wl, cudaStream_t s);
+// the work list of the tiled push from the tile bounds of all species (empty if
+// unsettled is given and set: the bounds are then not those of sorted particles)
+template <typename R> void launch_worklist(const Params<R> &p, const SortScratch &ss, const WorkList &wl,
+                                           const int *unsettled, cudaStream_t s);
 
 }  // namespace hff

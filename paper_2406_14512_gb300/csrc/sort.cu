@@ -446,7 +446,8 @@ __global__ void __launch_bounds__(256) k_unpack(const Record<R> *rec, Species<R>
 
 // Is a species in the state a sort leaves (no removed or appended particles,
 // keys ascending)?  Its tile bounds are taken afresh on the way; *unsettled is
-// set if not.
+// set if not, and its bounds then mean nothing: every run of a tile's particles
+// writes the same two entries.
 __global__ void __launch_bounds__(kSortThreads) k_settled(const int32_t *cell, const long long *count,
                                                           const long long *count_sorted, int species,
                                                           const __grid_constant__ SortArgs a, int *bounds, int ntiles,
@@ -480,9 +481,16 @@ __global__ void __launch_bounds__(kSortThreads) k_settled(const int32_t *cell, c
   if (__any_sync(0xffffffffu, bad) && lane == 0) *unsettled = 1;
 }
 
-// ceil(count/chunk) items per non-empty tile, species after species
+// ceil(count/chunk) items per non-empty tile, species after species.  The sum
+// is bounded (by the length that the list was given) for the bounds of sorted
+// particles only: after a load beside an unsettled species there are none yet,
+// the list is left empty, and the sort that follows makes it.
 __global__ void __launch_bounds__(1024) k_worklist(const int *bounds, int ntiles, int n_species, int chunk, int4 *items,
-                                                   int *n_items, int max_items, unsigned *status) {
+                                                   int *n_items, int max_items, unsigned *status, const int *unsettled) {
+  if (unsettled && *unsettled) {
+    if (threadIdx.x == 0) *n_items = 0;
+    return;
+  }
   __shared__ uint32_t w[33];
   __shared__ uint32_t carry;
   if (threadIdx.x == 0) carry = 0u;
@@ -498,7 +506,7 @@ __global__ void __launch_bounds__(1024) k_worklist(const int *bounds, int ntiles
       const uint32_t ex = block_excl_scan(ni, w, tot);
       for (uint32_t c = 0; c < ni; ++c) {
         const uint32_t slot = carry + ex + c;
-        if ((int)slot < max_items) {
+        if (slot < (uint32_t)max_items) {
           const int s0 = start[k] + (int)c * chunk;
           const int len = min(chunk, end[k] - s0);
           items[slot] = make_int4(species, k, s0, len);
@@ -511,7 +519,7 @@ __global__ void __launch_bounds__(1024) k_worklist(const int *bounds, int ntiles
       __syncthreads();
     }
   }
-  if (threadIdx.x == 0) *n_items = (int)min((int)carry, max_items);
+  if (threadIdx.x == 0) *n_items = (int)min(carry, (uint32_t)max_items);
 }
 
 static int bits_for(uint32_t v) {
@@ -621,8 +629,8 @@ void launch_materialize(const Params<R> &p, int s, cudaStream_t st) {
 }
 
 template <typename R>
-void launch_worklist(const Params<R> &p, const SortScratch &ss, const WorkList &wl, cudaStream_t st) {
-  k_worklist<<<1, 1024, 0, st>>>(ss.bounds, ss.ntiles, p.n_species, wl.chunk, wl.items, wl.n_items, wl.max_items, p.status);
+void launch_worklist(const Params<R> &p, const SortScratch &ss, const WorkList &wl, const int *unsettled, cudaStream_t st) {
+  k_worklist<<<1, 1024, 0, st>>>(ss.bounds, ss.ntiles, p.n_species, wl.chunk, wl.items, wl.n_items, wl.max_items, p.status, unsettled);
 }
 
 #define HFF_INST(R)                                                                                   \
@@ -631,7 +639,7 @@ void launch_worklist(const Params<R> &p, const SortScratch &ss, const WorkList &
                                       int *, cudaStream_t);                                            \
   template size_t load_record_bytes<R>();                                                              \
   template void launch_materialize<R>(const Params<R> &, int, cudaStream_t);                           \
-  template void launch_worklist<R>(const Params<R> &, const SortScratch &, const WorkList &, cudaStream_t);
+  template void launch_worklist<R>(const Params<R> &, const SortScratch &, const WorkList &, const int *, cudaStream_t);
 HFF_INST(float)
 HFF_INST(double)
 #undef HFF_INST
