@@ -8,6 +8,8 @@
 #include <string>
 #include <vector>
 
+#include <cuda.h>
+
 #include "../../include/hff.h"
 #include "diag.cuh"
 #include "hff_common.cuh"
@@ -1244,11 +1246,47 @@ Species<R> species_of(const void *const src[7]) {
   return s;
 }
 
+// Do [a, a + na) and [b, b + nb) overlap?
+bool meets(const void *a, size_t na, const void *b, size_t nb) {
+  const char *x = static_cast<const char *>(a), *y = static_cast<const char *>(b);
+  return x < y + nb && y < x + na;
+}
+
+// May a kernel of the current device read [a, a + bytes) as elements of `align`
+// bytes?  Device memory of this device, aligned, within one allocation.
+// Everything else goes through cudaMemcpyAsync, which copies from any memory
+// it knows, at any alignment, and answers a wrong pointer with an error where
+// a kernel would fault.
+bool readable_here(const void *a, size_t bytes, size_t align) {
+  if ((uintptr_t)a % align != 0) return false;
+  using Range = CUresult (*)(CUdeviceptr *, size_t *, CUdeviceptr);
+  static const Range range = [] {
+    void *f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+      f = nullptr;
+    return reinterpret_cast<Range>(f);
+  }();
+  int dev = 0;
+  cudaPointerAttributes at;
+  if (!range || cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&at, a) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  if (at.type != cudaMemoryTypeDevice || at.device != dev) return false;
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  if (range(&base, &size, (CUdeviceptr)(uintptr_t)a) != CUDA_SUCCESS) return false;
+  return (uintptr_t)a - (uintptr_t)base + bytes <= size;
+}
+
 // A load with sorting: the species' particles go straight from the caller's
-// device arrays (or, from the host, from its slots of the current buffer)
-// into sorted order there; the other species stay where they are, unless they
-// are not as a sort leaves them (particles moved, removed or appended since):
-// then all are sorted, as on the cadence, and only that sort makes a work list.
+// device arrays (or, where a kernel cannot read those, from a copy in its slots
+// of the current buffer) into sorted order there; the other species stay where
+// they are, unless they are not as a sort leaves them (particles moved, removed
+// or appended since): then all are sorted, as on the cadence, and only that
+// sort makes a work list.
 // (The loaded species is sorted twice then.  Sorting once, from the caller's
 // order, gathers seven scattered words per particle instead of one record: a
 // load between steps, 2 x 1.25e7 particles on 1024^2, takes 1.57 ms with both
@@ -1260,20 +1298,28 @@ int load_sorted(hff_handle *h, int species, int64_t n, const void *const src[7],
     for (int k = 0; k < 7; ++k) mine[par][k] = h->base + h->o.part[par][species][k];
   const int pp = h->parity;
   const void *from[7];
-  bool inside = false;   // device arrays inside the instance's own memory
+  // device arrays that no kernel may read as they are, or that lie in the
+  // instance's own memory, in this species' slots of the current buffer
+  bool staged = where == HFF_HOST, inside = false, meets_mine = false;
   for (int k = 0; k < 7; ++k) {
     from[k] = src[k];
-    const char *c = static_cast<const char *>(src[k]);
+    if (where == HFF_HOST || n == 0) continue;
     const size_t b = (size_t)n * (k == 0 ? 4 : sizeof(R));
-    if (where == HFF_DEVICE && n > 0 && c < h->base + h->o.total && c + b > h->base) inside = true;
+    staged = staged || !readable_here(src[k], b, k == 0 ? 4 : sizeof(R));
+    inside = inside || meets(src[k], b, h->base, h->o.total);
+    for (int m = 0; m < 7; ++m)
+      meets_mine = meets_mine || meets(src[k], b, mine[pp][m], (size_t)h->c.capacity * (m == 0 ? 4 : sizeof(R)));
   }
   // records fit the other parity's arrays of two or more species
   void *rec = h->c.n_species >= 2 ? (void *)(h->base + h->o.part[pp ^ 1][0][0]) : nullptr;
-  if (where == HFF_HOST || inside) {
-    // staged in the current buffer (read by the packing before the sorted
-    // particles overwrite it), or in the other one where there is no packing
-    const int to = rec && !inside ? pp : pp ^ 1;
-    if (inside) rec = nullptr;
+  // the records, or the sorted particles, would overwrite a source inside
+  staged = staged || (inside && (rec || meets_mine));
+  if (staged) {
+    // in the current buffer (read by the packing before the sorted particles
+    // overwrite it); in the other one, without packing, where the source lies
+    // in the current slots or there is no packing
+    const int to = rec && !meets_mine ? pp : pp ^ 1;
+    if (to != pp) rec = nullptr;
     for (int k = 0; k < 7; ++k) {
       const cudaMemcpyKind kind = where == HFF_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
       if (n > 0) CK(cudaMemcpyAsync(mine[to][k], src[k], (size_t)n * (k == 0 ? 4 : sizeof(R)), kind, h->st));

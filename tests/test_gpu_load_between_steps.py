@@ -113,3 +113,39 @@ def test_load_from_views_between_steps():
     live = _host(sim, 1)
     sim.load_device(0, {k: v[1000:] for k, v in sim.particle_views(0).items()})
     _check(cfg, sim, [_sorted(cfg, {k: v[1000:] for k, v in live[0].items()})])
+
+
+def test_load_from_views_taken_before_another_load():
+    """A load between steps moves every species to the other buffer; the arrays
+    of a view taken before it can still be loaded, in part, too."""
+    hff, cfg, ps = _setup("fp32", n_pairs=100_000, nr=128, nt=96)
+    sim = hff.Sim(cfg)
+    for s in range(2):
+        sim.load(s, ps[s])
+    sim.step(3)
+    live = _host(sim, 2)
+    v = sim.particle_views(0)
+    sim.load(1, ps[1])
+    sim.load_device(0, {k: a[1000:] for k, a in v.items()})
+    _check(cfg, sim, [_sorted(cfg, {k: a[1000:] for k, a in live[0].items()}), _sorted(cfg, ps[1])])
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("n_species", [1, 2])
+@pytest.mark.parametrize("offset", [1, 4])
+def test_load_from_device_arrays_at_any_address(prec, n_species, offset):
+    """Device arrays that start between the addresses of their elements (one
+    packed buffer: the cells, then the reals, FP64 ones at a multiple of four)."""
+    import torch
+    hff, cfg, ps = _setup(prec, n_species=n_species, n_pairs=100_000, nr=128, nt=96)
+    sim = hff.Sim(cfg)
+    for s in range(n_species):
+        sim.load(s, ps[s])
+    new = {k: v[::-1].astype(np.int32 if k == "cell" else sim.real) for k, v in ps[0].items()}
+    raw = [np.zeros(offset, np.uint8)] + [np.ascontiguousarray(new[k]).view(np.uint8) for k in KEYS]
+    buf = torch.from_numpy(np.concatenate(raw)).cuda()
+    at = buf.data_ptr() + np.cumsum([len(r) for r in raw])[:-1]
+    assert any(int(a) % (4 if k == 0 else new["xo"].itemsize) for k, a in enumerate(at)) or (prec, offset) == ("fp32", 4)
+    hff.hff_load_particles(sim.h, 0, 0, len(new["cell"]), [int(a) for a in at], hff.DEVICE)
+    want = [new] + [{k: v.astype(new[k].dtype) for k, v in p.items()} for p in ps[1:]]
+    _check(cfg, sim, [_sorted(cfg, w) for w in want])
