@@ -203,6 +203,8 @@ struct Offsets {
   size_t items;
   size_t qnode, rows, psi64;
   size_t jacc;           // flux accumulators of the push
+  size_t records;        // FP32: flux records of the push's blocks (crowded items)
+  int record_blocks;     // the most blocks of the push
   size_t fsnap;          // halo snapshot of the fused field update
   int seg_rows;          // rows per segment of the fused field update
   size_t ev[8];          // pair-creation events: key cell xo yo ur ut up w
@@ -228,6 +230,15 @@ struct Small {  // device counters, one 256-byte block
   int n_items;
   int next, done;             // work queue of the tiled push (both 0 between pushes)
 };
+
+// halo of the tiled push: farthest drift between sorts (Courant-bounded)
+int halo_of(const hff_config &c) {
+  const double dt = courant_dt(c), dlog = std::log(c.r_max / c.r_min) / c.nr;
+  const double dxi = -std::log(1.0 - dt / c.r_min) / dlog;
+  const double deta = std::asin(std::fmin(1.0, dt / c.r_min)) / (kPi / c.nt);
+  const double d = std::fmax(dxi, deta);
+  return (int)std::ceil((c.sort_every > 0 ? c.sort_every : 1) * d + 1e-9);
+}
 
 int tile_r_of(const hff_config &c) { return c.tile_r > 0 ? c.tile_r : 16; }
 int tile_t_of(const hff_config &c) { return c.tile_t > 0 ? c.tile_t : 32; }
@@ -289,6 +300,9 @@ void layout(const hff_config &c, Offsets &o) {
   for (int k = 0; k < 8; ++k) o.ev[k] = o.ev_cap ? L.take((size_t)o.ev_cap * (k < 2 ? 4 : R)) : 0;
   o.spec = L.take(4096 * 8);
   o.jacc = cap ? L.take(push_acc_bytes(c.nr, c.nt, R)) : 0;
+  const bool records = cap && c.sort_every > 0 && c.precision == HFF_FP32;
+  o.record_blocks = records ? push_record_blocks(tr, tt, halo_of(c)) : 0;
+  o.records = records ? L.take(std::min(o.record_blocks, o.max_items) * push_record_bytes(tr, tt, halo_of(c))) : 0;
   o.qnode = L.take(nn * 8);
   o.rows = L.take((nr + 1) * 8 * 8);
   o.psi64 = L.take(nn * 8);
@@ -1167,18 +1181,13 @@ static int init_one(const hff_config *cfg, void *dev_mem, size_t bytes, void *st
         cudaStreamSynchronize(h->st) != cudaSuccess)
       return bail(fail(HFF_ERR_CUDA, "init copy failed"));
   }
-  // halo of the tiled push: farthest drift between sorts (Courant-bounded)
-  {
-    const double dxi = -std::log(1.0 - h->dt / cfg->r_min) / h->g.dlog;
-    const double deta = std::asin(std::fmin(1.0, h->dt / cfg->r_min)) / h->g.dth;
-    const double d = std::fmax(dxi, deta);
-    h->halo = (int)std::ceil((cfg->sort_every > 0 ? cfg->sort_every : 1) * d + 1e-9);
-  }
+  h->halo = halo_of(h->c);
   h->wl.items = reinterpret_cast<int4 *>(h->base + h->o.items);
   h->wl.n_items = &h->small->n_items;
   h->wl.next = &h->small->next;
   h->wl.done = &h->small->done;
   h->wl.max_items = h->o.max_items;
+  h->wl.records = reinterpret_cast<float *>(h->base + h->o.records);
   h->wl.chunk = chunk_of(*cfg);
   h->ss.keys = reinterpret_cast<uint32_t *>(h->base + h->o.keys);
   h->ss.idx = reinterpret_cast<uint32_t *>(h->base + h->o.idx);
@@ -1216,6 +1225,8 @@ static int init_one(const hff_config *cfg, void *dev_mem, size_t bytes, void *st
       if (!push_tile_fits<float>(h->pf[0], h->halo)) return bail(fail(HFF_ERR_ARG, "tile + halo too large for shared memory"));
       if (set_push_smem<float>(smem) != cudaSuccess) return bail(fail(HFF_ERR_CUDA, "cannot set shared memory size"));
       h->push_grid = nsm * std::max(1, std::min(8, push_tiled_blocks_per_sm<float>(smem)));
+      // every block that can get an item has records (a list has at most max_items)
+      if (h->o.record_blocks) h->push_grid = std::min(h->push_grid, h->o.record_blocks);
     }
   } else {
     fill_params<double>(h);

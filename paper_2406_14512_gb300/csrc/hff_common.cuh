@@ -314,19 +314,29 @@ template <typename R> void launch_combine(R *dst, const R *a, const R *b, int64_
 constexpr int kPushThreads = 256;
 constexpr int kMaxItem = 8192;
 
+// an item's first word: its species, how it deposits (see push_tiled; neither
+// until its first push has looked), and times kItemTotal the particles that its
+// tile holds of all species, at most kItemTotalMax
+constexpr int kItemDirect = 4, kItemOwn = 8, kItemTotal = 16;
+constexpr int kItemTotalMax = 1 << 26;
+static_assert(kMaxSpecies <= kItemDirect, "item word");
+
 struct WorkList {
-  int4 *items;          // (species, tile, start, count)
+  int4 *items;          // (species and total, tile, start, count)
   int *n_items;         // device count
   int *next;            // dynamic scheduling counter (0 between pushes)
   int *done;            // blocks of the running push that have finished
   int max_items;
   int chunk;            // particles per item
+  float *records;       // FP32: flux records of the region of each block's tile (zero between items)
 };
 
 template <typename R> void launch_push_tail(const Params<R> &p, cudaStream_t s, int grid);
 template <typename R> void launch_push_tiled(const Params<R> &p, const WorkList &wl, int halo,
                                              cudaStream_t s, int grid, bool gather);
 template <typename R> size_t push_tiled_smem(const Params<R> &p, int halo);
+int push_record_blocks(int tile_r, int tile_t, int halo);    // blocks with records of their own
+size_t push_record_bytes(int tile_r, int tile_t, int halo);  // and what each of them takes
 template <typename R> bool push_tile_fits(const Params<R> &p, int halo);  // accepted by hff_init
 // the push's flux accumulators added to J_PIC and cleared
 template <typename R> void launch_collect(const Params<R> &p, cudaStream_t s);

@@ -15,6 +15,7 @@
 //  * k_push_tail -- all particles of the no-sort configuration, the same way.
 // Both deposit into the flux accumulators in global memory (see deposit);
 // those become J_PIC at the end of the push stage (collect.cuh).
+#include <algorithm>
 #include <type_traits>
 
 #include "collect.cuh"
@@ -432,24 +433,47 @@ __device__ __forceinline__ void red_add4(float *p, float a, float b, float c, fl
 // the L2 adds, not the SM, whose FP64 pipe bounds the FP64 push.
 __device__ __forceinline__ int64_t acc_index(const Params<float> &p, int i, int j) { return 8 * ix(i, j, p.nt + 1); }
 __device__ __forceinline__ int64_t acc_index(const Params<double> &p, int i, int j) { return ix(i, j, p.nt + 2); }
+// Where a particle deposits: the mesh's accumulators (FP32 and FP64), or, in
+// crowded work items (FP32, see push_item), the block's own records of the
+// tile's region, and then summed by cell within the warp first where `share`.
+template <typename R>
+struct MeshAcc {
+  static constexpr bool kShare = false;
+  const Params<R> &p;
+  __device__ __forceinline__ R *at(int i, int j) const { return p.jacc + acc_index(p, i, j); }
+};
+struct TileAcc {
+  static constexpr bool kShare = true;
+  float *base;
+  int i0, j0, ld;
+  bool share;
+  __device__ __forceinline__ float *at(int i, int j) const { return base + 8 * ix(i - i0, j - j0, ld); }
+};
 // fluxes of one cell: J_r through its radial face at its two nodes, J_th
 // through its polar face at its two nodes
-__device__ __forceinline__ void add_faces(const Params<float> &p, int i, int j, float r0, float r1, float t0, float t1) {
-  red_add4(p.jacc + acc_index(p, i, j), r0, r1, t0, t1);
+template <typename A>
+__device__ __forceinline__ void add_faces(const Params<float> &, const A &acc, int i, int j, float r0, float r1,
+                                          float t0, float t1) {
+  red_add4(acc.at(i, j), r0, r1, t0, t1);
 }
-__device__ __forceinline__ void add_faces(const Params<double> &p, int i, int j, double r0, double r1, double t0,
-                                          double t1) {
+template <typename A>
+__device__ __forceinline__ void add_faces(const Params<double> &p, const A &acc, int i, int j, double r0, double r1,
+                                          double t0, double t1) {
   const int ld = p.nt + 2;
-  double *q = p.jacc + acc_index(p, i, j), *t = q + (int64_t)(p.nr + 2) * ld;
+  double *q = acc.at(i, j), *t = q + (int64_t)(p.nr + 2) * ld;
   atomicAdd(q, r0); atomicAdd(q + 1, r1);
   atomicAdd(t, t0); atomicAdd(t + ld, t1);
 }
-__device__ __forceinline__ void add_corners(const Params<float> &p, int i, int j, float a, float b, float c, float d) {
-  red_add4(p.jacc + acc_index(p, i, j) + 4, a, b, c, d);
+template <typename A>
+__device__ __forceinline__ void add_corners(const Params<float> &, const A &acc, int i, int j, float a, float b,
+                                            float c, float d) {
+  red_add4(acc.at(i, j) + 4, a, b, c, d);
 }
-__device__ __forceinline__ void add_corners(const Params<double> &p, int i, int j, double a, double b, double c, double d) {
+template <typename A>
+__device__ __forceinline__ void add_corners(const Params<double> &p, const A &acc, int i, int j, double a, double b,
+                                            double c, double d) {
   const int ld = p.nt + 2;
-  double *q = p.jacc + 2 * (int64_t)(p.nr + 2) * ld + acc_index(p, i, j);
+  double *q = acc.at(i, j) + 2 * (int64_t)(p.nr + 2) * ld;
   atomicAdd(q, a); atomicAdd(q + 1, b); atomicAdd(q + ld, c); atomicAdd(q + ld + 1, d);
 }
 
@@ -493,16 +517,16 @@ __device__ __forceinline__ bool sum_by_cell(int key, float (&v)[N]) {
   }
   return first;
 }
-__device__ __forceinline__ void add_faces_shared(const Params<float> &p, int i, int j, float r0, float r1, float t0,
-                                                 float t1) {
+__device__ __forceinline__ void add_faces_shared(const Params<float> &p, const TileAcc &acc, int i, int j, float r0,
+                                                 float r1, float t0, float t1) {
   float v[4] = {r0, r1, t0, t1};
-  if (sum_by_cell((int)ix(i, j, p.nt + 1), v)) add_faces(p, i, j, v[0], v[1], v[2], v[3]);
+  if (!acc.share || sum_by_cell((int)ix(i, j, p.nt + 1), v)) add_faces(p, acc, i, j, v[0], v[1], v[2], v[3]);
 }
 
 // sx, sy: the cell entered in either direction (-1, 0, 1)
-template <bool kShare, typename R>
-__device__ __forceinline__ void deposit(const Params<R> &p, R qw, int i, int j, int sx, int sy, R x0, R y0, R X1,
-                                        R Y1, R vphi) {
+template <typename R, typename A>
+__device__ __forceinline__ void deposit(const Params<R> &p, const A &acc, R qw, int i, int j, int sx, int sy, R x0, R y0,
+                                        R X1, R Y1, R vphi) {
   const R nq = -qw;
   R gx = nq * (x0 - X1), gy = nq * (y0 - Y1);
   R mx1 = R(0.5) * (x0 + X1), my1 = R(0.5) * (y0 + Y1), mx0 = R(1) - mx1, my0 = R(1) - my1;
@@ -517,33 +541,35 @@ __device__ __forceinline__ void deposit(const Params<R> &p, R qw, int i, int j, 
     const R mxc = R(0.5) * (x0 + Xc), myc = R(0.5) * (y0 + Yc);
     gx = nq * (x0 - Xc); gy = nq * (y0 - Yc);
     mx0 = R(1) - mxc - ax0; mx1 = mxc - ax1; my0 = R(1) - myc - ay0; my1 = myc - ay1;
-    if constexpr (kShare) {
-      if (sx) add_faces_shared(p, i + sx, j, gxo * my0, gxo * my1, gy * ax0, gy * ax1);
-      if (sy) add_faces_shared(p, i, j + sy, gx * ay0, gx * ay1, gyo * mx0, gyo * mx1);
-      if (sx && sy) add_faces_shared(p, i + sx, j + sy, gxo * ay0, gxo * ay1, gyo * ax0, gyo * ax1);
+    if constexpr (A::kShare) {
+      if (sx) add_faces_shared(p, acc, i + sx, j, gxo * my0, gxo * my1, gy * ax0, gy * ax1);
+      if (sy) add_faces_shared(p, acc, i, j + sy, gx * ay0, gx * ay1, gyo * mx0, gyo * mx1);
+      if (sx && sy) add_faces_shared(p, acc, i + sx, j + sy, gxo * ay0, gxo * ay1, gyo * ax0, gyo * ax1);
     } else {
-      if (sx) add_faces(p, i + sx, j, gxo * my0, gxo * my1, gy * ax0, gy * ax1);
-      if (sy) add_faces(p, i, j + sy, gx * ay0, gx * ay1, gyo * mx0, gyo * mx1);
-      if (sx && sy) add_faces(p, i + sx, j + sy, gxo * ay0, gxo * ay1, gyo * ax0, gyo * ax1);
+      if (sx) add_faces(p, acc, i + sx, j, gxo * my0, gxo * my1, gy * ax0, gy * ax1);
+      if (sy) add_faces(p, acc, i, j + sy, gx * ay0, gx * ay1, gyo * mx0, gyo * mx1);
+      if (sx && sy) add_faces(p, acc, i + sx, j + sy, gxo * ay0, gxo * ay1, gyo * ax0, gyo * ax1);
     }
     if (sx && (below_zero(wx) || at_least(wx, R(1)))) { ic += sx; wx -= R(sx); }
     if (sy && (below_zero(wy) || at_least(wy, R(1)))) { jc += sy; wy -= R(sy); }
   }
   const R qv = qw * vphi, a1 = qv * wx, a0 = qv - a1, a01 = a0 * wy, a11 = a1 * wy;
-  if constexpr (kShare) {
-    float v[8] = {gx * my0, gx * my1, gy * mx0, gy * mx1, a0 - a01, a01, a1 - a11, a11};
-    if (ic != i || jc != j) {   // mid-point in the cell entered: on its own
-      add_corners(p, ic, jc, v[4], v[5], v[6], v[7]);
-      v[4] = v[5] = v[6] = v[7] = 0.f;
+  if constexpr (A::kShare) {
+    if (acc.share) {
+      float v[8] = {gx * my0, gx * my1, gy * mx0, gy * mx1, a0 - a01, a01, a1 - a11, a11};
+      if (ic != i || jc != j) {   // mid-point in the cell entered: on its own
+        add_corners(p, acc, ic, jc, v[4], v[5], v[6], v[7]);
+        v[4] = v[5] = v[6] = v[7] = 0.f;
+      }
+      if (sum_by_cell(i * p.nt + j, v)) {
+        add_faces(p, acc, i, j, v[0], v[1], v[2], v[3]);
+        add_corners(p, acc, i, j, v[4], v[5], v[6], v[7]);
+      }
+      return;
     }
-    if (sum_by_cell(i * p.nt + j, v)) {
-      add_faces(p, i, j, v[0], v[1], v[2], v[3]);
-      add_corners(p, i, j, v[4], v[5], v[6], v[7]);
-    }
-    return;
   }
-  add_faces(p, i, j, gx * my0, gx * my1, gy * mx0, gy * mx1);
-  add_corners(p, ic, jc, a0 - a01, a01, a1 - a11, a11);
+  add_faces(p, acc, i, j, gx * my0, gx * my1, gy * mx0, gy * mx1);
+  add_corners(p, acc, ic, jc, a0 - a01, a01, a1 - a11, a11);
 }
 
 template <typename R> __device__ __forceinline__ R one_minus_ulp();
@@ -619,8 +645,8 @@ struct TileFacts {
 // One particle in cell (i, j): gather, push, move, kill rules, deposit, and
 // its new state in slot q (the slot it came from, unless the push also
 // performs a sort's payload gather, kGather, which writes w too).
-template <typename R, bool kGather, bool kShare, typename M>
-__device__ __forceinline__ void push_one(const M &m, const TileFacts &F, const Params<R> &p, const SpeciesConst<R> &K,
+template <typename R, bool kGather, typename M, typename A>
+__device__ __forceinline__ void push_one(const M &m, const A &acc, const TileFacts &F, const Params<R> &p, const SpeciesConst<R> &K,
                                          int q, int i, int j, R xo, R yo, R w, const R u[3], Tally<R> &tl) {
   using P = Series<R>;
   const int nt = p.nt;
@@ -692,7 +718,7 @@ __device__ __forceinline__ void push_one(const M &m, const TileFacts &F, const P
   }
   // off the mesh (no absorber), or force-free
   if (!dead) dead = (F.edge && i1 >= p.nr) || m.ff(i1, j1);
-  deposit<kShare, R>(p, K.q * w, i, j, sx, sy, xo, yo, X1, Y1, un[2] * ginv);
+  deposit<R>(p, acc, K.q * w, i, j, sx, sy, xo, yo, X1, Y1, un[2] * ginv);
   if (dead) {
     K.cell_out[q] = -1;
     tl.killed += w;
@@ -719,7 +745,7 @@ __device__ __noinline__ Tally<R> push_one_global(const Params<R> &p, int s, int 
   int i, j;
   decode_cell(p, cell, i, j);
   const R u[3] = {K.in(2, from), K.in(3, from), K.in(4, from)};
-  push_one<R, kGather, false>(g, TileFacts{false, true, true}, p, K, slot, i, j, K.in(0, from), K.in(1, from), K.in(5, from), u, tl);
+  push_one<R, kGather>(g, MeshAcc<R>{p}, TileFacts{false, true, true}, p, K, slot, i, j, K.in(0, from), K.in(1, from), K.in(5, from), u, tl);
   return tl;
 }
 
@@ -802,8 +828,8 @@ struct Prefetch {
 };
 
 // particles of slots q0 .. q1 of a work item, one per thread and round
-template <typename R, bool kGather, bool kShare>
-__device__ __forceinline__ void push_item(const SharedMesh<R> &m, const TileFacts &F, const Params<R> &p,
+template <typename R, bool kGather, typename A>
+__device__ __forceinline__ void push_item(const SharedMesh<R> &m, const A &acc, const TileFacts &F, const Params<R> &p,
                                           const SpeciesConst<R> &K, const Prefetch<R> &pre, int s, int q0, int q1, int lr,
                                           Tally<R> &tl) {
   // rounds whose particle was left for the global path: an item has at most
@@ -830,7 +856,7 @@ __device__ __forceinline__ void push_item(const SharedMesh<R> &m, const TileFact
     // a particle is handled in shared memory when its gather stencil and the
     // cells it can reach (start cell -1 .. +1) lie inside the region
     if ((unsigned)(i - m.i0 - 1) < (unsigned)(lr - 2) && (unsigned)(j - m.j0 - 1) < (unsigned)(m.lt - 2))
-      push_one<R, kGather, kShare>(m, F, p, K, slot, i, j, x, y, w, u, tl);
+      push_one<R, kGather>(m, acc, F, p, K, slot, i, j, x, y, w, u, tl);
     else
       left |= bit;
   }
@@ -838,6 +864,58 @@ __device__ __forceinline__ void push_item(const SharedMesh<R> &m, const TileFact
     const int slot = q0 + (int)threadIdx.x + kPushThreads * (__ffs(left) - 1);
     const int from = kGather ? (int)K.sidx[slot] : slot;
     tl.add(push_one_global<R, kGather>(p, s, slot, from, K.cell_in[from]));
+  }
+}
+
+// Crowded items (FP32).  An FP32 accumulator that takes the particles of a tile
+// one by one, over all its work items, loses more of their sum than one that
+// takes the sums of its items.  Relative error of J_r, against FP64, one by one
+// and by items: momenta at random 4.8e-7 and 4.6e-7 at 24 particles per cell and
+// species, 4.8 and 4.6 at 48, 5.3 and 4.8 at 100, 7.0 and 4.6 at 500, 14.4 and
+// 4.8 at 3000; equal momenta 1.2e-7 and 1.1e-7, 1.3 and 0.9, 1.6 and 0.8, 3.6 and
+// 0.8, 7.6 and 1.2.  So where an accumulator expects more than kCrowdMin
+// additions, the item deposits into the block's own records of its region (in
+// global memory: 20 to 30 KB, in the L2), which it adds to the mesh's at its
+// end.  What an accumulator expects is the tile's particles (all species; kept
+// in the list by the sort) times the chance that two particles of the item share
+// a cell, taken from how many sampled ones meet their like within their warp.
+// The push of 5e7 particles on 1024^2, 177 to a cell, takes 1.07 ms so and 1.02
+// one by one; 3e8 on 4096^2, where the current sheet (a fifth) is crowded and
+// the rest has 68 to a cell, 6.39 and 6.22 ms, and 6.75 with a limit of 64 (the
+// reductions at the end of an item are as many as those of 500 particles).
+constexpr float kCrowdMin = 96.f;
+constexpr float kCrowdItem = 4.f;
+// place of thread t's sample among the 256: a fixed permutation without pattern
+__device__ __forceinline__ int sample_place(int t) {
+  t = (t * 167 + 13) & 255;
+  t ^= t >> 4;
+  t = (t * 89 + 71) & 255;
+  return t ^ (t >> 3);
+}
+// met: sampled particles that share their cell with another one of their warp's,
+// in two samples of up to 256 (fewer in an item of w < 320 particles); n:
+// particles of the tile.  An item that itself brings an accumulator fewer than
+// kCrowdItem particles does without: its sums would be hardly fewer additions
+// than its particles, and cost as much.
+__device__ __forceinline__ bool crowded(int met, int w, int n) {
+  const int lanes = min(kPushThreads, w - kShareDist) / 8;   // sampled per warp
+  if (lanes < 2) return false;
+  const float got = (float)met / (float)(16 * lanes);        // chance to meet one's like among lanes - 1
+  auto chance = [&](float c) { return c < 1.f ? 1.f - exp2f((float)(lanes - 1) * log2f(1.f - c)) : 2.f; };
+  return got > chance(max(kCrowdMin / (float)max(n, 1), kCrowdItem / (float)w));
+}
+// the block's records of the region added to the mesh's, and cleared
+__device__ __forceinline__ void flush_records(const Params<float> &p, const TileAcc &t, int lr) {
+  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+  __syncthreads();   // every thread's reductions are visible to the block
+  for (int k = threadIdx.x; k < lr * t.ld; k += kPushThreads) {
+    float4 *rec = reinterpret_cast<float4 *>(t.base + 8 * k);
+    const float4 a = __ldcg(rec), c = __ldcg(rec + 1);
+    const int r = k / t.ld, i = t.i0 + r, j = t.j0 + k - r * t.ld;
+    if (i < 0 || j < 0 || i > p.nr || j > p.nt) continue;   // never deposited into
+    float *q = p.jacc + acc_index(p, i, j);
+    if (a.x != 0.f || a.y != 0.f || a.z != 0.f || a.w != 0.f) { __stcg(rec, z); red_add4(q, a.x, a.y, a.z, a.w); }
+    if (c.x != 0.f || c.y != 0.f || c.z != 0.f || c.w != 0.f) { __stcg(rec + 1, z); red_add4(q + 4, c.x, c.y, c.z, c.w); }
   }
 }
 
@@ -864,28 +942,32 @@ template <typename R, bool kGather>
 __global__ void __launch_bounds__(kPushThreads, push_tiled_min_blocks<R>())
     k_push_tiled(const __grid_constant__ Params<R> p, WorkList wl, int halo) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int lr = p.tile_r + 2 * halo + 2, lt = p.tile_t + 2 * halo + 2, area = lr * lt;
+  const int lrm = p.tile_r + 2 * halo + 2, ltm = p.tile_t + 2 * halo + 2;   // the largest region
   SharedMesh<R> m;
   Prefetch<R> pre;
   pre.slot = reinterpret_cast<R *>(smem);
-  m.s_rn = reinterpret_cast<R *>(m.carve(smem + 7 * kPushThreads * sizeof(R), area));
-  m.s_sn = m.s_rn + lr; m.s_cn = m.s_sn + lt;
-  m.s_ff = reinterpret_cast<uint8_t *>(m.s_cn + lt);
-  m.lt = lt;
+  m.s_rn = reinterpret_cast<R *>(m.carve(smem + 7 * kPushThreads * sizeof(R), lrm * ltm));
+  m.s_sn = m.s_rn + lrm; m.s_cn = m.s_sn + ltm;
+  m.s_ff = reinterpret_cast<uint8_t *>(m.s_cn + ltm);
   __shared__ int s_item;
   const int nr = p.nr, nt = p.nt, n1 = nt + 1;
   Tally<R> tl{R(0), R(0), 0u, 0u};
   const int ni = *wl.n_items;
   for (int it = blockIdx.x; it < ni;) {   // the first item by block, later ones from the queue
     const int4 item = wl.items[item_order(it, ni)];
-    const int s = item.x, tile = item.y;
+    const int s = item.x & 3, tile = item.y;
     const int ti = tile / p.ntt, tj = tile - ti * p.ntt;
-    m.i0 = ti * p.tile_r - halo - 1;
-    m.j0 = tj * p.tile_t - halo - 1;
+    // a step's drift in cells falls like 1 / r (or faster), and so does the halo
+    // (particles beyond it would take the global path)
+    const int hl = min(halo, (int)ceil((R)halo * p.r_min / p.t.rn[max(ti * p.tile_r - halo, 0)]));
+    const int lr = p.tile_r + 2 * hl + 2, lt = p.tile_t + 2 * hl + 2, area = lr * lt;
+    m.i0 = ti * p.tile_r - hl - 1;
+    m.j0 = tj * p.tile_t - hl - 1;
+    m.lt = lt;
     const SpeciesConst<R> K(p, s, kGather);
     int ca = -1, cb = -2;   // cells of a sampled pair of particles (read here, behind the staging too)
     if constexpr (sizeof(R) == 4) {
-      const int qa = item.z + kShareDist + (int)threadIdx.x * max(1, (item.w - kShareDist) / kPushThreads);
+      const int qa = item.z + kShareDist + sample_place(threadIdx.x) * max(1, (item.w - kShareDist) / kPushThreads);
       if (qa < item.z + item.w) {
         ca = K.cell_in[kGather ? (int)K.sidx[qa] : qa];
         cb = K.cell_in[kGather ? (int)K.sidx[qa - kShareDist] : qa - kShareDist];
@@ -924,10 +1006,25 @@ __global__ void __launch_bounds__(kPushThreads, push_tiled_min_blocks<R>())
       F.shell = r0 * r0 < p.shell_r2 * R(1.001);
       F.edge = ra == 0 || rb == nr || ca == 0 || cb == nt || rb >= p.i_abs;
     }
+    bool plain = true;
     if constexpr (sizeof(R) == 4) {
-      if (share) push_item<R, kGather, true>(m, F, p, K, pre, s, item.z, item.z + item.w, lr, tl);
+      bool own = item.x & kItemOwn;
+      if (!(item.x & (kItemDirect | kItemOwn))) {   // the list's first push decides for the later ones
+        const unsigned pa = __match_any_sync(0xffffffffu, ca >= 0 ? ca : -1 - (int)threadIdx.x);
+        const unsigned pb = __match_any_sync(0xffffffffu, cb >= 0 ? cb : -1 - (int)threadIdx.x);
+        const int met = __syncthreads_count((pa & (pa - 1)) != 0) + __syncthreads_count((pb & (pb - 1)) != 0);
+        own = crowded(met, item.w, item.x / kItemTotal);
+        if (threadIdx.x == 0) wl.items[item_order(it, ni)].x = item.x | (own ? kItemOwn : kItemDirect);
+      }
+      plain = !own && !share;
+      if (!plain) {
+        const TileAcc t = own ? TileAcc{wl.records + (int64_t)blockIdx.x * (8 * lrm * ltm), m.i0, m.j0, lt, share}
+                              : TileAcc{p.jacc, 0, 0, n1, share};
+        push_item<R, kGather>(m, t, F, p, K, pre, s, item.z, item.z + item.w, lr, tl);
+        if (own) flush_records(p, t, lr);
+      }
     }
-    if (sizeof(R) != 4 || !share) push_item<R, kGather, false>(m, F, p, K, pre, s, item.z, item.z + item.w, lr, tl);
+    if (plain) push_item<R, kGather>(m, MeshAcc<R>{p}, F, p, K, pre, s, item.z, item.z + item.w, lr, tl);
     if (threadIdx.x == 0) s_item = (int)gridDim.x + atomicAdd(wl.next, 1);
     __syncthreads();
     it = s_item;   // next written after the barrier behind the next staging
@@ -941,10 +1038,23 @@ __global__ void __launch_bounds__(kPushThreads, push_tiled_min_blocks<R>())
   }
 }
 
-template <typename R> size_t push_tiled_smem(const Params<R> &p, int halo) {
-  const size_t lr = p.tile_r + 2 * halo + 2, lt = p.tile_t + 2 * halo + 2, area = lr * lt;
+template <typename R> size_t push_tiled_smem(int tile_r, int tile_t, int halo) {
+  const size_t lr = tile_r + 2 * halo + 2, lt = tile_t + 2 * halo + 2, area = lr * lt;
   return 7 * kPushThreads * sizeof(R) + area * SharedMesh<R>::bytes_per_location() +
          (lr + 2 * lt) * sizeof(R);
+}
+template <typename R> size_t push_tiled_smem(const Params<R> &p, int halo) {
+  return push_tiled_smem<R>(p.tile_r, p.tile_t, halo);
+}
+
+// The blocks' own records: one region per block of the largest grid (at most
+// push_tiled_min_blocks per SM of 152, and what shared memory leaves room for)
+int push_record_blocks(int tile_r, int tile_t, int halo) {
+  const size_t smem = push_tiled_smem<float>(tile_r, tile_t, halo);
+  return 152 * (int)std::max<size_t>(1, std::min<size_t>(push_tiled_min_blocks<float>(), 228 * 1024 / (smem + 1024)));
+}
+size_t push_record_bytes(int tile_r, int tile_t, int halo) {
+  return (size_t)(tile_r + 2 * halo + 2) * (tile_t + 2 * halo + 2) * 32;
 }
 
 // The tiles and cadences that hff_init accepts: those whose region, two

@@ -502,6 +502,10 @@ __global__ void __launch_bounds__(1024) k_worklist(const int *bounds, int ntiles
       int cnt = 0;
       if (k < ntiles) cnt = end[k] - start[k];
       const uint32_t ni = cnt > 0 ? (uint32_t)((cnt + chunk - 1) / chunk) : 0u;
+      int64_t total = 0;   // of the tile, all species
+      for (int t = 0; t < n_species && ni; ++t)
+        total += bounds[(int64_t)(2 * t + 1) * (ntiles + 1) + k] - bounds[(int64_t)2 * t * (ntiles + 1) + k];
+      const int word = species + kItemTotal * (int)min(total, (int64_t)kItemTotalMax);
       uint32_t tot;
       const uint32_t ex = block_excl_scan(ni, w, tot);
       for (uint32_t c = 0; c < ni; ++c) {
@@ -509,7 +513,7 @@ __global__ void __launch_bounds__(1024) k_worklist(const int *bounds, int ntiles
         if (slot < (uint32_t)max_items) {
           const int s0 = start[k] + (int)c * chunk;
           const int len = min(chunk, end[k] - s0);
-          items[slot] = make_int4(species, k, s0, len);
+          items[slot] = make_int4(word, k, s0, len);
         } else {
           atomicOr(status, kStWorklist);
         }
