@@ -11,14 +11,18 @@ namespace hff {
 // hardware instructions (about 1-2 ulp, denormals flushed): their arguments
 // here are squared norms, radii and ratios of per-step increments, never
 // denormal, and the results enter quantities compared with the FP64 oracle at
-// 1e-5 relative.  FP64 ones from the hardware's approximations (better than
-// 2^-18) by one step of third order: with e = 1 - x y the reciprocal is
-// y / (1 - e) = y (1 + e + e^2 + O(e^3)); with e = 1 - x y^2 the reciprocal
-// square root is y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2 / 8 + O(e^3)); the
-// remainders are below 2^-54.  Three and five FP64 operations instead of the
-// eight to ten of the library's (correctly rounded or nearly so): the FP64
-// push is bound by the FP64 pipe, two operations per clock and SM.  Arguments
-// near the ends of the range go to the library.
+// 1e-5 relative.  FP64 ones from the hardware's approximations y (the upper 32
+// bits of a double, 20 bits after the point: taken as better than 2^-19) by one
+// step of a series.  With e = 1 - x y the reciprocal is y / (1 - e) =
+// y (1 + e + e^2 + e^3 + O(e^4)), the remainder below 2^-75.  With e = 1 - x y^2,
+// where y^2 is exact, the reciprocal square root is y (1 - e)^(-1/2) =
+// y (1 + e/2 + 3 e^2 / 8 + O(e^3)), the remainder (5/16) e^3 below 2^-55.  What is
+// left is the rounding of the last operation.  Over 4e6 arguments the reciprocal
+// is that of 1 / x and the root that of rsqrt to the last bit (without e^3, and
+// with x y rounded before its product with y, they were off by 1.002 and 1.25
+// times half an ulp).  Four and five FP64 operations instead of the eight to ten
+// of the library's: the FP64 push is bound by the FP64 pipe, two operations per
+// clock and SM.  Arguments near the ends of the range go to the library.
 __device__ __forceinline__ float rsq(float x) {
   float y;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -35,7 +39,7 @@ __device__ __forceinline__ double rsq(double x) {
   if (!mid_range(x)) return rsqrt(x);
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-(x * y), y, 1.0);
+  const double e = fma(-x, y * y, 1.0);
   return fma(y * e, fma(0.375, e, 0.5), y);
 }
 __device__ __forceinline__ double rcp(double x) {
@@ -43,7 +47,7 @@ __device__ __forceinline__ double rcp(double x) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);
+  return fma(y, fma(fma(e, e, e), e, e), y);
 }
 
 // float -> double: for normal numbers the bits moved on the integer pipe (a
