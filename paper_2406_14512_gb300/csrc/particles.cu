@@ -145,8 +145,10 @@ __device__ __forceinline__ bool well_below(double a, double b) {
 
 // Small-argument Taylor expansions about 0, for the per-step increments that
 // the Courant condition keeps small; callers switch to the library functions
-// outside |x| < kSmall, where every truncation error is below 1e-12 of the
-// value in FP64 and 5e-9 in FP32 (a twelfth of its rounding).
+// outside |x| < kSmall (log1p outside 0.03125), where every truncation error is
+// below 2e-13 of the value (for cosm, of the cosine) in FP64 (log1p's, x^8 / 9;
+// the others below 1e-15) and 5e-10 in FP32 (the binomial ones, (35/64) q^3; a
+// hundredth of its rounding).
 // c[0] + c[1] x + .. by Horner's rule
 template <typename R, int N>
 __device__ __forceinline__ R poly(R x, const double (&c)[N]) {
@@ -164,7 +166,7 @@ template <typename R> struct Series {
   static __device__ __forceinline__ R cosm(R x2) { const double c[] = {-0.5, 1.0 / 24, -1.0 / 720}; return poly(x2, c); }
   static __device__ __forceinline__ R atanc(R t2) { const double c[] = {1.0, -1.0 / 3, 0.2, -1.0 / 7, 1.0 / 9}; return poly(t2, c); }
   static __device__ __forceinline__ R log1pc(R x) {
-    const double c[] = {1.0, -0.5, 1.0 / 3, -0.25, 0.2, -1.0 / 6, 1.0 / 7};
+    const double c[] = {1.0, -0.5, 1.0 / 3, -0.25, 0.2, -1.0 / 6, 1.0 / 7, -0.125};
     return poly(x, c);
   }
   static __device__ __forceinline__ R expm1c(R x) {
@@ -179,7 +181,7 @@ template <> struct Series<float> {
   static __device__ __forceinline__ R sinc(R x2) { const double c[] = {1.0, -1.0 / 6, 1.0 / 120}; return poly(x2, c); }
   static __device__ __forceinline__ R cosm(R x2) { const double c[] = {-0.5, 1.0 / 24}; return poly(x2, c); }
   static __device__ __forceinline__ R atanc(R t2) { const double c[] = {1.0, -1.0 / 3, 0.2}; return poly(t2, c); }
-  static __device__ __forceinline__ R log1pc(R x) { const double c[] = {1.0, -0.5, 1.0 / 3, -0.25, 0.2}; return poly(x, c); }
+  static __device__ __forceinline__ R log1pc(R x) { const double c[] = {1.0, -0.5, 1.0 / 3, -0.25, 0.2, -1.0 / 6}; return poly(x, c); }
   static __device__ __forceinline__ R expm1c(R x) { const double c[] = {1.0, 0.5, 1.0 / 6, 1.0 / 24, 1.0 / 120}; return poly(x, c); }
   static __device__ __forceinline__ R omc(R q) { const double c[] = {0.5, -3.0 / 8, 5.0 / 16}; return poly(q, c); }
   static __device__ __forceinline__ R sqm(R q) { const double c[] = {0.5, -1.0 / 8, 1.0 / 16}; return poly(q, c); }

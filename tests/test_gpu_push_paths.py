@@ -92,3 +92,36 @@ def test_fp64_momentum_whose_square_overflows():
     assert big.sum() > 50 and np.array_equal(after["cell"][big], before["cell"][big])
     assert np.array_equal(after["ur"][big], before["ur"][big]) and np.array_equal(after["xo"][big], before["xo"][big])
     assert sim.status() == 0
+
+
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+def test_fp64_displacement_at_the_end_of_the_series(sign):
+    """Radial moves of 2.4% to 3.4% of the radius, on both sides of where log1p
+    leaves its series for the library: the new offset against the oracle.  The
+    series ends below x^9 / 9 (1e-13 of the value at 0.03125); in cells of
+    log(r) = 0.1 that is 3e-14, and the oracle's and the push's own rounding (a
+    few 2^-53 over 0.1) as much again: 1e-13."""
+    hff, workloads, oracle = _libs()
+    cfg = workloads._base(32, 16, float(np.exp(3.2)), 3.0, "dipole", seed=5)
+    cfg.update(precision="fp64", capacity=6000, sort_every=4, inject=False, shell_r=0.5)
+    rng = np.random.default_rng(8)
+    n = 4000
+    sim, ref = hff.Sim(cfg), oracle.Oracle(cfg)
+    dt = sim.info().dt
+    for f in ("E_r", "E_th", "E_ph", "B_r", "B_th", "B_ph"):
+        z = np.zeros(ref.shape(f))
+        sim.set(f, z)
+        ref.set(f, z)
+    xi = np.log(dt / rng.uniform(0.024, 0.034, n)) / 0.1
+    ps = []
+    for s in range(2):
+        ps.append(dict(cell=(xi.astype(np.int32) * 16 + rng.integers(3, 13, n)).astype(np.int32), xo=xi % 1.0, yo=rng.random(n),
+                       ur=np.full(n, sign * 1e4), ut=np.zeros(n), up=np.zeros(n), w=np.full(n, 1e-6)))
+        sim.load(s, ps[s])
+        ref.set_particles(s, ps[s])
+    ref.sort_now()
+    sim.step_stages(1, ST["node"] | ST["push"])
+    ref.step(1, ST["node"] | ST["push"])
+    for s in range(2):
+        bad, _, e = particle_mismatches(sim.particles(s), ref.particles(s), 16)
+        assert bad == 0 and e < 1e-13, (s, bad, e)
