@@ -206,7 +206,7 @@ struct Offsets {
   size_t records;        // FP32: flux records of the push's blocks (crowded items)
   int record_blocks;     // the most blocks of the push
   size_t fsnap;          // halo snapshot of the fused field update
-  int seg_rows;          // rows per segment of the fused field update
+  int seg_rows;          // least rows per segment of the fused field update (its snapshot's size)
   size_t ev[8];          // pair-creation events: key cell xo yo ur ut up w
   size_t spec;           // spectrum bins (on request)
   int64_t ev_cap;
@@ -307,7 +307,8 @@ void layout(const hff_config &c, Offsets &o) {
   o.rows = L.take((nr + 1) * 8 * 8);
   o.psi64 = L.take(nn * 8);
   // segments of the fused field update: one wave of its blocks on the 152 SMs
-  // of a GB300 (a property of the grid, so that hff_plan needs no GPU)
+  // of a GB300 (a property of the grid, so that hff_plan needs no GPU); hff_init
+  // lengthens them where the device holds fewer
   o.seg_rows = fuse_seg_rows(c.nr, c.nt, 152 * kFuseBlocksPerSm, R, filtered(c));
   o.fsnap = fused_fields(c) ? L.take(fuse_snap_bytes(c.nr, c.nt, o.seg_rows, R, filtered(c))) : 0;
   o.total = (L.off + 255) & ~size_t(255);
@@ -330,6 +331,7 @@ struct hff_handle {
   double dt = 0, psi_unit = 0, xi_abs = 0;
   int halo = 0, push_grid = 0, tail_grid = 0;
   bool fused = false;  // the field update runs as the fused pass (fused_fields)
+  int seg_rows = 0;    // rows per segment of the fused field update (>= o.seg_rows)
   Params<float> pf[2];
   Params<double> pd[2];
   WorkList wl{};
@@ -718,7 +720,7 @@ int enqueue_step(hff_handle *h, int par, int stages, cudaStream_t s, int parts =
   }
   if (fused) {
     // the whole field update in one pass; J_PIC cleared for the next deposit
-    launch_field_fused<R>(p, h->o.seg_rows, h->base + h->o.fsnap, collect, s);
+    launch_field_fused<R>(p, h->seg_rows, h->base + h->o.fsnap, collect, s);
     // J_r, J_th, J_ph lie one after the other (see layout)
     CK(cudaMemsetAsync(p.f.jr, 0, (size_t)(h->o.f[12] - h->o.f[9]), s));
   } else {
@@ -1210,12 +1212,22 @@ static int init_one(const hff_config *cfg, void *dev_mem, size_t bytes, void *st
     const size_t psm = cfg->precision == HFF_FP64 ? psi_smem<double>(cfg->nt) : psi_smem<float>(cfg->nt);
     const cudaError_t e = cfg->precision == HFF_FP64 ? set_psi_smem<double>(psm) : set_psi_smem<float>(psm);
     if (e != cudaSuccess) return bail(fail(HFF_ERR_CUDA, "cannot set the flux-prefix shared memory size"));
-    const cudaError_t e2 = cfg->precision == HFF_FP64
-                               ? set_field_fused_smem<double>(field_fused_smem<double>(h->o.seg_rows))
-                               : set_field_fused_smem<float>(field_fused_smem<float>(h->o.seg_rows));
-    if (set_sort_smem() != cudaSuccess) return bail(fail(HFF_ERR_CUDA, "cannot set the sort's shared memory size"));
-    if (e2 != cudaSuccess) return bail(fail(HFF_ERR_CUDA, "cannot set the fused field update's shared memory size"));
     h->fused = fused_fields(*cfg);
+    h->seg_rows = h->o.seg_rows;
+    if (h->fused) {
+      // one wave of the fused field update on this device, which may hold fewer
+      // blocks than the plan (a GB300's) assumes: longer segments then
+      const bool d = cfg->precision == HFF_FP64, filt = filtered(*cfg);
+      auto allow = [&](int rows) {
+        return d ? set_field_fused_smem<double>(field_fused_smem<double>(rows)) : set_field_fused_smem<float>(field_fused_smem<float>(rows));
+      };
+      cudaError_t e2 = allow(h->seg_rows);
+      const int occ = d ? field_fused_blocks_per_sm<double>(h->seg_rows, filt) : field_fused_blocks_per_sm<float>(h->seg_rows, filt);
+      h->seg_rows = std::max(h->seg_rows, fuse_seg_rows(cfg->nr, cfg->nt, std::max(1, occ) * nsm, d ? 8 : 4, filt));
+      if (e2 == cudaSuccess) e2 = allow(h->seg_rows);
+      if (e2 != cudaSuccess) return bail(fail(HFF_ERR_CUDA, "cannot set the fused field update's shared memory size"));
+    }
+    if (set_sort_smem() != cudaSuccess) return bail(fail(HFF_ERR_CUDA, "cannot set the sort's shared memory size"));
   }
   if (cfg->precision == HFF_FP32) {
     fill_params<float>(h);

@@ -978,6 +978,12 @@ template <typename R> cudaError_t set_field_fused_smem(size_t bytes) {
   const cudaError_t e = raise_smem_limit<field_fused_fn<R, false>>(bytes);
   return e != cudaSuccess ? e : raise_smem_limit<field_fused_fn<R, true>>(bytes);
 }
+// resident blocks per SM of the pass with segments of seg_rows rows; 0 on error
+template <typename R> int field_fused_blocks_per_sm(int seg_rows, bool filt) {
+  int n = 0;
+  const void *f = filt ? field_fused_fn<R, true>() : field_fused_fn<R, false>();
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, 32 * fuse_warps(sizeof(R)), field_fused_smem<R>(seg_rows)) == cudaSuccess ? n : 0;
+}
 // rows per segment: as many segments as fit the strips into wave_blocks
 // resident blocks (one wave: every block walks its rows once, none waits
 // for a second wave), at least 32 rows so that the warm-up stays a small
@@ -1107,7 +1113,8 @@ template <typename R> void launch_combine(R *dst, const R *a, const R *b, int64_
   template void launch_blend_out<R>(const Params<R> &, R *, R *, R *, uint8_t *, cudaStream_t); \
   template void launch_field_fused<R>(const Params<R> &, int, void *, bool, cudaStream_t);      \
   template size_t field_fused_smem<R>(int);                                                         \
-  template cudaError_t set_field_fused_smem<R>(size_t);
+  template cudaError_t set_field_fused_smem<R>(size_t);                        \
+  template int field_fused_blocks_per_sm<R>(int, bool);
 HFF_INST(float)
 HFF_INST(double)
 #undef HFF_INST

@@ -302,7 +302,8 @@ template <typename R> void launch_blend_out(const Params<R> &p, R *fr, R *ft, R 
 // Ampere, renormalisation, return, Faraday half with absorber) in one pass
 // over row segments of seg_rows rows
 template <typename R> void launch_field_fused(const Params<R> &p, int seg_rows, void *snap, bool collect, cudaStream_t s);
-constexpr int kFuseBlocksPerSm = 2;                                 // its resident blocks
+constexpr int kFuseBlocksPerSm = 2;                                 // its resident blocks on a GB300
+template <typename R> int field_fused_blocks_per_sm(int seg_rows, bool filt);  // and on this device
 int fuse_seg_rows(int nr, int nt, int wave_blocks, size_t real, bool filt);    // rows per segment of the launch
 size_t fuse_snap_bytes(int nr, int nt, int seg_rows, size_t real, bool filt);  // its halo snapshot
 template <typename R> size_t field_fused_smem(int seg_rows);
