@@ -1227,7 +1227,6 @@ static int init_one(const hff_config *cfg, void *dev_mem, size_t bytes, void *st
       if (e2 == cudaSuccess) e2 = allow(h->seg_rows);
       if (e2 != cudaSuccess) return bail(fail(HFF_ERR_CUDA, "cannot set the fused field update's shared memory size"));
     }
-    if (set_sort_smem() != cudaSuccess) return bail(fail(HFF_ERR_CUDA, "cannot set the sort's shared memory size"));
   }
   if (cfg->precision == HFF_FP32) {
     fill_params<float>(h);

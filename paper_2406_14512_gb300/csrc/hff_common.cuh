@@ -369,7 +369,6 @@ template <typename R> void launch_sort(const Params<R> &p, const SortScratch &ss
 template <typename R> void launch_load_sorted(const Params<R> &p, int species, const Species<R> &src, int64_t n,
                                               void *records, const SortScratch &ss, int *unsettled, cudaStream_t s);
 template <typename R> size_t load_record_bytes();
-cudaError_t set_sort_smem();
 // the deferred payload gather of a species, src -> sp by sidx (slots < count)
 template <typename R> void launch_materialize(const Params<R> &p, int species, cudaStream_t s);
 // loaded cells at or past ncells become removed particles; kStBadCell latched

@@ -220,6 +220,7 @@ __global__ void __launch_bounds__(kSortThreads, 5) k_scatter(const __grid_consta
   const int64_t n = *o.n, nb = sort_blocks(n), base = (int64_t)blockIdx.x * kSortBlock;
   if (base >= n) return;
   extern __shared__ __align__(16) unsigned char sort_smem[];
+  static_assert(sizeof(ScatterSmem) <= 48 * 1024, "what every kernel may have");
   ScatterSmem &m = *reinterpret_cast<ScatterSmem *>(sort_smem);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, tid = threadIdx.x, shift = 8 * a.pass;
   for (int w = 0; w < kSortWarps; ++w) m.cnt[w][tid] = 0;
@@ -532,12 +533,6 @@ static int bits_for(uint32_t v) {
   return b;
 }
 
-template <bool F> static const void *scatter_fn() { return reinterpret_cast<const void *>(&k_scatter<F>); }
-cudaError_t set_sort_smem() {
-  const cudaError_t e = raise_smem_limit<scatter_fn<true>>(sizeof(ScatterSmem));
-  return e != cudaSuccess ? e : raise_smem_limit<scatter_fn<false>>(sizeof(ScatterSmem));
-}
-
 // the radix passes over species 0 .. ns-1 of a (grids for `cap` slots)
 static void radix_passes(SortArgs &a, int ns, int64_t cap, cudaStream_t st) {
   const int nb = (int)std::max<int64_t>(1, (cap + kSortBlock - 1) / kSortBlock);
@@ -738,10 +733,6 @@ extern "C" int hff_tile_order_noalloc(const int32_t *cell, int64_t n, int32_t nr
     *n_live = 0;
     hff_noalloc_err = "";
     return HFF_OK;
-  }
-  if (set_sort_smem() != cudaSuccess) {
-    hff_noalloc_err = "hff_tile_order_noalloc: a CUDA call failed";
-    return HFF_ERR_CUDA;
   }
   SortArgs a{};
   SortOne &o = a.s[0];
