@@ -68,7 +68,8 @@ __global__ void __launch_bounds__(256) k_node_charge(Params<R> p, double *q, dou
       atomicAdd(a + n1 + 1, q11);
       const double u0 = to_double(p.sp[s].ur[k]), u1 = to_double(p.sp[s].ut[k]), u2 = to_double(p.sp[s].up[k]);
       const double g2 = fma(u2, u2, fma(u1, u1, fma(u0, u0, 1.0)));
-      ke = fma(w * ms, fma(g2, rsq(g2), -1.0), ke);
+      // gamma - 1; an infinite g2 keeps an infinite root (infinity times rsq would not)
+      ke = fma(w * ms, mid_range(g2) ? fma(g2, rsq(g2), -1.0) : sqrt(g2) - 1.0, ke);
       c += 1;
     }
     for (int o = 16; o > 0; o >>= 1) {

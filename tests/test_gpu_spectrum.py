@@ -39,3 +39,24 @@ def test_bins_at_their_edges(prec, nbins, lo, hi):
     slack = slack + np.roll(slack, 1) + np.roll(slack, -1)
     assert np.all(np.abs(got - want) <= slack), np.flatnonzero(np.abs(got - want) > slack)
     assert got.sum() == d["w"].astype(np.float64).sum()   # powers of two: sums are exact
+
+
+@pytest.mark.parametrize("big", [1e140, 1e160])
+def test_kinetic_energy_of_extreme_momenta(big):
+    """FP64 momenta whose square is near the end of the range (the sum is finite)
+    or beyond it (the energy is then infinite, not undefined)."""
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2406_14512_gb300 import hff, workloads
+    cfg = workloads.config("small_pic")
+    cfg.update(capacity=2000, precision="fp64", sort_every=4, inject=False)
+    p = workloads.particles(cfg, n_pairs=500, seed=3)[0]
+    p["ur"] = p["ur"].astype(np.float64)
+    p["ur"][::7] = big
+    sim = hff.Sim(cfg)
+    sim.load(0, p)
+    got = sim.diagnostics()[0].kinetic[0]
+    with np.errstate(over="ignore"):
+        u2 = sum(p[k].astype(np.float64) ** 2 for k in ("ur", "ut", "up"))
+    want = np.sum(p["w"].astype(np.float64) * cfg["m"][0] * (np.sqrt(1.0 + u2) - 1.0))
+    assert got == want if np.isinf(want) else abs(got - want) <= 1e-12 * want
