@@ -274,7 +274,9 @@ int hff_init(const hff_config *cfg, int n_inst, void *dev_mem, size_t bytes, voi
 /* Replace the particles of one species by n particles (SoA arrays as described
  * above; `where` = HFF_HOST or HFF_DEVICE says where the source arrays live).
  * Values must be in the configured precision.  The particles are sorted by
- * tile if sorting is enabled.  HFF_ERR_CAPACITY if n > capacity.  A cell
+ * tile if sorting is enabled, and so are the other species if they are not in
+ * order (after steps).  Device arrays may be any that cudaMemcpy could copy.
+ * HFF_ERR_CAPACITY if n > capacity.  A cell
  * index at or past nr * nt is invalid: the load completes with those
  * particles removed and returns HFF_ERR_ARG. */
 int hff_load_particles(hff_handle *h, int inst, int species, int64_t n, const int32_t *cell,
@@ -318,7 +320,8 @@ int hff_step_stages(hff_handle *h, int32_t nsteps, int32_t stages);
  * on the stream, so it takes effect for the steps queued after the call. */
 int hff_set_scalar(hff_handle *h, int which, double value);
 
-/* Device views of one species' particles (valid until the next hff_step).
+/* Device views of one species' particles (valid until the next hff_step or
+ * hff_load_particles, which may move the particles of every species).
  * Synchronises the stream to read the count. */
 int hff_particles(hff_handle *h, int inst, int species, hff_particle_view *out);
 

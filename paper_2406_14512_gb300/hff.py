@@ -377,7 +377,7 @@ class _InstanceOps:
 
     def particle_views(self, species: int) -> dict:
         """Torch views (on the device, inside the instance buffer) of one
-        species' particle arrays; valid until the next step."""
+        species' particle arrays; valid until the next step or load."""
         torch = self.torch
         v = hff_particles(self.h, self.inst, species)
         n, base = int(v.n), self.mem.data_ptr()
