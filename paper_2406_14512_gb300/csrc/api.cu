@@ -203,8 +203,6 @@ struct Offsets {
   size_t items;
   size_t qnode, rows, psi64;
   size_t jacc;           // flux accumulators of the push
-  size_t records;        // FP32: flux records of the push's blocks (crowded items)
-  int record_blocks;     // the most blocks of the push
   size_t fsnap;          // halo snapshot of the fused field update
   int seg_rows;          // least rows per segment of the fused field update (its snapshot's size)
   size_t ev[8];          // pair-creation events: key cell xo yo ur ut up w
@@ -292,7 +290,7 @@ void layout(const hff_config &c, Offsets &o) {
     o.hist = L.take(ns * o.hist_stride * 4);
     o.spart = L.take(ns * o.part_stride * 4);
     o.bounds = L.take(ns * 2 * ((size_t)o.ntiles + 1) * 4);
-    o.nsort = L.take((kMaxSpecies + 1) * 8);  // and the unsettled flag
+    o.nsort = L.take((kMaxSpecies + 1) * 8);  // and the unsettled flag and the push's claims
     o.items = L.take((size_t)o.max_items * sizeof(int4));
   }
   // pair-creation events of one step (bounded; overflow is latched)
@@ -300,9 +298,6 @@ void layout(const hff_config &c, Offsets &o) {
   for (int k = 0; k < 8; ++k) o.ev[k] = o.ev_cap ? L.take((size_t)o.ev_cap * (k < 2 ? 4 : R)) : 0;
   o.spec = L.take(4096 * 8);
   o.jacc = cap ? L.take(push_acc_bytes(c.nr, c.nt, R)) : 0;
-  const bool records = cap && c.sort_every > 0 && c.precision == HFF_FP32;
-  o.record_blocks = records ? push_record_blocks(tr, tt, halo_of(c)) : 0;
-  o.records = records ? L.take(std::min(o.record_blocks, o.max_items) * push_record_bytes(tr, tt, halo_of(c))) : 0;
   o.qnode = L.take(nn * 8);
   o.rows = L.take((nr + 1) * 8 * 8);
   o.psi64 = L.take(nn * 8);
@@ -1189,7 +1184,6 @@ static int init_one(const hff_config *cfg, void *dev_mem, size_t bytes, void *st
   h->wl.next = &h->small->next;
   h->wl.done = &h->small->done;
   h->wl.max_items = h->o.max_items;
-  h->wl.records = reinterpret_cast<float *>(h->base + h->o.records);
   h->wl.chunk = chunk_of(*cfg);
   h->ss.keys = reinterpret_cast<uint32_t *>(h->base + h->o.keys);
   h->ss.idx = reinterpret_cast<uint32_t *>(h->base + h->o.idx);
@@ -1198,6 +1192,12 @@ static int init_one(const hff_config *cfg, void *dev_mem, size_t bytes, void *st
   h->ss.bounds = reinterpret_cast<int *>(h->base + h->o.bounds);
   h->ss.n_sort = reinterpret_cast<long long *>(h->base + h->o.nsort);
   h->ss.unsettled = reinterpret_cast<int *>(h->ss.n_sort + kMaxSpecies);
+  // the push's own records: in the sort's keys and indices, idle between sorts
+  h->wl.claimed = h->ss.unsettled + 1;
+  if (cfg->sort_every > 0) {
+    h->wl.records = reinterpret_cast<float *>(h->base + h->o.keys);
+    h->wl.record_sets = (int)std::min<size_t>(1 << 20, (h->o.hist - h->o.keys) / push_record_bytes(h->c.tile_r, h->c.tile_t, h->halo));
+  }
   h->ss.stride = h->o.sort_stride;
   h->ss.hist_stride = h->o.hist_stride;
   h->ss.part_stride = h->o.part_stride;
@@ -1236,8 +1236,6 @@ static int init_one(const hff_config *cfg, void *dev_mem, size_t bytes, void *st
       if (!push_tile_fits<float>(h->pf[0], h->halo)) return bail(fail(HFF_ERR_ARG, "tile + halo too large for shared memory"));
       if (set_push_smem<float>(smem) != cudaSuccess) return bail(fail(HFF_ERR_CUDA, "cannot set shared memory size"));
       h->push_grid = nsm * std::max(1, std::min(8, push_tiled_blocks_per_sm<float>(smem)));
-      // every block that can get an item has records (a list has at most max_items)
-      if (h->o.record_blocks) h->push_grid = std::min(h->push_grid, h->o.record_blocks);
     }
   } else {
     fill_params<double>(h);

@@ -329,15 +329,16 @@ struct WorkList {
   int *done;            // blocks of the running push that have finished
   int max_items;
   int chunk;            // particles per item
-  float *records;       // FP32: flux records of the region of each block's tile (zero between items)
+  float *records;       // FP32: sets of flux records of a tile's region, one per block that needs one
+  int record_sets;      // how many
+  int *claimed;         // sets taken by the running push (0 between pushes)
 };
 
 template <typename R> void launch_push_tail(const Params<R> &p, cudaStream_t s, int grid);
 template <typename R> void launch_push_tiled(const Params<R> &p, const WorkList &wl, int halo,
                                              cudaStream_t s, int grid, bool gather);
 template <typename R> size_t push_tiled_smem(const Params<R> &p, int halo);
-int push_record_blocks(int tile_r, int tile_t, int halo);    // blocks with records of their own
-size_t push_record_bytes(int tile_r, int tile_t, int halo);  // and what each of them takes
+size_t push_record_bytes(int tile_r, int tile_t, int halo);  // of a set of records (WorkList)
 template <typename R> bool push_tile_fits(const Params<R> &p, int halo);  // accepted by hff_init
 // the push's flux accumulators added to J_PIC and cleared
 template <typename R> void launch_collect(const Params<R> &p, cudaStream_t s);

@@ -15,7 +15,6 @@
 //  * k_push_tail -- all particles of the no-sort configuration, the same way.
 // Both deposit into the flux accumulators in global memory (see deposit);
 // those become J_PIC at the end of the push stage (collect.cuh).
-#include <algorithm>
 #include <type_traits>
 
 #include "collect.cuh"
@@ -877,11 +876,11 @@ __device__ __forceinline__ void push_item(const SharedMesh<R> &m, const A &acc, 
 // 4.8 at 3000; equal momenta 1.2e-7 and 1.1e-7, 1.3 and 0.9, 1.6 and 0.8, 3.6 and
 // 0.8, 7.6 and 1.2.  So where an accumulator expects more than kCrowdMin
 // additions, the item deposits into the block's own records of its region (in
-// global memory: 20 to 30 KB, in the L2), which it adds to the mesh's at its
-// end.  What an accumulator expects is the tile's particles (all species; kept
+// the sort's scratch: 20 to 30 KB, in the L2), which it adds to the mesh's at
+// its end.  What an accumulator expects is the tile's particles (all species; kept
 // in the list by the sort) times the chance that two particles of the item share
 // a cell, taken from how many sampled ones meet their like within their warp.
-// The push of 5e7 particles on 1024^2, 177 to a cell, takes 1.07 ms so and 1.02
+// The push of 5e7 particles on 1024^2, 177 to a cell, takes 1.08 ms so and 1.02
 // one by one; 3e8 on 4096^2, where the current sheet (a fifth) is crowded and
 // the rest has 68 to a cell, 6.39 and 6.22 ms, and 6.75 with a limit of 64 (the
 // reductions at the end of an item are as many as those of 500 particles).
@@ -905,6 +904,21 @@ __device__ __forceinline__ bool crowded(int met, int w, int n) {
   const float got = (float)met / (float)(16 * lanes);        // chance to meet one's like among lanes - 1
   auto chance = [&](float c) { return c < 1.f ? 1.f - exp2f((float)(lanes - 1) * log2f(1.f - c)) : 2.f; };
   return got > chance(max(kCrowdMin / (float)max(n, 1), kCrowdItem / (float)w));
+}
+// A block's first crowded item: one of the sets of records (n floats each),
+// cleared (they lie in the sort's scratch).  A small instance may have fewer
+// sets than blocks; a block that finds none left deposits into the mesh's.
+__device__ __noinline__ void claim_records(float *records, int sets, int *claimed, int n, int *which) {
+  __syncthreads();   // *which has been read by all
+  if (threadIdx.x == 0) {
+    const int k = atomicAdd(claimed, 1);
+    *which = k < sets ? k : -2;
+  }
+  __syncthreads();
+  if (*which < 0) return;
+  float4 *rec = reinterpret_cast<float4 *>(records + (int64_t)*which * n);
+  for (int k = threadIdx.x; k < n / 4; k += kPushThreads) __stcg(rec + k, make_float4(0.f, 0.f, 0.f, 0.f));
+  __syncthreads();   // before any thread's reductions
 }
 // the block's records of the region added to the mesh's, and cleared
 __device__ __forceinline__ void flush_records(const Params<float> &p, const TileAcc &t, int lr) {
@@ -951,7 +965,8 @@ __global__ void __launch_bounds__(kPushThreads, push_tiled_min_blocks<R>())
   m.s_rn = reinterpret_cast<R *>(m.carve(smem + 7 * kPushThreads * sizeof(R), lrm * ltm));
   m.s_sn = m.s_rn + lrm; m.s_cn = m.s_sn + ltm;
   m.s_ff = reinterpret_cast<uint8_t *>(m.s_cn + ltm);
-  __shared__ int s_item;
+  __shared__ int s_item, s_records;   // which records are the block's (-1: none yet, -2: none left)
+  if (threadIdx.x == 0) s_records = -1;   // read behind the first staging's barrier
   const int nr = p.nr, nt = p.nt, n1 = nt + 1;
   Tally<R> tl{R(0), R(0), 0u, 0u};
   const int ni = *wl.n_items;
@@ -1018,9 +1033,11 @@ __global__ void __launch_bounds__(kPushThreads, push_tiled_min_blocks<R>())
         own = crowded(met, item.w, item.x / kItemTotal);
         if (threadIdx.x == 0) wl.items[item_order(it, ni)].x = item.x | (own ? kItemOwn : kItemDirect);
       }
+      if (own && s_records == -1) claim_records(wl.records, wl.record_sets, wl.claimed, 8 * lrm * ltm, &s_records);
+      own = own && s_records >= 0;
       plain = !own && !share;
       if (!plain) {
-        const TileAcc t = own ? TileAcc{wl.records + (int64_t)blockIdx.x * (8 * lrm * ltm), m.i0, m.j0, lt, share}
+        const TileAcc t = own ? TileAcc{wl.records + (int64_t)s_records * (8 * lrm * ltm), m.i0, m.j0, lt, share}
                               : TileAcc{p.jacc, 0, 0, n1, share};
         push_item<R, kGather>(m, t, F, p, K, pre, s, item.z, item.z + item.w, lr, tl);
         if (own) flush_records(p, t, lr);
@@ -1037,6 +1054,7 @@ __global__ void __launch_bounds__(kPushThreads, push_tiled_min_blocks<R>())
   if (threadIdx.x == 0 && atomicAdd(wl.done, 1) == (int)gridDim.x - 1) {
     *wl.next = 0;
     *wl.done = 0;
+    if constexpr (sizeof(R) == 4) *wl.claimed = 0;
   }
 }
 
@@ -1049,12 +1067,7 @@ template <typename R> size_t push_tiled_smem(const Params<R> &p, int halo) {
   return push_tiled_smem<R>(p.tile_r, p.tile_t, halo);
 }
 
-// The blocks' own records: one region per block of the largest grid (at most
-// push_tiled_min_blocks per SM of 152, and what shared memory leaves room for)
-int push_record_blocks(int tile_r, int tile_t, int halo) {
-  const size_t smem = push_tiled_smem<float>(tile_r, tile_t, halo);
-  return 152 * (int)std::max<size_t>(1, std::min<size_t>(push_tiled_min_blocks<float>(), 228 * 1024 / (smem + 1024)));
-}
+// what the records of a block's largest region take
 size_t push_record_bytes(int tile_r, int tile_t, int halo) {
   return (size_t)(tile_r + 2 * halo + 2) * (tile_t + 2 * halo + 2) * 32;
 }
